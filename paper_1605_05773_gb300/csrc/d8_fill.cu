@@ -23,13 +23,28 @@
 // nothing ends the fill: every tile is then at a fixed point of its final
 // halo, so F is the global fixed point.
 //
-// Measured: 8192 x 8192 raw fractal 6.7 ms, 700 x 933 0.47 ms (before: 105 and
-// 4.7 ms, 256 threads per tile with two waves over dirty cells, then sweeps of
-// four passes each until a whole sweep changed nothing; its lanes down a row
-// shared banks, and every change of a tile's border listed all eight
-// neighbours).
+// Start from above: the fixed point is reached from any start that is nowhere
+// below it, and the nearer the start, the fewer visits.  So the fill is first
+// bounded on coarser grids, side ratio 4 (k_fill_pool, then the same rounds).
+// A coarse cell is a block B of n x n cells with Z(B) its highest z, and its
+// value bounds F over the block: the block's cells can be reached from any
+// cell of an adjacent block in at most n steps inside B, each raising by one
+// up() and to no more than Z(B), so with X = max(Z(B), lowest adjacent value)
+//     max of F over B <= up^n(X) <= X + |X| b + a        (BlockBound below),
+// and blocks holding cells of the grid's edge keep the bound with X = Z(B).
+// Every state of that iteration from +inf bounds F, settled or not, so the
+// coarse grids get a fixed number of rounds and no host check; each level
+// starts from the bounds of the level above it.
+//
+// Measured: 8192 x 8192 raw fractal 5.9 ms, 8192 x 8192 noisy plane 1.16 ms,
+// 700 x 933 fractal 0.42 ms; without the coarse levels 6.5, 3.2 and 0.45 ms
+// (the fractal's lakes, thousands of cells wide, still fill one tile a round);
+// before (256 threads per tile, two waves over dirty cells, then sweeps of
+// four passes until a whole sweep changed nothing; lanes down a row shared
+// banks, and every change of a tile's border listed all eight neighbours) the
+// fractals took 105 and 4.7 ms.
 #include <cmath>
-#include <cstdio>
+#include <type_traits>
 
 #include "d8_device.cuh"
 
@@ -37,6 +52,7 @@ namespace d8 {
 namespace fill {
 
 constexpr int T = 64;
+constexpr int RATIO = 4;                // side ratio of a level to the next finer one
 constexpr int NTF = T;                  // one thread per row, or column, of the tile
 constexpr int HW = T + 2;               // rows and columns of a tile with its halo
 constexpr int RS = T + 3;               // row stride of those arrays: odd, so lanes down a column hit distinct banks
@@ -59,7 +75,22 @@ __device__ __forceinline__ float up(float m, float eps) {
   return fmaxf(__fadd_rn(m, eps), __fmaf_rn(fabsf(m), 0x1.00001p-24f, m));
 }
 
-__device__ __forceinline__ float relaxed(float zc, float m, float eps) { return zc > m ? zc : up(m, eps); }
+// The value a cell of elevation zc takes above its lowest neighbour m: on the
+// grid itself, and on a grid of blocks of n x n cells (a bound, see above).
+struct CellRaise {
+  float eps;
+  __device__ __forceinline__ float operator()(float zc, float m) const { return zc > m ? zc : up(m, eps); }
+};
+
+// up^n(x) <= x + n eps + n ulp(V), V the largest magnitude on the way, at most
+// (|x| + n eps)(1 + n 2^-22); ulp(V) <= 2^-23 V + 2^-149.  The factors leave
+// twice that and 8 2^-22 (|x| + n eps) more for this evaluation's roundings.
+struct BlockBound {
+  float a, b;
+  BlockBound(float n, float eps) : a(n * eps * 1.001f + (n + 8.0f) * 0x1p-22f * n * eps + 1e-38f), b((n + 8.0f) * 0x1p-22f) {}
+  __device__ __forceinline__ float of(float x) const { return __fadd_rn(__fmaf_rn(fabsf(x), b, x), a); }
+  __device__ __forceinline__ float operator()(float zc, float m) const { return of(fmaxf(zc, m)); }
+};
 
 __device__ __forceinline__ float min3(float a, float b, float c) {
   float r;
@@ -67,23 +98,86 @@ __device__ __forceinline__ float min3(float a, float b, float c) {
   return r;
 }
 
-// F = z on the grid's edge, +inf inside; non-finite z reported; the tiles on
-// the grid's border listed for the first round (no cell of another tile can
-// drop before one of them has: those start at +inf with +inf around)
-__global__ void k_fill_init(const float* z, int64_t H, int64_t W, int64_t ldz, float* F, int64_t ldF, int64_t ntx,
-                            int64_t nty, uint32_t* list, uint32_t* count, uint32_t* status) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// A level's start: its edge at z (blocks: at their bound), the inside at the
+// bounds of the next coarser level, or +inf without one; its tiles listed for
+// the first round, only those on its border when the inside is at +inf (no
+// other cell can drop before one of them has).  check: report non-finite z.
+template <class Raise>
+__global__ void k_fill_init(const float* z, int64_t H, int64_t W, int64_t ldz, float* F, int64_t ldF, Raise raise,
+                            const float* coarse, int64_t cW, int64_t ntx, int64_t nty, uint32_t* list,
+                            uint32_t* count, bool check, uint32_t* status) {
+  const int64_t stride = (int64_t)gridDim.x * gridDim.y * blockDim.x;
+  const int64_t t0 = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
   bool bad = false;
-  for (int64_t c = t0; c < H * W; c += stride) {
-    const int64_t i = c / W, j = c - i * W;
-    const float zc = z[i * ldz + j];
-    bad |= !isfinite(zc);
-    const bool edge = i == 0 || j == 0 || i == H - 1 || j == W - 1;
-    F[i * ldF + j] = edge ? zc : INFINITY;
+  // RATIO cells of a row per thread: they share one coarser cell
+  const int64_t j0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * RATIO;
+  const bool vec = (reinterpret_cast<uintptr_t>(F) & 15u) == 0 && ldF % RATIO == 0 && j0 + RATIO <= W;
+  for (int64_t i = blockIdx.y; i < H && j0 < W; i += gridDim.y) {
+    const float inside = coarse ? __ldg(&coarse[(i / RATIO) * cW + j0 / RATIO]) : INFINITY;
+    const bool row_edge = i == 0 || i == H - 1;
+    float v[RATIO];
+#pragma unroll
+    for (int k = 0; k < RATIO; k++) {
+      const int64_t j = j0 + k;
+      const bool edge = row_edge || j == 0 || j == W - 1;
+      v[k] = inside;
+      if (j < W && (edge || check)) {
+        const float zc = z[i * ldz + j];
+        bad |= check && !isfinite(zc);
+        if (edge) v[k] = zc;
+        if constexpr (std::is_same<Raise, BlockBound>::value)
+          if (edge) v[k] = raise.of(zc);
+      }
+    }
+    float* dst = F + i * ldF + j0;
+    if (vec) {
+      *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < RATIO; k++)
+        if (j0 + k < W) dst[k] = v[k];
+    }
   }
   for (int64_t t = t0; t < ntx * nty; t += stride) {
     const int64_t ty = t / ntx, tx = t - ty * ntx;
-    if (ty == 0 || tx == 0 || ty == nty - 1 || tx == ntx - 1) list[atomicAdd(count, 1u)] = (uint32_t)t;
+    if (coarse)
+      list[t] = (uint32_t)t;
+    else if (ty == 0 || tx == 0 || ty == nty - 1 || tx == ntx - 1)
+      list[atomicAdd(count, 1u)] = (uint32_t)t;
+  }
+  if (coarse && t0 == 0) *count = (uint32_t)(ntx * nty);
+  if (__syncthreads_or(bad) && threadIdx.x == 0) set_status(status, D8_ERR_NONFINITE);
+}
+
+// highest z of each RATIO x RATIO block (vec: rows of z are 16-byte aligned);
+// check: report non-finite z
+__global__ void k_fill_pool(const float* z, int64_t H, int64_t W, int64_t ldz, float* zc, int64_t cH, int64_t cW,
+                            bool vec, bool check, uint32_t* status) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  bool bad = false;
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < cH * cW; c += stride) {
+    const int64_t bi = c / cW, bj = c - bi * cW;
+    const int h = (int)min64(RATIO, H - bi * RATIO), w = (int)min64(RATIO, W - bj * RATIO);
+    const float* p = z + bi * RATIO * ldz + bj * RATIO;
+    float m = -INFINITY;
+    bool fin = true;
+#pragma unroll
+    for (int i = 0; i < RATIO; i++) {
+      if (i >= h) break;
+      if (vec && w == RATIO) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(p + i * ldz));
+        m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+        fin &= isfinite(v.x) && isfinite(v.y) && isfinite(v.z) && isfinite(v.w);
+      } else {
+        for (int j = 0; j < w; j++) {
+          const float v = __ldg(p + i * ldz + j);
+          m = fmaxf(m, v);
+          fin &= isfinite(v);
+        }
+      }
+    }
+    zc[c] = m;
+    bad |= check && !fin;
   }
   if (__syncthreads_or(bad) && threadIdx.x == 0) set_status(status, D8_ERR_NONFINITE);
 }
@@ -99,8 +193,8 @@ __global__ void k_fill_init(const float* z, int64_t H, int64_t W, int64_t ldz, f
 // issued before step q's store.  The chain per step is shuffle, minimum,
 // raise, select, minimum: about 50 cycles; the strides are compile-time
 // constants so that a step is about 20 instructions.
-template <int DS, int DL>
-__device__ __forceinline__ bool relax_pass(float* f, const float* zc, float eps) {
+template <int DS, int DL, class Raise>
+__device__ __forceinline__ bool relax_pass(float* f, const float* zc, Raise raise) {
   float su = f[-DS - DL], l = f[-DS], sd = f[-DS + DL];
   float cu = f[-DL], c = f[0], cd = f[DL];
   float ru = f[DS - DL], r = f[DS], rd = f[DS + DL];
@@ -118,7 +212,7 @@ __device__ __forceinline__ bool relax_pass(float* f, const float* zc, float eps)
     }
     const float beside = fminf(cu, cd);
     const float known = fminf(l, min3(min3(ru, r, rd), beside, behind));
-    const float v = relaxed(zq, min3(su, sd, known), eps);
+    const float v = raise(zq, min3(su, sd, known));
     changed |= v < c;
     c = fminf(v, c);
     f[0] = c;
@@ -140,21 +234,23 @@ __device__ __forceinline__ bool relax_pass(float* f, const float* zc, float eps)
 }
 
 // pass k: line tid left to right, right to left, then down, up
-__device__ __forceinline__ bool relax_dir(int k, float* Fh, const float* zh, float eps) {
+template <class Raise>
+__device__ __forceinline__ bool relax_dir(int k, float* Fh, const float* zh, Raise raise) {
   const int p = threadIdx.x + 1, row = p * RS, a = row + 1, b = row + T, c = RS + p, d = T * RS + p;
   switch (k & 3) {
-    case 0: return relax_pass<1, RS>(Fh + a, zh + a, eps);
-    case 1: return relax_pass<-1, RS>(Fh + b, zh + b, eps);
-    case 2: return relax_pass<RS, 1>(Fh + c, zh + c, eps);
-    default: return relax_pass<-RS, 1>(Fh + d, zh + d, eps);
+    case 0: return relax_pass<1, RS>(Fh + a, zh + a, raise);
+    case 1: return relax_pass<-1, RS>(Fh + b, zh + b, raise);
+    case 2: return relax_pass<RS, 1>(Fh + c, zh + c, raise);
+    default: return relax_pass<-RS, 1>(Fh + d, zh + d, raise);
   }
 }
 
 // One round over the listed tiles.  list / count: this round's tiles;
 // next / next_count: the tiles listed for the next round, each once
 // (mark[t] = stamp once t is listed).
+template <class Raise>
 __global__ void __launch_bounds__(NTF) k_fill_round(const float* z, int64_t H, int64_t W, int64_t ldz, float* F,
-                                                    int64_t ldF, float eps, int64_t ntx, int64_t nty,
+                                                    int64_t ldF, Raise raise, int64_t ntx, int64_t nty,
                                                     const uint32_t* list, const uint32_t* count, uint32_t* next,
                                                     uint32_t* next_count, uint32_t* queue, uint32_t* mark,
                                                     uint32_t stamp) {
@@ -192,7 +288,7 @@ __global__ void __launch_bounds__(NTF) k_fill_round(const float* z, int64_t H, i
     __syncthreads();
     bool any = false, settled = false;
     for (int k = 0; k < MAX_PASSES; k++) {
-      if (!__syncthreads_or(relax_dir(k, Fh, zh, eps))) {
+      if (!__syncthreads_or(relax_dir(k, Fh, zh, raise))) {
         settled = true;
         break;
       }
@@ -215,7 +311,7 @@ __global__ void __launch_bounds__(NTF) k_fill_round(const float* z, int64_t H, i
           const int a = hi + code_di(k), b = hj + code_dj(k);
           if (a >= 1 && b >= 1 && a <= T && b <= T) m = fminf(m, Fh[a * RS + b]);
         }
-        if (relaxed(zh[hi * RS + hj], m, eps) < Fh[hi * RS + hj]) {
+        if (raise(zh[hi * RS + hj], m) < Fh[hi * RS + hj]) {
           const int di = hi == 0 ? 0 : hi == HW - 1 ? 2 : 1, dj = hj == 0 ? 0 : hj == HW - 1 ? 2 : 1;
           atomicOr(dirs, 1u << (3 * di + dj));
         }
@@ -231,67 +327,181 @@ __global__ void __launch_bounds__(NTF) k_fill_round(const float* z, int64_t H, i
 
 }  // namespace fill
 
-constexpr int CHUNK = 16;  // rounds between host checks
+namespace fill {
 
-// workspace: counts of listed tiles (CHUNK + 1) and work queues (CHUNK), one
-// mark and two list entries per tile
-size_t fill_ws_bytes(int64_t H, int64_t W) {
-  const int64_t ntiles = ((H + fill::T - 1) / fill::T) * ((W + fill::T - 1) / fill::T);
-  return 256 + sizeof(uint32_t) * 3 * (size_t)ntiles;
+constexpr int CHUNK = 16;     // rounds between host checks, at most
+constexpr int FIRST = 8;      // rounds before the first check
+constexpr int MAX_LEVELS = 8;
+constexpr size_t HEAD = 256;  // bytes of a level's counts (CHUNK + 1) and work queues (CHUNK)
+static_assert(RATIO == 4, "k_fill_init and k_fill_pool move blocks' rows as float4");
+static_assert(sizeof(uint32_t) * (2 * CHUNK + 1) <= HEAD, "counts and queues fit the head");
+
+// A level's grid and its part of the workspace.  Level 0 is the grid itself.
+struct Level {
+  int64_t H, W, ntx, nty, ntiles;
+  const float* z;
+  int64_t ldz;
+  float* F;
+  int64_t ldF;
+  uint32_t* counts;  // counts[k]: tiles listed for round k of the chunk
+  uint32_t* queues;
+  uint32_t* mark;
+  uint32_t* list[2];
+};
+
+static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// Levels are added while the last one has more than one tile, for grids of
+// more than 8 tiles a side: smaller ones settle in about as many rounds as the
+// coarse grids would take (500 x 500: 343 us without levels, 400 with; 700 x
+// 933: 452 and 434; 3000 x 3000: 1464 and 934).  Returns their number; bytes: the workspace.
+// What must be zero at the start comes first, `zeroed` bytes of it.
+static int levels(int64_t H, int64_t W, void* ws, Level* lv, size_t* zeroed, size_t* bytes) {
+  int n = 0;
+  size_t at = 0;
+  char* base = static_cast<char*>(ws);
+  for (;;) {
+    Level& L = lv[n++];
+    L = Level{};
+    L.H = H;
+    L.W = W;
+    L.ntx = (W + T - 1) / T;
+    L.nty = (H + T - 1) / T;
+    L.ntiles = L.ntx * L.nty;
+    L.counts = reinterpret_cast<uint32_t*>(base + at);
+    L.queues = L.counts + CHUNK + 1;
+    L.mark = reinterpret_cast<uint32_t*>(base + at + HEAD);
+    at += HEAD + a256(sizeof(uint32_t) * (size_t)L.ntiles);
+    if (n == MAX_LEVELS || L.ntiles == 1 || (n == 1 && min64(L.ntx, L.nty) <= 8)) break;
+    H = (H + RATIO - 1) / RATIO;
+    W = (W + RATIO - 1) / RATIO;
+  }
+  *zeroed = at;
+  for (int l = 0; l < n; l++) {
+    Level& L = lv[l];
+    for (auto& q : L.list) {
+      q = reinterpret_cast<uint32_t*>(base + at);
+      at += a256(sizeof(uint32_t) * (size_t)L.ntiles);
+    }
+    if (l == 0) continue;
+    const size_t cells = a256(sizeof(float) * (size_t)L.H * (size_t)L.W);
+    L.z = reinterpret_cast<const float*>(base + at);
+    L.F = reinterpret_cast<float*>(base + at + cells);
+    L.ldz = L.ldF = L.W;
+    at += 2 * cells;
+  }
+  *bytes = at;
+  return n;
 }
 
-// The fill: init, then rounds until one lists nothing.  The host reads the
-// rounds' list counts every CHUNK rounds (synchronising the stream) and stops
-// after max_rounds with D8_ERR_TIMEOUT.
+static unsigned blocks_for(int64_t n, int sms) {
+  int64_t b = (n + 255) / 256;
+  if (b > (int64_t)sms * 16) b = (int64_t)sms * 16;
+  return (unsigned)(b < 1 ? 1 : b);
+}
+
+template <class Raise>
+static cudaError_t start_level(const Level& L, const Level* coarser, Raise raise, bool check, uint32_t* status, int sms,
+                               cudaStream_t s, int* nlaunch) {
+  const int64_t gx = (L.W + 256 * RATIO - 1) / (256 * RATIO);  // 256 threads, RATIO cells each, along a row
+  int64_t gy = (int64_t)sms * 16 / gx;
+  if (gy > L.H) gy = L.H;
+  if (gy > 65535) gy = 65535;
+  if (gy < 1) gy = 1;
+  k_fill_init<Raise><<<dim3((unsigned)gx, (unsigned)gy), 256, 0, s>>>(
+      L.z, L.H, L.W, L.ldz, L.F, L.ldF, raise, coarser ? coarser->F : nullptr, coarser ? coarser->W : 0, L.ntx, L.nty,
+      L.list[0], L.counts, check, status);
+  ++*nlaunch;
+  return cudaGetLastError();
+}
+
+// rounds first .. first + n - 1 of a level (n <= CHUNK), counts and queues at 0
+template <class Raise>
+static cudaError_t rounds(const Level& L, Raise raise, int64_t first, int n, int sms, cudaStream_t s, int* nlaunch) {
+  int per_sm = 1;
+  auto kern = k_fill_round<Raise>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Layout::bytes);
+  if (e != cudaSuccess) return e;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NTF, Layout::bytes) != cudaSuccess || per_sm < 1) {
+    cudaGetLastError();
+    per_sm = 1;
+  }
+  const int64_t grid = min64((int64_t)per_sm * sms, L.ntiles);
+  for (int k = 0; k < n; k++) {
+    const int64_t r = first + k;
+    kern<<<(unsigned)grid, NTF, Layout::bytes, s>>>(L.z, L.H, L.W, L.ldz, L.F, L.ldF, raise, L.ntx, L.nty,
+                                                    L.list[r & 1], L.counts + k, L.list[(r + 1) & 1],
+                                                    L.counts + k + 1, L.queues + k, L.mark, (uint32_t)(r + 1));
+    ++*nlaunch;
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace fill
+
+size_t fill_ws_bytes(int64_t H, int64_t W) {
+  fill::Level lv[fill::MAX_LEVELS];
+  size_t zeroed, bytes;
+  fill::levels(H, W, nullptr, lv, &zeroed, &bytes);
+  return bytes;
+}
+
+// The fill: the coarser levels from the coarsest, then the grid itself in
+// rounds until one lists nothing.  The host reads the rounds' list counts
+// every CHUNK rounds (synchronising the stream) and stops after max_rounds
+// with D8_ERR_TIMEOUT.
 cudaError_t run_fill(const float* z, int64_t H, int64_t W, int64_t ldz, float eps, float* F, int64_t ldF, void* ws,
                      uint32_t* status, cudaStream_t s, int64_t max_rounds, int64_t* rounds_out, bool* timed_out,
                      int* nlaunch) {
   using namespace fill;
-  const int64_t ntx = (W + T - 1) / T, nty = (H + T - 1) / T, ntiles = ntx * nty;
-  static_assert(sizeof(uint32_t) * (2 * CHUNK + 1) <= 256, "counts and queues fit the workspace's head");
-  uint32_t* counts = static_cast<uint32_t*>(ws);  // counts[k]: tiles listed for round k of the chunk
-  uint32_t* queues = counts + CHUNK + 1;
-  uint32_t* mark = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + 256);
-  uint32_t* list[2] = {mark + ntiles, mark + 2 * ntiles};
-  *timed_out = false;
+  Level lv[MAX_LEVELS];
+  size_t zeroed, bytes;
+  const int n = levels(H, W, ws, lv, &zeroed, &bytes);
+  Level& G = lv[0];
+  G.z = z;
+  G.ldz = ldz;
+  G.F = F;
+  G.ldF = ldF;
   eps = fmaxf(eps, 0x1p-149f);  // see up()
-  int dev = 0, sms = 1, per_sm = 1;
+  *timed_out = false;
+  int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaError_t e = cudaFuncSetAttribute(k_fill_round, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Layout::bytes);
-  if (e != cudaSuccess) return e;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fill_round, NTF, Layout::bytes) != cudaSuccess ||
-      per_sm < 1) {
-    cudaGetLastError();
-    per_sm = 1;
+  cudaError_t e = cudaMemsetAsync(ws, 0, zeroed, s);
+  for (int l = 1; l < n && e == cudaSuccess; l++) {
+    const Level &f = lv[l - 1], &c = lv[l];
+    const bool vec = (reinterpret_cast<uintptr_t>(f.z) & 15u) == 0 && f.ldz % 4 == 0;
+    k_fill_pool<<<blocks_for(c.H * c.W, sms), 256, 0, s>>>(f.z, f.H, f.W, f.ldz, const_cast<float*>(c.z), c.H, c.W, vec,
+                                                           l == 1, status);
+    ++*nlaunch;
+    e = cudaGetLastError();
   }
-  int64_t grid = (int64_t)per_sm * sms;
-  if (grid > ntiles) grid = ntiles;
-  e = cudaMemsetAsync(ws, 0, 256 + sizeof(uint32_t) * (size_t)ntiles, s);
+  for (int l = n - 1; l >= 1 && e == cudaSuccess; l--) {
+    const BlockBound bound((float)(1 << (2 * l)), eps);
+    e = start_level(lv[l], l + 1 < n ? &lv[l + 1] : nullptr, bound, false, status, sms, s, nlaunch);
+    // a change crosses about two tiles a round where it matters: bounds left
+    // higher than they could be only cost the finer level visits
+    const int64_t side = lv[l].ntx > lv[l].nty ? lv[l].ntx : lv[l].nty;
+    const int r = side == 1 ? 1 : (int)min64(CHUNK, 3 + side / 2);
+    if (e == cudaSuccess) e = rounds(lv[l], bound, 0, r, sms, s, nlaunch);
+  }
+  if (e == cudaSuccess) e = start_level(G, n > 1 ? &lv[1] : nullptr, CellRaise{eps}, n == 1, status, sms, s, nlaunch);
   if (e != cudaSuccess) return e;
-  int64_t nb = (H * W + 255) / 256;
-  if (nb > (int64_t)sms * 16) nb = (int64_t)sms * 16;
-  k_fill_init<<<(unsigned)(nb < 1 ? 1 : nb), 256, 0, s>>>(z, H, W, ldz, F, ldF, ntx, nty, list[0], counts, status);
-  ++*nlaunch;
   int64_t r = 0;
   for (;;) {
-    for (int k = 0; k < CHUNK; k++, r++) {
-      k_fill_round<<<(unsigned)grid, NTF, Layout::bytes, s>>>(z, H, W, ldz, F, ldF, eps, ntx, nty, list[r & 1],
-                                                              counts + k, list[(r + 1) & 1], counts + k + 1,
-                                                              queues + k, mark, (uint32_t)(r + 1));
-      ++*nlaunch;
-    }
+    const int m = r == 0 ? FIRST : CHUNK;
+    e = rounds(G, CellRaise{eps}, r, m, sms, s, nlaunch);
+    r += m;
     uint32_t h[CHUNK + 1];
-    e = cudaMemcpyAsync(h, counts, sizeof(h), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, G.counts, sizeof(uint32_t) * (m + 1), cudaMemcpyDeviceToHost, s);
     // the last count is the next chunk's first
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(counts, counts + CHUNK, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(counts + 1, 0, sizeof(uint32_t) * 2 * CHUNK, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(G.counts, G.counts + m, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(G.counts + 1, 0, sizeof(uint32_t) * 2 * CHUNK, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
-    for (int k = 1; k <= CHUNK; k++) {
+    for (int k = 1; k <= m; k++) {
       if (h[k] == 0) {  // the first round that listed nothing
-        *rounds_out = r - CHUNK + k;
+        *rounds_out = r - m + k;
         return cudaGetLastError();
       }
     }

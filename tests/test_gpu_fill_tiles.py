@@ -11,14 +11,14 @@ import oracle
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [(3, 700), (63, 65), (64, 64), (66, 127), (97, 33), (129, 191), (193, 256), (320, 66)]
+SHAPES = [(3, 700), (63, 65), (64, 64), (66, 127), (97, 33), (129, 191), (193, 256), (320, 66), (577, 643)]  # the last with coarse levels
 
 
 def _surfaces(H, W):
     rng = np.random.default_rng(H * 1000 + W)
     yield "fractal", demgen.fractal_raw(H, W, seed=H * 7 + W) - np.float32(500.0)
     yield "pits", rng.integers(-3, 4, size=(H, W)).astype(np.float32) * np.float32(0.5)
-    z = np.ascontiguousarray(demgen.serpentine_dem(321, 700)[:H, :W])
+    z = np.ascontiguousarray(demgen.serpentine_dem(577, 700)[:H, :W])
     z[H // 2, W // 2] = z.max()  # a dam across the channel: everything above it fills
     yield "serpentine", z
 
