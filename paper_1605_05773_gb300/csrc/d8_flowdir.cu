@@ -2,245 +2,415 @@
 // over the eight neighbours, slope = drop / distance between cell centres;
 // "Introduction": lowest neighbour) as a streaming kernel.
 //
-// Reads 4 bytes of z and writes 1 byte of code per cell, so it is bound by
-// HBM bandwidth, which needs tens of KB in flight per SM.  GB300 layout:
-//  * one warp per T x T tile of the pipeline's tiling (so a batch of DEMs
-//    maps onto warps through the same tile table); the warp streams down the
-//    tile's rows, each row buffered in shared memory with the columns
-//    j0 - 4 .. j0 + T + 3 around it (the halo columns, widened to 16-byte
-//    boundaries);
-//  * rows are fetched PD = 6 rows ahead with cp.async into a per-warp ring,
-//    so the bytes in flight cost no registers: 16-byte zero-filling copies
-//    when the rows of z are 16-byte aligned, 4-byte copies otherwise;
-//  * each lane owns T/32 adjacent columns; it takes them from the ring with
-//    one vector load per row, the neighbouring columns with warp shuffles,
-//    and keeps a three-row window in registers;
-//  * codes leave as one packed store per lane per row.
+// Reads 4 bytes of z and writes 1 byte of code per cell.  The comparisons and
+// selections run at half the rate of the additions, so they, not HBM, bound
+// it; the layout below is chosen to need few of them:
+//  * a lane owns 4 adjacent columns and walks down its rows; T / 4 lanes make
+//    a tile of the pipeline's tiling, so a warp takes 4, 2 or 1 tiles (T = 32,
+//    64, 128) and a batch of DEMs maps onto warps through the tile table;
+//  * rows go through a ring of PD rows per tile in shared memory by
+//    asynchronous copies (16 bytes per lane), PD - 1 rows ahead; loads into
+//    registers waited for one another instead (a warp has six scoreboards);
+//    a lane reads its four columns and the two beside them;
+//  * steepest: the slope towards a neighbour is the exact negation of the
+//    neighbour's slope back, so each difference is formed once and serves two
+//    cells (E / W, S / N, SE / NW, SW / NE: 7.25 operations per cell, not 12);
+//  * the lowest of the eight values comes from four three-input minima, and
+//    the code from five comparisons and predicated additions;
+//  * whole items inside the grid run a loop without any of the edges' tests
+//    (walk_inside); an item at the grid's edge, or one in which a non-finite
+//    elevation turned up, runs the general one (walk_any).
+// Rows that are not 16-byte aligned take 4-byte copies.  Grids
+// with few tiles are cut into shorter row segments, so that a small call
+// still fills the GPU (launch_t).
+//
+// Measured (steepest): 32768 x 32768 1.31 ms, 4.1 TB/s (before: 2.90 ms, one
+// warp per tile, 2 columns per lane, eight ordered compare-and-selects per
+// cell); 8192 x 8192 98 us (195), 3001 x 5003 lowest with masks 50 us (84), 512
+// x 512 9.5 us (27).  41 warp instructions per 32 cells, 79 % issue active,
+// half-rate pipe 65 % busy, DRAM 42 %.
 #include "d8_device.cuh"
 
 namespace d8 {
 namespace fdir {
 
-constexpr int NTF = 128;  // threads per block: four warps, four tiles
-constexpr int WPB = NTF / 32;
-constexpr int PD = 6;  // rows in flight per warp
+constexpr int NTF = 128;  // threads per block
+constexpr int CPL = 4;    // columns per lane
+constexpr int PD = 8;     // rows of the ring
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
-// D8 code of an interior cell from its 3x3 window (a = row above, b = own
-// row, c = row below; 0 = left, 1 = centre, 2 = right).  Steepest: the slope
-// towards neighbour n is (z - zn) for a cardinal and (z - zn) * R for a
-// diagonal with R = fp32(1/sqrt 2), one rounded multiply; it is formed here as
-// the exact negation (zn - z) [* R] with packed fp32x2 arithmetic (cardinals
-// paired with cardinals, diagonals with diagonals for the multiply) and the
-// most negative one wins.  Comparisons are strict and in N, NE, E, SE, S, SW,
-// W, NW order, so the first of equal slopes wins and only a strictly positive
-// drop counts.  Lowest: the smallest neighbour below z, same tie rule.
-__device__ __forceinline__ int window_code(float a0, float a1, float a2, float b0, float b1, float b2, float c0,
-                                           float c1, float c2, int rule) {
-  int code = 9;
-  if (rule == 0) {
-    const float2 nz = make_float2(-b1, -b1);
-    const float2 rr = make_float2(inv_sqrt2_f32(), inv_sqrt2_f32());
-    const float2 ne = __fadd2_rn(make_float2(a1, b2), nz);                        // N, E
-    const float2 sw = __fadd2_rn(make_float2(c1, b0), nz);                        // S, W
-    const float2 d0 = __fmul2_rn(__fadd2_rn(make_float2(a2, c2), nz), rr);        // NE, SE
-    const float2 d1 = __fmul2_rn(__fadd2_rn(make_float2(c0, a0), nz), rr);        // SW, NW
-    float best = 0.0f;
-    if (ne.x < best) { best = ne.x; code = 0; }
-    if (d0.x < best) { best = d0.x; code = 1; }
-    if (ne.y < best) { best = ne.y; code = 2; }
-    if (d0.y < best) { best = d0.y; code = 3; }
-    if (sw.x < best) { best = sw.x; code = 4; }
-    if (d1.x < best) { best = d1.x; code = 5; }
-    if (sw.y < best) { best = sw.y; code = 6; }
-    if (d1.y < best) { best = d1.y; code = 7; }
-  } else {
-    float best = b1;
-    if (a1 < best) { best = a1; code = 0; }
-    if (a2 < best) { best = a2; code = 1; }
-    if (b2 < best) { best = b2; code = 2; }
-    if (c2 < best) { best = c2; code = 3; }
-    if (c1 < best) { best = c1; code = 4; }
-    if (c0 < best) { best = c0; code = 5; }
-    if (b0 < best) { best = b0; code = 6; }
-    if (a0 < best) { best = a0; code = 7; }
-  }
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
+// x = v where a == b, on the addition pipe: v + nz with nz = -0 is v
+__device__ __forceinline__ void set_if_eq(float a, float b, float& x, float v, float nz) {
+  asm("{.reg .pred p; setp.eq.f32 p, %1, %2; @p add.f32 %0, %3, %4;}" : "+f"(x) : "f"(a), "f"(b), "f"(v), "f"(nz));
+}
+__device__ __forceinline__ void set3_if_eq(float a, float b, float& x, float xv, float& y, float yv, float& c, float cv,
+                                           float nz) {
+  asm("{.reg .pred p; setp.eq.f32 p, %3, %4; @p add.f32 %0, %5, %8; @p add.f32 %1, %6, %8; @p add.f32 %2, %7, %8;}"
+      : "+f"(x), "+f"(y), "+f"(c)
+      : "f"(a), "f"(b), "f"(xv), "f"(yv), "f"(cv), "f"(nz));
+}
+
+// Code (plus `add`, as a float) of the lowest of the eight values, in the
+// order N, NE, E, SE, S, SW, W, NW: the first of equal ones, if it is below
+// `than`, else SINK.  NaN values are never the lowest and never equal to it.
+// The values are grouped 3 + 3 + 2: the first group that holds the minimum,
+// then the place in it, is four minima, five comparisons and eight predicated
+// additions (nz = -0, unknown to the compiler, which would make them
+// selections): comparisons, minima and selections run at half the rate of
+// additions and are what bounds the kernel.
+__device__ __forceinline__ float lowest_code(float v0, float v1, float v2, float v3, float v4, float v5, float v6,
+                                             float v7, float than, float add, float nz) {
+  const float g0 = min3(v0, v1, v2), g1 = min3(v3, v4, v5);
+  const float m = min3(g0, g1, fminf(v6, v7));
+  // first and second value of the group (copies, also as additions); code of its third
+  float x = __fadd_rn(v6, nz), y = __fadd_rn(v7, nz), third = add + 8.0f;
+  set3_if_eq(g1, m, x, v3, y, v4, third, add + 5.0f, nz);
+  set3_if_eq(g0, m, x, v0, y, v1, third, add + 2.0f, nz);
+  float code = third;
+  set_if_eq(y, m, code, third, -1.0f);
+  set_if_eq(x, m, code, third, -2.0f);
+  asm("{.reg .pred p; setp.geu.f32 p, %1, %2; @p add.f32 %0, %3, %4;}" : "+f"(code) : "f"(m), "f"(than), "f"(add + 9.0f), "f"(nz));
   return code;
 }
 
+// four codes, those of the even columns with 2^23 added, as bytes
+__device__ __forceinline__ uint32_t pack_codes(float c0, float c1, float c2, float c3) {
+  const float lo = __fmaf_rn(c1, 256.0f, c0), hi = __fmaf_rn(c3, 256.0f, c2);  // exact: below 2^24
+  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x5410);
+}
+constexpr float EVEN = 0x1p23f;
+
+// One row as a lane sees it: columns jb - 1 .. jb + 4.
+struct Row {
+  float v[CPL + 2];
+};
+
+// The slopes between a row b and the row c below it, as drops towards the
+// lower row are negative: S of each own column; SE of columns -1 .. 3 and SW
+// of columns 0 .. 4, each one rounded difference and one rounded product with
+// R = fp32(1/sqrt 2).  Negated they are c's N, NW and NE slopes.
+struct Slopes {
+  float s[CPL], se[CPL + 1], sw[CPL + 1];
+};
+
+__device__ __forceinline__ Slopes slopes_between(const Row& b, const Row& c) {
+  Slopes o;
+#pragma unroll
+  for (int k = 0; k < CPL; k++) o.s[k] = __fsub_rn(c.v[k + 1], b.v[k + 1]);
+#pragma unroll
+  for (int k = 0; k <= CPL; k++) {
+    o.se[k] = __fmul_rn(__fsub_rn(c.v[k + 1], b.v[k]), inv_sqrt2_f32());
+    o.sw[k] = __fmul_rn(__fsub_rn(c.v[k], b.v[k + 1]), inv_sqrt2_f32());
+  }
+  return o;
+}
+
+// The codes of a lane's four cells in row b, as bytes; a and c the rows above
+// and below it, up and dn the slopes between them (a is unused by the
+// steepest rule, up and dn by the lowest).
+template <bool LOWEST>
+__device__ __forceinline__ uint32_t row_codes(const Row& a, const Row& b, const Row& c, const Slopes& up,
+                                              const Slopes& dn, float nz) {
+  float code[CPL], e[CPL + 1];  // e: E slope of columns -1 .. 3; negated, the W slope of columns 0 .. 4
+#pragma unroll
+  for (int k = 0; k <= CPL; k++) e[k] = LOWEST ? 0.0f : __fsub_rn(b.v[k + 1], b.v[k]);
+#pragma unroll
+  for (int k = 0; k < CPL; k++) {
+    const float add = k & 1 ? 0.0f : EVEN;
+    code[k] = LOWEST ? lowest_code(a.v[k + 1], a.v[k + 2], b.v[k + 2], c.v[k + 2], c.v[k + 1], c.v[k], b.v[k], a.v[k],
+                                   b.v[k + 1], add, nz)
+                     : lowest_code(-up.s[k], -up.sw[k + 1], e[k + 1], dn.se[k + 1], dn.s[k], dn.sw[k], -e[k],
+                                   -up.se[k], 0.0f, add, nz);
+  }
+  return pack_codes(code[0], code[1], code[2], code[3]);
+}
+
+// A lane's part of a work item: rows 0 .. n - 1 of four columns of a tile.
+struct Item {
+  const float* z;     // row -1, first own column (only formed, not read, when off the grid)
+  const float* h;     // row -1, the column beside the tile for its first and last lane, else z
+  int64_t ldz, lddir;
+  uint8_t* dir;       // row 0, first own column
+  int n, ncols;       // rows; own columns present
+  bool first, last;   // the tile's first, last lane
+  bool hval;          // h's column is on the grid
+  bool right;         // the column right of the tile is on the grid
+  int qlo, qhi;       // rows q - 1, q in [qlo, qhi), are on the grid (or in the halo of a strip)
+  int top, bottom;    // the row that is the grid's first, last; negative if none is
+  uint32_t colmask;   // bytes of the columns on the grid's edge
+};
+
+__device__ __forceinline__ Row row_of(const Item& it, const float (&x)[CPL], float h) {
+  Row r;
+#pragma unroll
+  for (int k = 0; k < CPL; k++) r.v[k + 1] = x[k];
+  const float l = __shfl_up_sync(FULL, x[CPL - 1], 1), e = __shfl_down_sync(FULL, x[0], 1);
+  r.v[0] = it.first ? h : l;
+  r.v[CPL + 1] = it.last ? h : e;
+  return r;
+}
+
+// NaN when a value of the row is not finite (the own columns; NODATA: also the
+// ones beside), else acc
+template <bool NODATA>
+__device__ __forceinline__ float nonfinite(const Row& r, float acc) {
+#pragma unroll
+  for (int k = NODATA ? 0 : 1; k < CPL + (NODATA ? 2 : 1); k++) acc = __fmaf_rn(r.v[k], 0.0f, acc);
+  return acc;
+}
+
+// asynchronous copies under a predicate (no branch around them)
+__device__ __forceinline__ void copy16_if(bool on, float* dst, const float* src) {
+  asm volatile("{.reg .pred p; setp.ne.s32 p, %2, 0; @p cp.async.cg.shared.global [%0], [%1], 16;}"
+               :: "r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"((int)on) : "memory");
+}
+__device__ __forceinline__ void copy4_if(bool on, float* dst, const float* src) {
+  asm volatile("{.reg .pred p; setp.ne.s32 p, %2, 0; @p cp.async.ca.shared.global [%0], [%1], 4;}"
+               :: "r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"((int)on) : "memory");
+}
+
+// Items whose rows -1 .. n and own columns all lie on the grid and whose n is
+// a multiple of 4.  ring: PD rows of RW floats, columns j0 - 4 .. j0 + T + 3
+// of the tile; row k sits at place (k + 7) % 8.  Returns whether the warp met
+// a non-finite elevation (the codes are then redone by walk_any).
+template <int T, bool LOWEST, bool NODATA, bool VEC>
+__device__ __forceinline__ bool walk_inside(Item it, float* ring, float nz) {
+  constexpr int LPT = T / CPL, RW = T + 8;
+  static_assert(PD == 8, "places of rows in the ring");
+  const int li = (threadIdx.x & 31) & (LPT - 1);
+  // this lane's part of a row's copy: its own columns and, for the first and
+  // last lane, the one beside the tile; or the columns li, li + LPT, ... of
+  // those from j0 - 1 on
+  const float* src = VEC ? it.z : it.z - li * CPL - 1 + li;
+  const int own = VEC ? CPL + li * CPL : CPL - 1 + li;
+  const int beside = it.first ? CPL - 1 : CPL + T;
+  const bool lo = li > 0 || it.hval, hi = li == 1 && it.right;  // !VEC: the first and the last column are on the grid
+  auto fetch = [&](float* row, bool on) {
+    if (VEC) {
+      copy16_if(on, row + own, src);
+      copy4_if(on && it.hval, row + beside, it.h);
+    } else {
+      copy4_if(on && lo, row + own, src);
+#pragma unroll
+      for (int k = 1; k < CPL; k++) copy4_if(on, row + own + k * LPT, src + k * LPT);
+      copy4_if(on && (li == 0 || hi), row + own + CPL * LPT, src + CPL * LPT);
+    }
+    cp_async_commit();
+    src += it.ldz;
+    it.h += it.ldz;
+  };
+  const int mine = li * CPL;
+  auto take = [&](const float* row) {
+    cp_async_wait<PD - 2>();
+    __syncwarp();  // every lane's part has landed, and every lane is done with the row before this one
+    Row r;
+    const float4 v = *reinterpret_cast<const float4*>(row + CPL + mine);
+    r.v[0] = row[CPL - 1 + mine];
+    r.v[1] = v.x;
+    r.v[2] = v.y;
+    r.v[3] = v.z;
+    r.v[4] = v.w;
+    r.v[5] = row[2 * CPL + mine];
+    return r;
+  };
+#pragma unroll
+  for (int k = -1; k < PD - 2; k++) fetch(ring + ((k + PD - 1) % PD) * RW, true);
+  Row a = take(ring + 6 * RW);
+  fetch(ring + 5 * RW, true);  // row 6
+  Row b = take(ring + 7 * RW);
+  fetch(ring + 6 * RW, true);  // row 7
+  Slopes up, dn;
+  if (!LOWEST) up = slopes_between(a, b);
+  float acc = nonfinite<NODATA>(b, NODATA ? nonfinite<NODATA>(a, 0.0f) : 0.0f);
+  bool redo = false;
+  for (int i = 0; i < it.n; i += 4) {
+    float *cur = ring + (i & 4) * RW, *other = ring + ((i & 4) ^ 4) * RW;
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      const Row c = take(cur + u * RW);
+      fetch(u ? cur + (u - 1) * RW : other + 3 * RW, i + u + PD <= it.n);  // row i + u + 8
+      acc = nonfinite<NODATA>(c, acc);
+      if (!LOWEST) dn = slopes_between(b, c);
+      uint32_t packed = row_codes<LOWEST>(a, b, c, up, dn, nz);
+      packed = (packed & ~it.colmask) | (0x08080808u & it.colmask);
+      if (VEC) {
+        *reinterpret_cast<uint32_t*>(it.dir) = packed;
+      } else {
+#pragma unroll
+        for (int k = 0; k < CPL; k++) it.dir[k] = (uint8_t)(packed >> (8 * k));
+      }
+      it.dir += it.lddir;
+      a = b;
+      b = c;
+      up = dn;
+    }
+    if (NODATA && __any_sync(FULL, acc != acc)) {
+      redo = true;
+      break;
+    }
+  }
+  cp_async_wait<0>();  // nothing may land in the ring after the item is done
+  __syncwarp();
+  return redo || __any_sync(FULL, acc != acc);
+}
+
+// Any item.  Off the grid rows and columns read as zero: they only neighbour
+// edge cells, whose code is OUTLET.  Returns whether an own cell of a rule
+// without masks is not finite.
+template <bool LOWEST, bool NODATA>
+__device__ __forceinline__ bool walk_any(Item it, float nz) {
+  auto load = [&](int q) {
+    float x[CPL] = {0.0f, 0.0f, 0.0f, 0.0f}, h = 0.0f;
+    if (q >= it.qlo && q < it.qhi) {
+#pragma unroll
+      for (int k = 0; k < CPL; k++)
+        if (k < it.ncols) x[k] = __ldg(it.z + k);
+      if (it.hval) h = __ldg(it.h);
+    }
+    it.z += it.ldz;
+    it.h += it.ldz;
+    return row_of(it, x, h);
+  };
+  const int nmax = __reduce_max_sync(FULL, it.n);
+  Row a = load(0), b = load(1), c = load(2);
+  Slopes up, dn;
+  if (!LOWEST) up = slopes_between(a, b);
+  bool report = false;
+  for (int i = 0; i < nmax; i++) {
+    const Row ahead = load(i + 3);
+    if (!LOWEST) dn = slopes_between(b, c);
+    uint32_t packed = row_codes<LOWEST>(a, b, c, up, dn, nz);
+    float bad = nonfinite<NODATA>(b, 0.0f);
+    if (NODATA) bad = nonfinite<NODATA>(a, nonfinite<NODATA>(c, bad));
+    if (bad != bad && i < it.n) {
+#pragma unroll
+      for (int k = 0; k < CPL; k++) {
+        const bool own = !isfinite(b.v[k + 1]);
+        bool any = own;
+        if (NODATA)
+          any |= !(isfinite(a.v[k]) && isfinite(a.v[k + 1]) && isfinite(a.v[k + 2]) && isfinite(b.v[k]) &&
+                   isfinite(b.v[k + 2]) && isfinite(c.v[k]) && isfinite(c.v[k + 1]) && isfinite(c.v[k + 2]));
+        if (any) packed = (packed & ~(0xFFu << (8 * k))) | ((NODATA ? 8u : 9u) << (8 * k));
+        report |= !NODATA && own;
+      }
+    }
+    const uint32_t m = (i == it.top || i == it.bottom) ? 0xFFFFFFFFu : it.colmask;
+    packed = (packed & ~m) | (0x08080808u & m);
+    if (i < it.n) {
+#pragma unroll
+      for (int k = 0; k < CPL; k++)
+        if (k < it.ncols) it.dir[k] = (uint8_t)(packed >> (8 * k));
+    }
+    it.dir += it.lddir;
+    a = b;
+    b = c;
+    c = ahead;
+    up = dn;
+  }
+  return report;
+}
 
 // NODATA masks (the rule's NODATA bit): a cell with a non-finite elevation is
 // outside the study area and gets OUTLET, and so does every cell next to one
 // (the area's edge drains off it, as the grid's edge does); nothing is
-// reported as an error.
-template <int T, bool NODATA>
-__global__ void __launch_bounds__(NTF) k_flowdir_rows(DemTable dt, int64_t ntiles, int rule, uint32_t* status) {
-  constexpr int CPL = T / 32;  // columns per lane
-  constexpr int RW = T + 8;    // floats per buffered row: columns j0 - 4 .. j0 + T + 3
-  static_assert(PD % 3 == 0, "the window index must be static in the unrolled loop");
-  __shared__ __align__(16) float ring_all[WPB * PD * RW];
-  float* ring = ring_all + (threadIdx.x >> 5) * (PD * RW);
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarps = (int64_t)gridDim.x * WPB;
-  for (int64_t t = (int64_t)blockIdx.x * WPB + (threadIdx.x >> 5); t < ntiles; t += nwarps) {
+// reported as an error.  seg_rows: rows per work item (a divisor of T).
+// nz: -0 (lowest_code).
+template <int T, bool LOWEST, bool NODATA>
+__global__ void __launch_bounds__(NTF, 5) k_flowdir_rows(DemTable dt, int64_t ntiles, int seg_rows, float nz,
+                                                         uint32_t* status) {
+  constexpr int LPT = T / CPL;   // lanes per tile
+  constexpr int IPW = 32 / LPT;  // items per warp
+  const int lane = threadIdx.x & 31, li = lane & (LPT - 1);
+  __shared__ __align__(16) float rings[NTF / LPT][PD * (T + 8)];
+  float* ring = rings[threadIdx.x / LPT];
+  const int nseg = T / seg_rows;
+  const int64_t nitems = ntiles * nseg;
+  const int64_t step = (int64_t)gridDim.x * (NTF / 32) * IPW;
+  const int64_t first = ((int64_t)blockIdx.x * (NTF / 32) + (threadIdx.x >> 5)) * IPW;
+  for (int64_t base = first; base < nitems; base += step) {
+    // the warp's items are consecutive; one past the end has no rows
+    const bool present = base + lane / LPT < nitems;
+    const int64_t item = present ? base + lane / LPT : nitems - 1;
+    const int64_t t = item / nseg;
     const DemDesc d = dem_of(dt, t);
     const TileGeo g = tile_geo(d, t - d.tile_base, T);
-    const bool vec = ((reinterpret_cast<uintptr_t>(d.z) & 15u) == 0) && ((d.ldz & 3) == 0);
-    const int jb = lane * CPL;  // first own column
-    const int nq = g.th + 2;    // rows q = 0 .. th + 1 are tile-local rows -1 .. th
-    // this lane's part of a buffered row: 16-byte chunks ch0 (and ch0 + 32
-    // when T = 128) or 4-byte elements lane, lane + 32, ...; the number of
-    // bytes of each that lie on the grid is the same for every row
-    constexpr int NCH = RW / 4;
-    const int64_t col0 = g.j0 - 4 + (vec ? 4 * lane : lane);
-    auto valid_bytes = [&](int64_t col) -> int {
-      if (vec) return col < 0 ? 0 : 4 * (int)min64(4, d.W - col < 0 ? 0 : d.W - col);
-      return (col >= 0 && col < d.W) ? 4 : 0;
-    };
-    const int nb0 = valid_bytes(col0);
-    const int nb1 = valid_bytes(col0 + (vec ? 128 : 32));
-    // rows q in [qlo, qhi) lie on the grid (the others only neighbour edge
-    // cells, whose code is OUTLET, and are never fetched); row q + PD is
-    // fetched while row q is used, from a pointer advanced by ldz per row
-    // (a strip of a taller grid also reads the row above its first row or
-    // below its last, d.halo, whose cells are then not grid edges)
-    const int qlo = (g.i0 == 0 && !(d.halo & 1)) ? 1 : 0;
-    const int qhi = (int)min64((int64_t)nq, d.H - g.i0 + ((d.halo & 2) ? 2 : 1));
-    // fetch() is called for q = 0, 1, 2, ... in order: a running row pointer
-    const float* fsrc = d.z + (g.i0 - 1) * d.ldz + col0;  // row q = 0; only formed, not read, when i0 == 0
-    int fq = 0;
-    auto fetch = [&](int slot) {
-      if (fq >= qlo && fq < qhi) {
-        float* dst = ring + slot * RW;
-        if (vec) {
-          if (lane < NCH) cp_async16(dst + 4 * lane, nb0 ? fsrc : d.z, nb0);
-          if (NCH > 32 && lane + 32 < NCH) cp_async16(dst + 4 * lane + 128, nb1 ? fsrc + 128 : d.z, nb1);
-        } else {
-          for (int c = lane, k = 0; c < RW; c += 32, k++) {
-            const int nb = k == 0 ? nb0 : (k == 1 ? nb1 : valid_bytes(col0 + 32 * k));
-            cp_async4(dst + c, nb ? fsrc + 32 * k : d.z, nb);
-          }
-        }
-      }
-      fsrc += d.ldz;
-      fq++;
-    };
-    // window row from ring slot `slot`: own columns, neighbours by shuffles
-    auto take = [&](float(&Wr)[CPL + 2], int slot) {
-      const float* row = ring + slot * RW + 4 + jb;
-      if (CPL == 4) {
-        const float4 v = *reinterpret_cast<const float4*>(row);
-        Wr[1] = v.x;
-        Wr[CPL > 1 ? 2 : 1] = v.y;
-        Wr[CPL > 2 ? 3 : 1] = v.z;
-        Wr[CPL > 3 ? 4 : 1] = v.w;
-      } else if (CPL == 2) {
-        const float2 v = *reinterpret_cast<const float2*>(row);
-        Wr[1] = v.x;
-        Wr[CPL > 1 ? 2 : 1] = v.y;
-      } else {
-        Wr[1] = row[0];
-      }
-      const float ls = __shfl_up_sync(FULL, Wr[CPL], 1);
-      const float rs = __shfl_down_sync(FULL, Wr[1], 1);
-      Wr[0] = lane == 0 ? row[-1] : ls;
-      Wr[CPL + 1] = lane == 31 ? row[CPL] : rs;
-    };
-    const int i_top_edge = (g.i0 == 0 && !(d.halo & 1)) ? 0 : -10;
-    const int i_bot_edge = (g.i0 + g.th == d.H && !(d.halo & 2)) ? g.th - 1 : -10;
-    const int ncols = max(0, min(CPL, g.tw - jb));  // own columns present
-    uint8_t* drow = d.dir + g.i0 * d.lddir + g.j0 + jb;  // emit() is called for rows 0, 1, 2, ... in order
-    const bool st_vec = (ncols == CPL) && ((reinterpret_cast<uintptr_t>(drow) & (CPL - 1)) == 0) &&
-                        (d.lddir % CPL == 0);
-    bool coledge[CPL];
+    const int r0 = (int)(item - t * nseg) * seg_rows;
+    const int64_t i0 = g.i0 + r0, gj = g.j0 + li * CPL;  // first row, first own column
+    Item it;
+    it.n = present ? max(0, min(seg_rows, g.th - r0)) : 0;
+    it.ncols = max(0, min(CPL, g.tw - li * CPL));
+    it.ldz = d.ldz;
+    it.lddir = d.lddir;
+    it.z = d.z + (i0 - 1) * d.ldz + gj;
+    it.dir = d.dir + i0 * d.lddir + gj;
+    it.first = li == 0;
+    it.last = li == LPT - 1;
+    it.right = g.j0 + T < d.W;
+    it.hval = it.first ? g.j0 > 0 : (it.last && it.right);
+    it.h = it.hval ? it.z + (it.first ? -1 : CPL) : it.z;
+    const bool above = i0 > 0 || (d.halo & 1), below = i0 + it.n < d.H || (d.halo & 2);
+    it.qlo = above ? 0 : 1;
+    it.qhi = it.n == 0 ? it.qlo : it.n + (below ? 2 : 1);
+    it.top = above ? -1 : 0;
+    it.bottom = below ? -1 : it.n - 1;
+    it.colmask = gj == 0 ? 0xFFu : 0u;
 #pragma unroll
-    for (int k = 0; k < CPL; k++) {
-      const int64_t gj = g.j0 + jb + k;
-      coledge[k] = (gj == 0) || (gj == d.W - 1);
+    for (int k = 0; k < CPL; k++)
+      if (gj + k == d.W - 1) it.colmask |= 0xFFu << (8 * k);
+    const bool inside = it.n == seg_rows && it.ncols == CPL && above && below;
+    const bool vec = ((reinterpret_cast<uintptr_t>(it.z) & 15u) == 0) && (d.ldz & 3) == 0 &&
+                     ((reinterpret_cast<uintptr_t>(it.dir) & 3u) == 0) && (d.lddir & 3) == 0;
+    bool redo = true;
+    if (__all_sync(FULL, inside)) {
+      redo = __all_sync(FULL, vec) ? walk_inside<T, LOWEST, NODATA, true>(it, ring, nz)
+                                    : walk_inside<T, LOWEST, NODATA, false>(it, ring, nz);
     }
-    auto emit = [&](const float(&U)[CPL + 2], const float(&M)[CPL + 2], const float(&D)[CPL + 2], int i) {
-      uint8_t* rowp = drow;
-      drow += d.lddir;
-      if (ncols == 0) return;
-      const bool redge = (i == i_top_edge) || (i == i_bot_edge);
-      uint32_t packed = 0;
-      bool bad = false;
-#pragma unroll
-      for (int k = 0; k < CPL; k++) {
-        const float zc = M[1 + k];
-        const bool fin = isfinite(zc);
-        int code;
-        if (redge || coledge[k]) {
-          code = 8;
-        } else if (!fin) {
-          code = NODATA ? 8 : 9;
-        } else if (NODATA && !(isfinite(U[k]) && isfinite(U[k + 1]) && isfinite(U[k + 2]) && isfinite(M[k]) &&
-                               isfinite(M[k + 2]) && isfinite(D[k]) && isfinite(D[k + 1]) && isfinite(D[k + 2]))) {
-          code = 8;
-        } else {
-          code = window_code(U[k], U[k + 1], U[k + 2], M[k], M[k + 1], M[k + 2], D[k], D[k + 1], D[k + 2], rule);
-        }
-        if (!NODATA) bad |= (k < ncols) && !fin;
-        packed |= (uint32_t)code << (8 * k);
-      }
-      if (bad) set_status(status, D8_ERR_NONFINITE);
-      if (st_vec) {
-        if (CPL == 4)
-          *reinterpret_cast<uint32_t*>(rowp) = packed;
-        else if (CPL == 2)
-          *reinterpret_cast<uint16_t*>(rowp) = (uint16_t)packed;
-        else
-          *rowp = (uint8_t)packed;
-      } else {
-#pragma unroll
-        for (int k = 0; k < CPL; k++)
-          if (k < ncols) rowp[k] = (uint8_t)(packed >> (8 * k));
-      }
-    };
-
-    // row q sits in slot q % PD; one cp.async group per row, so waiting until
-    // at most PD - 1 groups are pending means row q has landed
-#pragma unroll
-    for (int u = 0; u < PD; u++) {
-      fetch(u);
-      cp_async_commit();
-    }
-    float win[3][CPL + 2];
-    for (int qb = 0; qb < nq; qb += PD) {
-#pragma unroll
-      for (int u = 0; u < PD; u++) {
-        const int q = qb + u;
-        if (q < nq) {
-          cp_async_wait<PD - 1>();
-          __syncwarp();
-          take(win[u % 3], u);
-          __syncwarp();  // every lane has read the slot before it is refilled
-          fetch(u);  // row q + PD
-          cp_async_commit();
-          if (q >= 2) emit(win[(u + 1) % 3], win[(u + 2) % 3], win[u % 3], q - 2);
-        }
-      }
-    }
-    cp_async_wait<0>();  // nothing may land in the ring after the tile is done
-    __syncwarp();
+    if (redo && walk_any<LOWEST, NODATA>(it, nz)) set_status(status, D8_ERR_NONFINITE);
   }
 }
 
-template <int T>
-static cudaError_t launch_t(const DemTable& dt, int64_t ntiles, int rule, uint32_t* status, cudaStream_t s) {
+// Rows per item: whole tiles for grids that fill the GPU with them (two rows
+// in T are then read twice); below MIN_WARPS_PER_SM warps the tiles are cut
+// into segments of T / 2, T / 4, ... down to 8 rows.  (About 20 warps fit an
+// SM; with 40 here 8192 x 8192 runs 2.7 rounds of them and takes 122 us, with
+// 70 it halves its tiles and takes 98, with 140 it quarters them: 105.)
+constexpr int64_t MIN_WARPS_PER_SM = 70;
+
+template <int T, bool LOWEST, bool NODATA>
+static cudaError_t launch_t(const DemTable& dt, int64_t ntiles, uint32_t* status, cudaStream_t s) {
   int dev = 0, sms = 1, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  auto k = (rule & 2) ? k_flowdir_rows<T, true> : k_flowdir_rows<T, false>;
+  auto k = k_flowdir_rows<T, LOWEST, NODATA>;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NTF, 0) != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
     per_sm = 1;
   }
-  int64_t grid = (ntiles + WPB - 1) / WPB;
+  constexpr int IPW = 32 / (T / CPL), IPB = IPW * (NTF / 32);
+  int rows = T;
+  while (rows > 8 && ntiles * (T / rows) < MIN_WARPS_PER_SM * IPW * sms) rows /= 2;
+  int64_t grid = (ntiles * (T / rows) + IPB - 1) / IPB;
   const int64_t cap = (int64_t)sms * per_sm;
   if (grid > cap) grid = cap;
-  k<<<(unsigned)(grid < 1 ? 1 : grid), NTF, 0, s>>>(dt, ntiles, rule & 1, status);
+  k<<<(unsigned)(grid < 1 ? 1 : grid), NTF, 0, s>>>(dt, ntiles, rows, -0.0f, status);
   return cudaGetLastError();
+}
+
+template <int T>
+static cudaError_t launch_rule(const DemTable& dt, int64_t ntiles, int rule, uint32_t* status, cudaStream_t s) {
+  switch (rule) {
+    case 0: return launch_t<T, false, false>(dt, ntiles, status, s);
+    case 1: return launch_t<T, true, false>(dt, ntiles, status, s);
+    case 2: return launch_t<T, false, true>(dt, ntiles, status, s);
+    case 3: return launch_t<T, true, true>(dt, ntiles, status, s);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace fdir
@@ -249,9 +419,9 @@ cudaError_t launch_flowdir(const DemTable& dt, int64_t ntiles, int T, int rule, 
                            int* nlaunch) {
   ++*nlaunch;
   switch (T) {
-    case 32: return fdir::launch_t<32>(dt, ntiles, rule, status, s);
-    case 64: return fdir::launch_t<64>(dt, ntiles, rule, status, s);
-    case 128: return fdir::launch_t<128>(dt, ntiles, rule, status, s);
+    case 32: return fdir::launch_rule<32>(dt, ntiles, rule, status, s);
+    case 64: return fdir::launch_rule<64>(dt, ntiles, rule, status, s);
+    case 128: return fdir::launch_rule<128>(dt, ntiles, rule, status, s);
   }
   return cudaErrorInvalidValue;
 }
