@@ -128,7 +128,9 @@ struct HPlan {
 int hier_levels(int T, int64_t max_side, int* S, int* G, int max_levels);
 cudaError_t launch_combine_hier(const HPlan& hp, cudaStream_t s, int* nlaunch);
 
-// tile passes, unit counts or weighted (d8_unit.cu)
+// tile pass of unit counts, ring walks (d8_count.cu)
+cudaError_t launch_up_count(const DemTable& dt, const Pipe& p, cudaStream_t s);
+// tile passes: unit counts with the lane-mask walk, weighted; finalise (d8_unit.cu)
 cudaError_t launch_up_unit(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s);
 cudaError_t launch_down_unit(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s);
 

@@ -1,12 +1,18 @@
-// d8_unit.cu -- the unit-count tile passes (the headline path).
+// d8_unit.cu -- tile passes: weighted areas, unit counts of 128 x 128 tiles and
+// under the lane-mask strategy (other unit counts: d8_count.cu), and the
+// finalising passes.
 //
 //  k_up_unit    per tile: codes from the direction field, the in-tile
 //               dependency count (Algorithm 1), the in-tile up-slope counts
-//               with inflow from other tiles unknown = 0 (Algorithms 2-4),
-//               written to A, and the perimeter summary.
-//  k_fin_unit   per tile finalise (Algorithms 7-8): A already holds the
-//               in-tile counts; the resolved inflow from neighbouring tiles
-//               is pushed down the in-tile paths it reaches and added there.
+//               or weighted areas with inflow from other tiles unknown = 0
+//               (Algorithms 2-4), written to A, and the perimeter summary.
+//               (A 128 x 128 tile's count and cell index do not fit one word
+//               of d8_count.cu.)
+//  k_up_lm      the same for unit counts with the lane-mask walk.
+//  k_fin_unit,  per tile finalise (Algorithms 7-8): A already holds the
+//  k_fin_w      in-tile counts or areas; the resolved inflow from neighbouring
+//               tiles is pushed down the in-tile paths it reaches and added
+//               there.
 //
 // Layout choices for GB300:
 //  * one packed 32-bit word per cell in shared memory holds the cell's
@@ -15,16 +21,13 @@
 //    to its down-slope cell and tells the sender whether it was the last
 //    input; only then does the sender continue (Algorithm 2's tail
 //    recursion).  The in-tile count of a 128 x 128 tile fits in 16 bits;
-//  * the walks are latency-bound, so shared memory per tile is kept small
-//    (the word array, a uint16 segment record per cell and a 64-entry ring
-//    of pending sources per warp: 24.6 KB for 64 x 64) to fit eight tiles per
-//    SM, and the launch bounds hold registers to the same eight;
-//  * each warp feeds idle lanes from its ring with ballots (no shared
-//    atomics), refilling the ring by scanning its own cells as it goes;
-//  * every walk records its segment (the cells it finished) and where the
-//    segment ended (at a tile exit or path end, or at the junction where
-//    another walk took over), so the exit of any perimeter cell's in-tile
-//    path is a short chase over segment records instead of a walk over cells;
+//  * each warp feeds idle lanes from a ring of pending starts with ballots (no
+//    shared atomics), refilling the ring by scanning its own cells as it goes;
+//  * unit counts: every walk records its segment (the cells it finished) and
+//    where the segment ended (at a tile exit or path end, or at the junction
+//    where another walk took over), so the exit of any perimeter cell's
+//    in-tile path is a short chase over segment records instead of a walk over
+//    cells;
 //  * the first pass writes the in-tile counts to A, so the finalising pass
 //    only walks the paths down-slope of the perimeter cells that receive
 //    inflow from other tiles, adding that inflow along them, instead of
@@ -1069,7 +1072,11 @@ static unsigned persistent_grid_u(K kernel, int threads, size_t smem, int64_t nt
 template <int T, bool WT>
 static cudaError_t launch_up_unit_t(const DemTable& dt, const Pipe& p, cudaStream_t s) {
   const size_t bytes = UpLayout<T, WT>::bytes;
-  auto k = (!WT && p.strat == STRAT_LANE_MASK) ? k_up_lm<T> : k_up_unit<T, WT>;
+  void (*k)(DemTable, Pipe);
+  if constexpr (WT || T == 128)
+    k = (!WT && p.strat == STRAT_LANE_MASK) ? k_up_lm<T> : k_up_unit<T, WT>;
+  else
+    k = k_up_lm<T>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   k<<<persistent_grid_u(k, UpThreads<T, WT>::N, bytes, p.ntiles), UpThreads<T, WT>::N, bytes, s>>>(dt, p);
@@ -1089,6 +1096,9 @@ static cudaError_t launch_down_unit_t(const DemTable& dt, const Pipe& p, cudaStr
 }  // namespace unit
 
 cudaError_t launch_up_unit(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s) {
+  // d8_count.cu's words hold tiles up to 64 a side (8192 x 8192 fractal, T =
+  // 64: 262 us there, 435 in k_up_unit)
+  if (!weighted && p.strat != STRAT_LANE_MASK && p.T <= 64) return launch_up_count(dt, p, s);
   switch (p.T) {
     case 32: return weighted ? unit::launch_up_unit_t<32, true>(dt, p, s) : unit::launch_up_unit_t<32, false>(dt, p, s);
     case 64: return weighted ? unit::launch_up_unit_t<64, true>(dt, p, s) : unit::launch_up_unit_t<64, false>(dt, p, s);
