@@ -77,6 +77,7 @@ struct d8_batch {
   // layered combine: per level l >= 1, a table of per-DEM unit grids and a
   // unit -> DEM map (level 0 uses the tile table above)
   int nlev = 0;
+  bool solve = false;
   bool need_top = false;
   int lev_S[HMAX + 1] = {};
   int64_t lev_units[HMAX + 1] = {};
@@ -170,6 +171,7 @@ Pipe carve_pipe(void* base, int64_t ntiles, int T, size_t vbytes, uint32_t* stat
 
 // ---- layered combine plan (single DEM or batch) ---------------------------
 struct HShape {
+  bool solve = false;  // no levels: one launch over the tiles (HPlan::solve)
   int nlev = 0;
   int S[HMAX + 1] = {};
   int64_t nunits[HMAX + 1] = {};
@@ -177,13 +179,18 @@ struct HShape {
 };
 
 // Levels above tiles of side T for the given DEM shapes.
-HShape hier_shape(int T, int n, const int64_t* H, const int64_t* W) {
+// Unit counts of grids up to solve_side take the single-launch combine: at 512
+// x 512 24 us against 59 for the four group launches and 10 more between them.
+// Not under strategy "jump", whose point is fields with long chains: they would
+// run in one block.
+HShape hier_shape(int T, int n, const int64_t* H, const int64_t* W, bool weighted, int strat) {
   HShape hs;
   int64_t mx = 1;
   for (int k = 0; k < n; k++) mx = H[k] > mx ? H[k] : (W[k] > mx ? W[k] : mx);
   for (int k = 0; k < n; k++) mx = W[k] > mx ? W[k] : mx;
   int S[HMAX], G[HMAX];
-  hs.nlev = hier_levels(T, mx, S, G, HMAX - 1);
+  hs.solve = !weighted && strat != STRAT_JUMP && mx > T && mx <= solve_side(T);
+  hs.nlev = hs.solve ? 0 : hier_levels(T, mx, S, G, HMAX - 1);
   hs.S[0] = T;
   for (int l = 1; l <= hs.nlev; l++) hs.S[l] = S[l - 1] * G[l - 1];
   for (int l = 0; l <= hs.nlev; l++) {
@@ -191,7 +198,7 @@ HShape hier_shape(int T, int n, const int64_t* H, const int64_t* W) {
     for (int k = 0; k < n; k++) {
       const int64_t nu = ((H[k] + hs.S[l] - 1) / hs.S[l]) * ((W[k] + hs.S[l] - 1) / hs.S[l]);
       u += nu;
-      if (l == hs.nlev && nu > 1) hs.need_top = true;
+      if (l == hs.nlev && nu > 1 && !hs.solve) hs.need_top = true;
     }
     hs.nunits[l] = u;
   }
@@ -217,6 +224,7 @@ size_t hier_bytes(const HShape& hs, size_t vb) {
 HPlan carve_hier(void* base, const HShape& hs, const Pipe& p, const DemTable* dts, bool weighted) {
   HPlan hp{};
   hp.weighted = weighted;
+  hp.solve = hs.solve;
   hp.top.jump = p.strat == STRAT_JUMP;
   hp.nlev = hs.nlev;
   hp.need_top = hs.need_top;
@@ -309,7 +317,7 @@ d8_status run_forward(d8_ctx* c, const DemDesc& d0, int mode, int rule, cudaStre
   const bool weighted = (mode == UP_WEIGHTED);
   const size_t vb = weighted ? 8 : 4;
   if (up_smem_bytes(T, mode) == 0 || down_smem_bytes(T, weighted) == 0) return D8_ERR_ARG;
-  const HShape hs = hier_shape(T, 1, &d.H, &d.W);
+  const HShape hs = hier_shape(T, 1, &d.H, &d.W, weighted, c->strat);
   const size_t hb = hier_bytes(hs, vb);
   const size_t pb = align256(pipe_bytes(ntiles, T, vb));
   d8_status st = ensure_ws(c, pb + hb);
@@ -344,7 +352,7 @@ d8_status run_forward(d8_ctx* c, const DemDesc& d0, int mode, int rule, cudaStre
       dts[l] = single(dl);
     }
     const HPlan hp = carve_hier(static_cast<char*>(c->ws) + pb, hs, p, dts, weighted);
-    c->last_levels = hs.nlev;
+    c->last_levels = hs.solve ? 1 : hs.nlev;
     c->last_top_units = hs.need_top ? hs.nunits[hs.nlev] : 0;
     c->last_jump = hp.top.jump;
     c->last_counters = hs.need_top ? hp.top.counters : nullptr;
@@ -352,6 +360,8 @@ d8_status run_forward(d8_ctx* c, const DemDesc& d0, int mode, int rule, cudaStre
     e = launch_combine_hier(hp, s, &sc.n);
   }
   if (e != cudaSuccess) return cuda_fail(e);
+  p.recv = !weighted;
+  if (p.recv && hs.nlev == 0 && !hs.solve) p.S = nullptr;
   {
     StageScope sc(c, ST_DOWN, s);
     e = launch_down(dt, p, weighted, s, &sc.n);
@@ -703,8 +713,9 @@ d8_status d8_batch_plan(d8_ctx* c, int n, const int64_t* H, const int64_t* W, d8
     for (int64_t t = 0; t < d.ntx * d.nty; t++) tile_dem[(size_t)(d.tile_base + t)] = k;
   }
   std::vector<int64_t> Hv(H, H + n), Wv(W, W + n);
-  const HShape hs = hier_shape(b->T, n, Hv.data(), Wv.data());
+  const HShape hs = hier_shape(b->T, n, Hv.data(), Wv.data(), false, b->strat);
   b->nlev = hs.nlev;
+  b->solve = hs.solve;
   b->need_top = hs.need_top;
   for (int l = 0; l <= hs.nlev; l++) {
     b->lev_S[l] = hs.S[l];
@@ -759,6 +770,7 @@ static cudaError_t batch_enqueue(d8_batch* b, int rule, cudaStream_t s, int* n_u
   p.strat = b->strat;
   HShape hs;
   hs.nlev = b->nlev;
+  hs.solve = b->solve;
   hs.need_top = b->need_top;
   DemTable dts[HMAX + 1];
   dts[0] = dt;
@@ -778,6 +790,8 @@ static cudaError_t batch_enqueue(d8_batch* b, int rule, cudaStream_t s, int* n_u
   cudaError_t e = cudaMemsetAsync(p.queue, 0, sizeof(uint32_t) * 16, s);
   if (e == cudaSuccess) e = launch_up(dt, p, UP_UNIT_Z, rule, s, n_up);
   if (e == cudaSuccess) e = launch_combine_hier(hp, s, n_comb);
+  p.recv = true;
+  if (b->nlev == 0 && !b->solve) p.S = nullptr;
   if (e == cudaSuccess) e = launch_down(dt, p, false, s, n_down);
   return e;
 }

@@ -14,12 +14,13 @@
 // atomics, a short walk because few units remain.  k_group_down then runs
 // each level back down: the resolved inflow across a group's border seeds
 // its child exits and the same walks give every child exit its final area;
-// at level 0 that is the final area of every tile exit, which the tiles'
-// finalising pass reads.
+// at level 0 the final areas of the tile exits give the tiles' receivers their
+// inflow, which the finalising pass reads.
 //
 // Unit counts travel as uint32, weighted areas as float-float values (fp32
 // arithmetic throughout, with compensated atomic adds).
 #include <cstring>
+#include <type_traits>
 
 #include "d8_device.cuh"
 
@@ -91,13 +92,55 @@ __device__ __forceinline__ UnitGeo unit_geo(const DemDesc& d, int64_t uy, int64_
 __device__ __forceinline__ uint32_t pd_par(uint32_t w) { return w >> 16; }
 __device__ __forceinline__ uint32_t pd_deg(uint32_t w) { return w & 0xFFFFu; }
 
-template <int S, int G, class V, class CV>
-__device__ int group_load(const DemDesc& cd, int64_t gy, int64_t gx, const uint16_t* cpex, const CV* cpval,
-                          uint16_t* spx, V* val, uint32_t* pd) {
+// A group's extent in cells (ragged at the right and bottom), and that of its
+// child (a, b): everything inside a group is 32-bit arithmetic.
+struct GroupGeo {
+  int h, w;
+};
+template <int S, int G>
+__device__ __forceinline__ GroupGeo group_geo(const DemDesc& d, int64_t gy, int64_t gx) {
+  return GroupGeo{(int)min64(G * S, d.H - gy * (G * S)), (int)min64(G * S, d.W - gx * (G * S))};
+}
+template <int S>
+__device__ __forceinline__ int child_h(const GroupGeo& g, int a) { return min(S, g.h - a * S); }
+template <int S>
+__device__ __forceinline__ int child_w(const GroupGeo& g, int b) { return min(S, g.w - b * S); }
+
+// node of the group's cell (i, j), which lies on its child's perimeter
+template <int S, int G>
+__device__ __forceinline__ int node_of(const GroupGeo& g, int i, int j) {
+  const int a = i / S, b = j / S;
+  return (a * G + b) * (4 * S) + slot_of(i - a * S, j - b * S, child_h<S>(g, a), child_w<S>(g, b), S);
+}
+
+// the cell of node n, relative to the group
+template <int S, int G>
+__device__ __forceinline__ void cell_of(const GroupGeo& g, int n, int& i, int& j) {
+  const int lt = n / (4 * S), a = lt / G, b = lt % G;
+  slot_cell(n - lt * (4 * S), child_h<S>(g, a), child_w<S>(g, b), S, i, j);
+  i += a * S;
+  j += b * S;
+}
+
+// The node that child exit n (exit code pe) drains into, or -1 if its cell
+// lies in another group.
+template <int S, int G>
+__device__ __forceinline__ int target_node(const GroupGeo& g, int n, uint16_t pe) {
+  int i, j;
+  cell_of<S, G>(g, n, i, j);
+  i += code_di(pe & 7);
+  j += code_dj(pe & 7);
+  if ((unsigned)i >= (unsigned)(G * S) || (unsigned)j >= (unsigned)(G * S)) return -1;
+  return node_of<S, G>(g, i, j);
+}
+
+template <int S, int G, int NT, class V, class CV>
+__device__ int group_load(const DemDesc& cd, const GroupGeo& gg, int64_t gy, int64_t gx, const uint16_t* cpex,
+                          const CV* cpval, uint16_t* spx, V* val, uint32_t* pd) {
   constexpr int NS = G * G * 4 * S;
   constexpr int SPT = 4 * S;  // slots per child, a multiple of 8
-  constexpr int NQ = NS / 8 / NTG > 0 ? NS / 8 / NTG : 1;
-  static_assert(SPT % 8 == 0 && NS % (8 * NTG) == 0, "eight slots per load, whole rounds per thread");
+  constexpr int NQ = NS / 8 / NT > 0 ? NS / 8 / NT : 1;
+  static_assert(SPT % 8 == 0 && NS % (8 * NT) == 0, "eight slots per load, whole rounds per thread");
   int exits = 0;
   // eight consecutive slots of one child per 16-byte load of codes, with
   // their values loaded unconditionally beside them: every load of this
@@ -106,7 +149,7 @@ __device__ int group_load(const DemDesc& cd, int64_t gy, int64_t gx, const uint1
   CV v8[NQ][8];
 #pragma unroll
   for (int r = 0; r < NQ; r++) {
-    const int n = (threadIdx.x + r * NTG) * 8;
+    const int n = (threadIdx.x + r * NT) * 8;
     const int lt = n / SPT, s = n - lt * SPT;
     const int64_t cy = gy * G + lt / G, cx = gx * G + lt % G;
     pe8[r] = make_uint4(PEX_TERM | (PEX_TERM << 16), PEX_TERM | (PEX_TERM << 16), PEX_TERM | (PEX_TERM << 16),
@@ -123,7 +166,7 @@ __device__ int group_load(const DemDesc& cd, int64_t gy, int64_t gx, const uint1
   }
 #pragma unroll
   for (int r = 0; r < NQ; r++) {
-    const int n = (threadIdx.x + r * NTG) * 8;
+    const int n = (threadIdx.x + r * NT) * 8;
     const uint16_t* pe = reinterpret_cast<const uint16_t*>(&pe8[r]);
     V vo[8];
 #pragma unroll
@@ -139,30 +182,19 @@ __device__ int group_load(const DemDesc& cd, int64_t gy, int64_t gx, const uint1
     *reinterpret_cast<uint4*>(pd + n + 4) = make_uint4(0, 0, 0, 0);
   }
   __syncthreads();
-  for (int n = threadIdx.x; n < NS; n += NTG) {
+  for (int n = threadIdx.x; n < NS; n += NT) {
     const uint16_t pe = spx[n];
     uint16_t pr = N_NONE;
     if (pe & PEX_EXIT) {
-      const int lt = n / (4 * S), s = n - lt * (4 * S);
-      const int64_t cy = gy * G + lt / G, cx = gx * G + lt % G;
-      const UnitGeo u = unit_geo(cd, cy, cx, S);
-      int i, j;
-      slot_cell(s, u.h, u.w, S, i, j);
-      const int k = pe & 7;
-      const int64_t ti = u.i0 + i + code_di(k), tj = u.j0 + j + code_dj(k);
-      const int64_t ty = ti / S, tx = tj / S;
-      const int64_t a = ty - gy * G, b = tx - gx * G;
-      if (a >= 0 && b >= 0 && a < G && b < G) {
-        const UnitGeo tu = unit_geo(cd, ty, tx, S);
-        const int lt2 = (int)(a * G + b);
-        const int n2 = lt2 * (4 * S) + slot_of((int)(ti - tu.i0), (int)(tj - tu.j0), tu.h, tu.w, S);
+      const int n2 = target_node<S, G>(gg, n, pe);
+      if (n2 >= 0) {
         const uint16_t pe2 = spx[n2];
         if (pe2 & PEX_EXIT)
           pr = (uint16_t)n2;
         else if (pe2 == PEX_TERM)
           pr = N_ROOT;
         else
-          pr = (uint16_t)(lt2 * (4 * S) + pe2);
+          pr = (uint16_t)(n2 / (4 * S) * (4 * S) + pe2);
         if (pr < N_NONE) atomicAdd(&pd[pr], 1u);
       } else {
         pr = N_OUT;
@@ -179,15 +211,15 @@ __device__ int group_load(const DemDesc& cd, int64_t gy, int64_t gx, const uint1
 // parent, then (after a block fence) decrements the parent's children count;
 // the last child continues at the parent (its acquire-release count atomic
 // orders it after every child's addition).  Returns the number of nodes this thread finished.
-template <int S, int G, class V>
+template <int S, int G, int NT, class V>
 __device__ int group_walk(uint16_t* spx, V* val, uint32_t* pd, uint16_t* srcl) {
   constexpr int NS = G * G * 4 * S;
-  constexpr int NW = NTG / 32;
+  constexpr int NW = NT / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint16_t* my = srcl + warp * (NS / NW);
   int n = 0;
-  for (int r = 0; r < NS / NTG; r++) {
-    const int c = threadIdx.x + r * NTG;
+  for (int r = 0; r < NS / NT; r++) {
+    const int c = threadIdx.x + r * NT;
     const bool s = (spx[c] & PEX_EXIT) && pd_deg(pd[c]) == 0u;
     const unsigned m = __ballot_sync(FULL, s);
     if (s) my[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)c;
@@ -256,24 +288,21 @@ __global__ void __launch_bounds__(NTG) k_group_up(DemTable cdt, DemTable gdt, co
       misc[0] = 0;
       misc[1] = 0;
     }
-    const int exits = group_load<S, G, V, CV>(cd, gy, gx, cpex, cpval, spx, val, pd);
-    const int done = group_walk<S, G, V>(spx, val, pd, srcl);
+    const GroupGeo gg = group_geo<S, G>(gd, gy, gx);
+    const int exits = group_load<S, G, NTG, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
+    const int done = group_walk<S, G, NTG, V>(spx, val, pd, srcl);
     atomicAdd(&misc[0], done);
     atomicAdd(&misc[1], exits);
     __syncthreads();
     // every exit node must have been finished, else the exit graph has a cycle
     if (threadIdx.x == 0 && misc[0] != misc[1]) set_status(status, D8_ERR_CYCLE);
     // the group's own perimeter summary
-    const UnitGeo gg = unit_geo(gd, gy, gx, GS);
     for (int gs = threadIdx.x; gs < 4 * GS; gs += NTG) {
       int ci, cj;
       uint16_t gpe = PEX_TERM;
       V gv{};
       if (slot_cell(gs, gg.h, gg.w, GS, ci, cj)) {
-        const int a = ci / S, b = cj / S;
-        const UnitGeo cu = unit_geo(cd, gy * G + a, gx * G + b, S);
-        const int lt = a * G + b;
-        const int n0 = lt * (4 * S) + slot_of(ci - a * S, cj - b * S, cu.h, cu.w, S);
+        const int n0 = node_of<S, G>(gg, ci, cj);
         const uint16_t pe = spx[n0];
         int x = -1;
         if (pe & PEX_EXIT) {
@@ -284,16 +313,14 @@ __global__ void __launch_bounds__(NTG) k_group_up(DemTable cdt, DemTable gdt, co
             x = n0;
           }
         } else if (pe != PEX_TERM) {
-          x = lt * (4 * S) + pe;
+          x = n0 / (4 * S) * (4 * S) + pe;
         }
         if (x >= 0) {
           for (int it = 0; it < NS && pd_par(pd[x]) < N_NONE; it++) x = (int)pd_par(pd[x]);
           if (pd_par(pd[x]) == N_OUT) {
-            const int xlt = x / (4 * S), xs = x - xlt * (4 * S);
-            const UnitGeo xu = unit_geo(cd, gy * G + xlt / G, gx * G + xlt % G, S);
             int xi, xj;
-            slot_cell(xs, xu.h, xu.w, S, xi, xj);
-            gpe = (uint16_t)slot_of((xlt / G) * S + xi, (xlt % G) * S + xj, gg.h, gg.w, GS);
+            cell_of<S, G>(gg, x, xi, xj);
+            gpe = (uint16_t)slot_of(xi, xj, gg.h, gg.w, GS);
           }
         }
       }
@@ -304,7 +331,29 @@ __global__ void __launch_bounds__(NTG) k_group_up(DemTable cdt, DemTable gdt, co
   }
 }
 
-template <int S, int G, class V, class CV>
+// infl[n] = the sum of the final areas of the group's child exits that drain
+// into node n's cell
+template <int S, int G, int NT>
+__device__ __forceinline__ void receivers_inflow(const GroupGeo& g, const uint16_t* spx, const uint32_t* val,
+                                                 uint32_t* infl) {
+  constexpr int NS = G * G * 4 * S;
+  for (int n = threadIdx.x; n < NS; n += NT) infl[n] = 0u;
+  __syncthreads();
+  for (int n = threadIdx.x; n < NS; n += NT) {
+    const uint16_t pe = spx[n];
+    if (!(pe & PEX_EXIT)) continue;
+    const int n2 = target_node<S, G>(g, n, pe);
+    if (n2 >= 0) atomicAdd(&infl[n2], val[n]);
+  }
+}
+
+// The group's border inflow and its children's final values.  RECV (unit
+// counts, the children are tiles): cfin gets per slot not the exits' final
+// areas but the receivers' inflow, the sum of the final areas of the exits of
+// other tiles that drain into the slot's cell, which is what the finalising
+// pass needs (it then reads one contiguous row per tile; gathering the areas
+// there took the codes around every tile and scattered loads).
+template <int S, int G, class V, class CV, bool RECV>
 __global__ void __launch_bounds__(NTG) k_group_down(DemTable cdt, DemTable gdt, const uint16_t* cpex, const CV* cpval,
                                                       V* cfin, const V* gfin, int64_t ngroups, uint32_t* queue) {
   using L = GroupLayout<S, G, V>;
@@ -322,15 +371,22 @@ __global__ void __launch_bounds__(NTG) k_group_down(DemTable cdt, DemTable gdt, 
     const DemDesc cd = dem_by_index(cdt, dem);
     const int64_t lg = gu - gd.tile_base;
     const int64_t gy = lg / gd.ntx, gx = lg % gd.ntx;
-    group_load<S, G, V, CV>(cd, gy, gx, cpex, cpval, spx, val, pd);
+    const GroupGeo gg = group_geo<S, G>(gd, gy, gx);
+    group_load<S, G, NTG, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
     // inflow across the group border: each border cell r receives the final
     // areas of the outside cells draining into it; the inflow then follows
     // r's path inside its child unit to that child's exit
-    const UnitGeo gg = unit_geo(gd, gy, gx, GS);
-    for (int gs = threadIdx.x; gs < 4 * GS; gs += NTG) {
+    constexpr int NB = 4 * GS / NTG;  // border slots per thread
+    static_assert(4 * GS % NTG == 0, "whole rounds over the border");
+    V bin[RECV ? NB : 1];  // inflow across the border and the child slot it enters
+    int bslot[RECV ? NB : 1];
+#pragma unroll 1
+    for (int r = 0; r < NB; r++) {
+      const int gs = threadIdx.x + r * NTG;
+      if (RECV) bslot[RECV ? r : 0] = -1;
       int ci, cj;
       if (!slot_cell(gs, gg.h, gg.w, GS, ci, cj)) continue;
-      const int64_t gi = gg.i0 + ci, gj = gg.j0 + cj;
+      const int64_t gi = gy * GS + ci, gj = gx * GS + cj;
       V in{};
       bool any = false;
 #pragma unroll
@@ -344,26 +400,82 @@ __global__ void __launch_bounds__(NTG) k_group_down(DemTable cdt, DemTable gdt, 
         any = true;
       }
       if (!any) continue;
-      const int a = ci / S, b = cj / S;
-      const UnitGeo cu = unit_geo(cd, gy * G + a, gx * G + b, S);
-      const int lt = a * G + b;
-      const int n0 = lt * (4 * S) + slot_of(ci - a * S, cj - b * S, cu.h, cu.w, S);
+      const int n0 = node_of<S, G>(gg, ci, cj);
       const uint16_t pe = spx[n0];
       if (pe & PEX_EXIT)
         vatomic_add(&val[n0], in);
       else if (pe != PEX_TERM)
-        vatomic_add(&val[lt * (4 * S) + pe], in);
+        vatomic_add(&val[n0 / (4 * S) * (4 * S) + pe], in);
+      if (RECV) {
+        bin[RECV ? r : 0] = in;
+        bslot[RECV ? r : 0] = n0;
+      }
     }
     __syncthreads();
-    group_walk<S, G, V>(spx, val, pd, srcl);
+    group_walk<S, G, NTG, V>(spx, val, pd, srcl);
     __syncthreads();
+    if constexpr (RECV) {
+      uint32_t* infl = pd;  // the walk is done with it
+      receivers_inflow<S, G, NTG>(gg, spx, val, infl);
+#pragma unroll 1
+      for (int r = 0; r < NB; r++)
+        if (bslot[r] >= 0) atomicAdd(&infl[bslot[r]], bin[r]);
+      __syncthreads();
+    }
     for (int n = threadIdx.x; n < NS; n += NTG) {
-      if (!(spx[n] & PEX_EXIT)) continue;
+      if (!RECV && !(spx[n] & PEX_EXIT)) continue;
       const int lt = n / (4 * S), s = n - lt * (4 * S);
       const int64_t cy = gy * G + lt / G, cx = gx * G + lt % G;
-      cfin[(cd.tile_base + cy * cd.ntx + cx) * (4 * S) + s] = val[n];
+      if (RECV && (cy >= cd.nty || cx >= cd.ntx)) continue;
+      V* dst = cfin + (cd.tile_base + cy * cd.ntx + cx) * (4 * S) + s;
+      if constexpr (RECV)
+        *dst = pd[n];
+      else
+        *dst = val[n];
     }
   }
+}
+
+// The whole combine of a grid that one group covers (unit counts): load, walk,
+// receivers' inflow, one block of NTS threads per DEM.  One launch instead of
+// two up and two down; a 512 x 512 grid's 64 tiles are one group of 8 x 8.
+constexpr int NTS = 1024;
+template <int S, int G>
+__global__ void __launch_bounds__(NTS) k_group_solve(DemTable dt, const uint16_t* pex, const uint32_t* pval,
+                                                       uint32_t* inflow, uint32_t* status) {
+  using L = GroupLayout<S, G, uint32_t>;
+  extern __shared__ __align__(16) unsigned char sm[];
+  uint16_t* spx = reinterpret_cast<uint16_t*>(sm + L::off_spx);
+  uint32_t* val = reinterpret_cast<uint32_t*>(sm + L::off_val);
+  uint32_t* pd = reinterpret_cast<uint32_t*>(sm + L::off_pd);
+  uint16_t* srcl = reinterpret_cast<uint16_t*>(sm + L::off_src);
+  int* misc = reinterpret_cast<int*>(sm + L::off_misc);
+  const DemDesc d = dem_by_index(dt, blockIdx.x);
+  const GroupGeo gg = group_geo<S, G>(d, 0, 0);
+  if (threadIdx.x < 2) misc[threadIdx.x] = 0;
+  const int exits = group_load<S, G, NTS, uint32_t, uint32_t>(d, gg, 0, 0, pex, pval, spx, val, pd);
+  const int done = group_walk<S, G, NTS, uint32_t>(spx, val, pd, srcl);
+  atomicAdd(&misc[0], done);
+  atomicAdd(&misc[1], exits);
+  __syncthreads();
+  if (threadIdx.x == 0 && misc[0] != misc[1]) set_status(status, D8_ERR_CYCLE);
+  receivers_inflow<S, G, NTS>(gg, spx, val, pd);
+  __syncthreads();
+  for (int n = threadIdx.x; n < L::NS; n += NTS) {
+    const int lt = n / (4 * S), cy = lt / G, cx = lt % G;
+    if (cy < d.nty && cx < d.ntx) inflow[(d.tile_base + cy * d.ntx + cx) * (4 * S) + (n - lt * (4 * S))] = pd[n];
+  }
+}
+
+template <int S, int G>
+static cudaError_t launch_solve(const HLevel& t, uint32_t* status, cudaStream_t s) {
+  constexpr size_t bytes = GroupLayout<S, G, uint32_t>::bytes;
+  auto k = k_group_solve<S, G>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  k<<<(unsigned)t.dt.ndem, NTS, bytes, s>>>(t.dt, t.pex, static_cast<const uint32_t*>(t.pval),
+                                            static_cast<uint32_t*>(t.fin), status);
+  return cudaGetLastError();
 }
 
 // ---- top level: Algorithms 5-6 over the remaining units, in global memory
@@ -631,11 +743,11 @@ static cudaError_t launch_level_up(const DemTable& cdt, const DemTable& gdt, con
   return cudaGetLastError();
 }
 
-template <int S, int G, class V, class CV>
+template <int S, int G, class V, class CV, bool RECV>
 static cudaError_t launch_level_down(const DemTable& cdt, const DemTable& gdt, const uint16_t* cpex, const void* cpval,
                                      void* cfin, const void* gfin, int64_t ngroups, uint32_t* queue, cudaStream_t s) {
   using L = GroupLayout<S, G, V>;
-  auto k = k_group_down<S, G, V, CV>;
+  auto k = k_group_down<S, G, V, CV, RECV>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
   if (e != cudaSuccess) return e;
   int per_sm = 1, dev = 0, sms = 1;
@@ -745,7 +857,7 @@ static cudaError_t combine_hier_t(const HPlan& hp, cudaStream_t s, int* nlaunch)
     ++*nlaunch;                                                                                                  \
     continue;                                                                                                    \
   }
-    D8_UP(32, 4) D8_UP(64, 4) D8_UP(128, 2) D8_UP(256, 2) D8_UP(512, 2)
+    D8_UP(32, 4) D8_UP(64, 4) D8_UP(128, 2) D8_UP(256, 2)
 #undef D8_UP
     return cudaErrorInvalidValue;
   }
@@ -759,27 +871,28 @@ static cudaError_t combine_hier_t(const HPlan& hp, cudaStream_t s, int* nlaunch)
     e = l0 ? launch_top<SS, V, CV0>(t.dt, t, hp.top, s, nlaunch) : launch_top<SS, V, V>(t.dt, t, hp.top, s, nlaunch); \
     break;
     switch (t.S) {
-      D8_TOP(32) D8_TOP(64) D8_TOP(128) D8_TOP(256) D8_TOP(512) D8_TOP(1024)
+      D8_TOP(32) D8_TOP(64) D8_TOP(128) D8_TOP(256) D8_TOP(512)
       default: return cudaErrorInvalidValue;
     }
 #undef D8_TOP
     if (e != cudaSuccess) return e;
   }
-  // down: level l -> l-1
+  // down: level l -> l-1 (at the tiles: unit counts leave the receivers' inflow)
+  constexpr bool RECV = std::is_same<V, uint32_t>::value;
   for (int l = hp.nlev; l >= 1 && e == cudaSuccess; l--) {
     const HLevel& c = hp.lev[l - 1];
     const HLevel& g = hp.lev[l];
     const int S = c.S, G = g.S / c.S;
 #define D8_DN(SS, GG)                                                                                               \
   if (S == SS && G == GG) {                                                                                        \
-    e = l == 1 ? launch_level_down<SS, GG, V, CV0>(c.dt, g.dt, c.pex, c.pval, c.fin, g.fin, g.nunits,               \
-                                                   hp.queue + 16 + l, s)                                           \
-               : launch_level_down<SS, GG, V, V>(c.dt, g.dt, c.pex, c.pval, c.fin, g.fin, g.nunits, hp.queue + 16 + l, \
-                                                 s);                                                               \
+    e = l == 1 ? launch_level_down<SS, GG, V, CV0, RECV>(c.dt, g.dt, c.pex, c.pval, c.fin, g.fin, g.nunits,         \
+                                                         hp.queue + 16 + l, s)                                     \
+               : launch_level_down<SS, GG, V, V, false>(c.dt, g.dt, c.pex, c.pval, c.fin, g.fin, g.nunits,          \
+                                                        hp.queue + 16 + l, s);                                     \
     ++*nlaunch;                                                                                                    \
     continue;                                                                                                      \
   }
-    D8_DN(32, 4) D8_DN(64, 4) D8_DN(128, 2) D8_DN(256, 2) D8_DN(512, 2)
+    D8_DN(32, 4) D8_DN(64, 4) D8_DN(128, 2) D8_DN(256, 2)
 #undef D8_DN
     return cudaErrorInvalidValue;
   }
@@ -788,7 +901,18 @@ static cudaError_t combine_hier_t(const HPlan& hp, cudaStream_t s, int* nlaunch)
 
 }  // namespace cmb
 
+int solve_side(int T) { return T == 128 ? 512 : 8 * T; }
+
 cudaError_t launch_combine_hier(const HPlan& hp, cudaStream_t s, int* nlaunch) {
+  if (hp.solve) {
+    ++*nlaunch;
+    switch (hp.lev[0].S) {
+      case 32: return cmb::launch_solve<32, 8>(hp.lev[0], hp.status, s);
+      case 64: return cmb::launch_solve<64, 8>(hp.lev[0], hp.status, s);
+      case 128: return cmb::launch_solve<128, 4>(hp.lev[0], hp.status, s);
+    }
+    return cudaErrorInvalidValue;
+  }
   if (!hp.weighted) return cmb::combine_hier_t<uint32_t, uint32_t>(hp, s, nlaunch);
   return cmb::combine_hier_t<ff, ff>(hp, s, nlaunch);
 }

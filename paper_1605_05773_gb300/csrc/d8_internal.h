@@ -60,7 +60,8 @@ struct Pipe {
   uint16_t* pex;     // per slot: exit code of the in-tile path
   void* pval;        // per slot: in-tile area at exits (fwd) / path sum (bwd)
   uint32_t* P[2];    // flat combines (adjoint, allocation-free entry): pointer-jumping parents
-  void* S;           // per slot: final value at exits, read by the finalising pass
+  void* S;           // per slot, read by the finalising pass: final value at exits, or (recv) the receivers' inflow
+  bool recv;         // unit counts after the layered combine; S null: no inflow between tiles
   void* S2;          // flat combines: second value buffer (adjoint) / delta buffer (counts)
   uint32_t* flags;   // combine: per-round "still active" flags, MAX_ROUNDS+2
   uint32_t* status;  // device status word (OR of 1 << d8_status)
@@ -117,6 +118,7 @@ struct HTop {  // the top level's solve in global memory (queue method or pointe
 };
 struct HPlan {
   bool weighted;  // float-float values instead of uint32 counts
+  bool solve;     // one group covers every grid: no levels, one launch
   int nlev;  // group levels 1..nlev above the tiles
   HLevel lev[HMAX];
   bool need_top;
@@ -126,11 +128,17 @@ struct HPlan {
 };
 // group sides of the levels above tiles of side T, for grids up to max_side
 int hier_levels(int T, int64_t max_side, int* S, int* G, int max_levels);
+// the largest side of a grid that one group of the single-launch combine
+// covers (unit counts)
+int solve_side(int T);
 cudaError_t launch_combine_hier(const HPlan& hp, cudaStream_t s, int* nlaunch);
 
 // tile pass of unit counts, ring walks (d8_count.cu)
 cudaError_t launch_up_count(const DemTable& dt, const Pipe& p, cudaStream_t s);
-// tile passes: unit counts with the lane-mask walk, weighted; finalise (d8_unit.cu)
+// finalise of unit counts from the receivers' inflow (d8_final.cu)
+cudaError_t launch_down_count(const DemTable& dt, const Pipe& p, cudaStream_t s);
+// tile passes: unit counts of 128 x 128 tiles or with the lane-mask walk,
+// weighted; finalise, weighted or of unit counts from the exits' values (d8_unit.cu)
 cudaError_t launch_up_unit(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s);
 cudaError_t launch_down_unit(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s);
 

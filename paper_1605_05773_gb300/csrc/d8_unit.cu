@@ -9,8 +9,8 @@
 //               (A 128 x 128 tile's count and cell index do not fit one word
 //               of d8_count.cu.)
 //  k_up_lm      the same for unit counts with the lane-mask walk.
-//  k_fin_unit,  per tile finalise (Algorithms 7-8): A already holds the
-//  k_fin_w      in-tile counts or areas; the resolved inflow from neighbouring
+//  k_fin_unit,  per tile finalise (Algorithms 7-8) from the exits' final
+//  k_fin_w      values: A already holds the in-tile counts or areas; the resolved inflow from neighbouring
 //               tiles is pushed down the in-tile paths it reaches and added
 //               there.
 //
@@ -675,25 +675,14 @@ __device__ __forceinline__ uint32_t fin_ring_code(const uint8_t* ring, const Til
   return ring[2 * (T + 2) + T + li];
 }
 
-// Algorithms 7-8 restricted to where they change anything.  The final count
-// is A(c) + F(c), where A holds the in-tile counts and F(c) is the inflow
-// from other tiles routed through c.  Inflow enters a tile only at its
-// receivers (perimeter cells with an up-slope neighbour in another tile) and
-// follows the unique down-slope path from there, so F(c) is the sum of the
-// receivers' inflows over the receivers whose in-tile path passes through c.
-// Each receiver therefore walks its path once adding its inflow to every cell
-// on it: additions commute, so the walks need no ordering between them and
-// no reply from the shared atomics, and only the cells down-slope of a
-// receiver (about a sixth of a 64 x 64 tile on fractal terrain) are touched.
-// The work is the summed length of the receivers' in-tile paths (at most
-// 4T * T^2 for adversarial fields, about the sub-forest size on terrain).
-//
-// Memory: the tile's codes and the codes of the one-cell ring around it are
-// requested together (asynchronous copies into shared memory), so a tile
-// costs one round trip for them, one for the receivers' resolved inflows and
-// a read-modify-write of the 16-byte quads of A where the inflow is non-zero.  (Reading
-// the tile's whole A up front instead, into the array the walks add to, was
-// slower: the sparse read-modify-write moves fewer bytes.)
+// The finalise of unit counts when the combine leaves the exits' final values
+// (the allocation-free entry's flat combine; after the layered one d8_final.cu
+// reads the receivers' inflow): the same walks, with the receivers found and
+// their inflow gathered here.  The tile's codes and the codes of the one-cell
+// ring around it are requested together (asynchronous copies into shared
+// memory), so a tile costs one round trip for them, one for the receivers'
+// resolved inflows and a read-modify-write of the 16-byte quads of A where the
+// inflow is non-zero.
 template <int T>
 __global__ void __launch_bounds__(NTF, 8) k_fin_unit(DemTable dt, Pipe p) {
   using L = FinLayout<T>;
@@ -729,15 +718,6 @@ __global__ void __launch_bounds__(NTF, 8) k_fin_unit(DemTable dt, Pipe p) {
         if (li >= 0 && lj >= 0 && li < g.th && lj < g.tw) continue;
         if (fin_ring_code<T>(ring, g, li, lj) != (uint32_t)opposite(k)) continue;  // also rejects cells off the grid
         in += xval[global_slot(d, g.i0 + li, g.j0 + lj, T)];
-        any = true;
-      }
-      // flow entering across the grid's first or last row (a strip)
-      if (p.top_in && g.i0 + i == 0 && p.top_in[g.j0 + j]) {
-        in += p.top_in[g.j0 + j];
-        any = true;
-      }
-      if (p.bot_in && g.i0 + i == d.H - 1 && p.bot_in[g.j0 + j]) {
-        in += p.bot_in[g.j0 + j];
         any = true;
       }
       if (any) {
@@ -1086,7 +1066,11 @@ static cudaError_t launch_up_unit_t(const DemTable& dt, const Pipe& p, cudaStrea
 template <int T, bool WT>
 static cudaError_t launch_down_unit_t(const DemTable& dt, const Pipe& p, cudaStream_t s) {
   const size_t bytes = WT ? FinWLayout<T>::bytes : FinLayout<T>::bytes;
-  auto k = WT ? k_fin_w<T> : k_fin_unit<T>;
+  void (*k)(DemTable, Pipe);
+  if constexpr (WT)
+    k = k_fin_w<T>;
+  else
+    k = k_fin_unit<T>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   k<<<persistent_grid_u(k, NTF, bytes, p.ntiles), NTF, bytes, s>>>(dt, p);
@@ -1109,13 +1093,11 @@ cudaError_t launch_up_unit(const DemTable& dt, const Pipe& p, bool weighted, cud
 }
 
 cudaError_t launch_down_unit(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s) {
+  if (!weighted) return p.T == 64 ? unit::launch_down_unit_t<64, false>(dt, p, s) : cudaErrorInvalidValue;
   switch (p.T) {
-    case 32:
-      return weighted ? unit::launch_down_unit_t<32, true>(dt, p, s) : unit::launch_down_unit_t<32, false>(dt, p, s);
-    case 64:
-      return weighted ? unit::launch_down_unit_t<64, true>(dt, p, s) : unit::launch_down_unit_t<64, false>(dt, p, s);
-    case 128:
-      return weighted ? unit::launch_down_unit_t<128, true>(dt, p, s) : unit::launch_down_unit_t<128, false>(dt, p, s);
+    case 32: return unit::launch_down_unit_t<32, true>(dt, p, s);
+    case 64: return unit::launch_down_unit_t<64, true>(dt, p, s);
+    case 128: return unit::launch_down_unit_t<128, true>(dt, p, s);
   }
   return cudaErrorInvalidValue;
 }
