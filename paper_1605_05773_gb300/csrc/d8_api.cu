@@ -190,7 +190,7 @@ HShape hier_shape(int T, int n, const int64_t* H, const int64_t* W, bool weighte
   for (int k = 0; k < n; k++) mx = W[k] > mx ? W[k] : mx;
   int S[HMAX], G[HMAX];
   hs.solve = !weighted && strat != STRAT_JUMP && mx > T && mx <= solve_side(T);
-  hs.nlev = hs.solve ? 0 : hier_levels(T, mx, S, G, HMAX - 1);
+  hs.nlev = hs.solve ? 0 : hier_levels(T, mx, !weighted && strat != STRAT_JUMP, S, G, HMAX - 1);
   hs.S[0] = T;
   for (int l = 1; l <= hs.nlev; l++) hs.S[l] = S[l - 1] * G[l - 1];
   for (int l = 0; l <= hs.nlev; l++) {
@@ -219,6 +219,12 @@ size_t hier_bytes(const HShape& hs, size_t vb) {
   return b;
 }
 
+// The counters that start at zero: the tile passes' queues, which end the pipe's
+// part of the workspace, and the combine's, which begin the levels' part.
+cudaError_t zero_counters(const Pipe& p, cudaStream_t s) {
+  return cudaMemsetAsync(p.queue, 0, align256(sizeof(uint32_t) * 16) + align256(sizeof(uint32_t) * 64), s);
+}
+
 // Carve the level arrays; level 0 takes the tile pipeline's arrays.  `dts`
 // holds each level's DEM table (filled by the caller).
 HPlan carve_hier(void* base, const HShape& hs, const Pipe& p, const DemTable* dts, bool weighted) {
@@ -237,6 +243,10 @@ HPlan carve_hier(void* base, const HShape& hs, const Pipe& p, const DemTable* dt
   hp.lev[0].fin = p.S;
   const size_t vb = weighted ? 8 : 4;
   char* q = static_cast<char*>(base);
+  hp.queue = reinterpret_cast<uint32_t*>(q);
+  hp.top.counters = hp.queue + 48;
+  hp.top.status = p.status;
+  q += align256(sizeof(uint32_t) * 64);
   for (int l = 1; l <= hs.nlev; l++) {
     const size_t ns = (size_t)hs.nunits[l] * 4 * hs.S[l];
     HLevel& L = hp.lev[l];
@@ -256,16 +266,13 @@ HPlan carve_hier(void* base, const HShape& hs, const Pipe& p, const DemTable* dt
     q += align256(nt * 4);
     hp.top.par2 = reinterpret_cast<uint32_t*>(q);
     q += align256(nt * 4);
-    hp.top.deg = reinterpret_cast<uint32_t*>(q);  // 8 bytes per slot (unit counts pack value and count)
+    hp.top.node = reinterpret_cast<unsigned long long*>(q);
     q += align256(nt * 8);
     hp.top.list = reinterpret_cast<uint32_t*>(q);
     q += align256(nt * 4);
     hp.top.flags = reinterpret_cast<uint32_t*>(q);
     q += align256(sizeof(uint32_t) * (MAX_ROUNDS + 2));
   }
-  hp.queue = reinterpret_cast<uint32_t*>(q);
-  hp.top.counters = hp.queue + 48;
-  hp.top.status = p.status;
   return hp;
 }
 
@@ -327,7 +334,7 @@ d8_status run_forward(d8_ctx* c, const DemDesc& d0, int mode, int rule, cudaStre
   p.top_in = top_in;
   p.bot_in = bot_in;
   DemTable dt = single(d);
-  cudaError_t e = cudaMemsetAsync(p.queue, 0, sizeof(uint32_t) * 16, s);
+  cudaError_t e = zero_counters(p, s);
   if (e != cudaSuccess) return cuda_fail(e);
   if (mode == UP_UNIT_Z) {
     StageScope sc(c, ST_FLOWDIR, s);
@@ -787,7 +794,7 @@ static cudaError_t batch_enqueue(d8_batch* b, int rule, cudaStream_t s, int* n_u
     dts[l] = t;
   }
   const HPlan hp = carve_hier(static_cast<char*>(b->ws) + b->pipe_part, hs, p, dts, false);
-  cudaError_t e = cudaMemsetAsync(p.queue, 0, sizeof(uint32_t) * 16, s);
+  cudaError_t e = zero_counters(p, s);
   if (e == cudaSuccess) e = launch_up(dt, p, UP_UNIT_Z, rule, s, n_up);
   if (e == cudaSuccess) e = launch_combine_hier(hp, s, n_comb);
   p.recv = true;

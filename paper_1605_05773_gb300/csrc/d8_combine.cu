@@ -28,7 +28,9 @@ namespace d8 {
 
 namespace cmb {
 
-constexpr int NTG = 256;
+// threads per group: about 16 child slots each
+template <int S, int G>
+constexpr int NTG = G * G * 4 * S >= 8192 ? 1024 : 256;
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr uint16_t N_ROOT = 0xFFFFu;  // path ends inside the group
 constexpr uint16_t N_OUT = 0xFFFEu;   // parent lies outside the group (a group exit)
@@ -265,9 +267,9 @@ __device__ int group_walk(uint16_t* spx, V* val, uint32_t* pd, uint16_t* srcl) {
 }
 
 template <int S, int G, class V, class CV>
-__global__ void __launch_bounds__(NTG) k_group_up(DemTable cdt, DemTable gdt, const uint16_t* cpex, const CV* cpval,
-                                                    uint16_t* gpex, V* gpval, int64_t ngroups, uint32_t* queue,
-                                                    uint32_t* status) {
+__global__ void __launch_bounds__(NTG<S, G>) k_group_up(DemTable cdt, DemTable gdt, const uint16_t* cpex, const CV* cpval,
+                                                    uint16_t* gpex, V* gpval, unsigned long long* node,
+                                                    int64_t ngroups, uint32_t* queue, uint32_t* status) {
   using L = GroupLayout<S, G, V>;
   extern __shared__ __align__(16) unsigned char sm[];
   uint16_t* spx = reinterpret_cast<uint16_t*>(sm + L::off_spx);
@@ -275,7 +277,7 @@ __global__ void __launch_bounds__(NTG) k_group_up(DemTable cdt, DemTable gdt, co
   uint32_t* pd = reinterpret_cast<uint32_t*>(sm + L::off_pd);
   uint16_t* srcl = reinterpret_cast<uint16_t*>(sm + L::off_src);
   int* misc = reinterpret_cast<int*>(sm + L::off_misc);
-  constexpr int NS = L::NS;
+  constexpr int NS = L::NS, NT = NTG<S, G>;
   constexpr int GS = G * S;
   TileQueue tq(queue, ngroups);
   for (int64_t gu = tq.first(); gu < ngroups; gu = tq.next()) {
@@ -289,15 +291,15 @@ __global__ void __launch_bounds__(NTG) k_group_up(DemTable cdt, DemTable gdt, co
       misc[1] = 0;
     }
     const GroupGeo gg = group_geo<S, G>(gd, gy, gx);
-    const int exits = group_load<S, G, NTG, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
-    const int done = group_walk<S, G, NTG, V>(spx, val, pd, srcl);
+    const int exits = group_load<S, G, NT, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
+    const int done = group_walk<S, G, NT, V>(spx, val, pd, srcl);
     atomicAdd(&misc[0], done);
     atomicAdd(&misc[1], exits);
     __syncthreads();
     // every exit node must have been finished, else the exit graph has a cycle
     if (threadIdx.x == 0 && misc[0] != misc[1]) set_status(status, D8_ERR_CYCLE);
     // the group's own perimeter summary
-    for (int gs = threadIdx.x; gs < 4 * GS; gs += NTG) {
+    for (int gs = threadIdx.x; gs < 4 * GS; gs += NT) {
       int ci, cj;
       uint16_t gpe = PEX_TERM;
       V gv{};
@@ -326,6 +328,7 @@ __global__ void __launch_bounds__(NTG) k_group_up(DemTable cdt, DemTable gdt, co
       }
       gpex[gu * (4 * GS) + gs] = gpe;
       gpval[gu * (4 * GS) + gs] = gv;
+      if (node) node[gu * (4 * GS) + gs] = 0ull;  // below the top level: its words start at zero
     }
     // (the queue's barrier protects shared memory before the next group)
   }
@@ -354,16 +357,19 @@ __device__ __forceinline__ void receivers_inflow(const GroupGeo& g, const uint16
 // pass needs (it then reads one contiguous row per tile; gathering the areas
 // there took the codes around every tile and scattered loads).
 template <int S, int G, class V, class CV, bool RECV>
-__global__ void __launch_bounds__(NTG) k_group_down(DemTable cdt, DemTable gdt, const uint16_t* cpex, const CV* cpval,
-                                                      V* cfin, const V* gfin, int64_t ngroups, uint32_t* queue) {
+__global__ void __launch_bounds__(NTG<S, G>) k_group_down(DemTable cdt, DemTable gdt, const uint16_t* cpex, const CV* cpval,
+                                                      V* cfin, const V* gfin, int64_t ngroups, uint32_t* queue,
+                                                      const uint32_t* counters, uint32_t* status) {
   using L = GroupLayout<S, G, V>;
   extern __shared__ __align__(16) unsigned char sm[];
   uint16_t* spx = reinterpret_cast<uint16_t*>(sm + L::off_spx);
   V* val = reinterpret_cast<V*>(sm + L::off_val);
   uint32_t* pd = reinterpret_cast<uint32_t*>(sm + L::off_pd);
   uint16_t* srcl = reinterpret_cast<uint16_t*>(sm + L::off_src);
-  constexpr int NS = L::NS;
+  constexpr int NS = L::NS, NT = NTG<S, G>;
   constexpr int GS = G * S;
+  // below the top level: an exit its walks never finished lies on a cycle
+  if (counters && blockIdx.x == 0 && threadIdx.x == 0 && counters[1] != counters[2]) set_status(status, D8_ERR_CYCLE);
   TileQueue tq(queue, ngroups);
   for (int64_t gu = tq.first(); gu < ngroups; gu = tq.next()) {
     const DemDesc gd = dem_of(gdt, gu);
@@ -372,17 +378,17 @@ __global__ void __launch_bounds__(NTG) k_group_down(DemTable cdt, DemTable gdt, 
     const int64_t lg = gu - gd.tile_base;
     const int64_t gy = lg / gd.ntx, gx = lg % gd.ntx;
     const GroupGeo gg = group_geo<S, G>(gd, gy, gx);
-    group_load<S, G, NTG, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
+    group_load<S, G, NT, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
     // inflow across the group border: each border cell r receives the final
     // areas of the outside cells draining into it; the inflow then follows
     // r's path inside its child unit to that child's exit
-    constexpr int NB = 4 * GS / NTG;  // border slots per thread
-    static_assert(4 * GS % NTG == 0, "whole rounds over the border");
+    constexpr int NB = 4 * GS / NT;  // border slots per thread
+    static_assert(4 * GS % NT == 0, "whole rounds over the border");
     V bin[RECV ? NB : 1];  // inflow across the border and the child slot it enters
     int bslot[RECV ? NB : 1];
 #pragma unroll 1
     for (int r = 0; r < NB; r++) {
-      const int gs = threadIdx.x + r * NTG;
+      const int gs = threadIdx.x + r * NT;
       if (RECV) bslot[RECV ? r : 0] = -1;
       int ci, cj;
       if (!slot_cell(gs, gg.h, gg.w, GS, ci, cj)) continue;
@@ -412,17 +418,17 @@ __global__ void __launch_bounds__(NTG) k_group_down(DemTable cdt, DemTable gdt, 
       }
     }
     __syncthreads();
-    group_walk<S, G, NTG, V>(spx, val, pd, srcl);
+    group_walk<S, G, NT, V>(spx, val, pd, srcl);
     __syncthreads();
     if constexpr (RECV) {
       uint32_t* infl = pd;  // the walk is done with it
-      receivers_inflow<S, G, NTG>(gg, spx, val, infl);
+      receivers_inflow<S, G, NT>(gg, spx, val, infl);
 #pragma unroll 1
       for (int r = 0; r < NB; r++)
         if (bslot[r] >= 0) atomicAdd(&infl[bslot[r]], bin[r]);
       __syncthreads();
     }
-    for (int n = threadIdx.x; n < NS; n += NTG) {
+    for (int n = threadIdx.x; n < NS; n += NT) {
       if (!RECV && !(spx[n] & PEX_EXIT)) continue;
       const int lt = n / (4 * S), s = n - lt * (4 * S);
       const int64_t cy = gy * G + lt / G, cx = gx * G + lt % G;
@@ -480,139 +486,100 @@ static cudaError_t launch_solve(const HLevel& t, uint32_t* status, cudaStream_t 
 
 // ---- top level: Algorithms 5-6 over the remaining units, in global memory
 
+// A node's word: children left (bits 32..47), children in all (bits 48..63)
+// and, unit counts, the value (low half).  The count of all children tells the
+// sources (exits without any) from nodes whose children have arrived.  (A unit
+// of side 512 has 2048 slots and at most nine units drain into one: 16 bits.)
+constexpr unsigned long long CHILD = (1ull << 32) | (1ull << 48), LEFT = 1ull << 32;
+__device__ __forceinline__ uint32_t left_of(unsigned long long w) { return (uint32_t)(w >> 32) & 0xFFFFu; }
+
+// parents, children counts and values (the words were zeroed by the level below)
 template <int S, class V, class CV>
-__global__ void k_top_init(DemTable dt, const uint16_t* pex, const CV* pval, V* fin, uint32_t* par, uint32_t* deg,
-                           int64_t nslots) {
+__global__ void k_top_init(DemTable dt, const uint16_t* pex, const CV* pval, V* fin, uint32_t* par,
+                           unsigned long long* node, int64_t nslots) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nslots; g += stride) {
     const uint16_t pe = pex[g];
+    if (!(pe & PEX_EXIT)) continue;
+    const int64_t t = g / (4 * S);
+    const int s = (int)(g - t * (4 * S));
+    const DemDesc d = dem_of(dt, t);
+    const int64_t lt = t - d.tile_base;
+    const UnitGeo u = unit_geo(d, lt / d.ntx, lt % d.ntx, S);
+    int i, j;
+    slot_cell(s, u.h, u.w, S, i, j);
+    const int k = pe & 7;
+    const int64_t y = global_slot(d, u.i0 + i + code_di(k), u.j0 + j + code_dj(k), S);
+    const uint16_t pey = pex[y];
     uint32_t pr = ROOT;
-    if (pe & PEX_EXIT) {
-      const int64_t t = g / (4 * S);
-      const int s = (int)(g - t * (4 * S));
-      const DemDesc d = dem_of(dt, t);
-      const int64_t lt = t - d.tile_base;
-      const UnitGeo u = unit_geo(d, lt / d.ntx, lt % d.ntx, S);
-      int i, j;
-      slot_cell(s, u.h, u.w, S, i, j);
-      const int k = pe & 7;
-      const int64_t y = global_slot(d, u.i0 + i + code_di(k), u.j0 + j + code_dj(k), S);
-      const uint16_t pey = pex[y];
-      if (pey & PEX_EXIT)
-        pr = (uint32_t)y;
-      else if (pey != PEX_TERM)
-        pr = (uint32_t)((y / (4 * S)) * (4 * S) + pey);
-      if constexpr (std::is_same<V, uint32_t>::value) {
-        // unit counts: children left (high half) and value (low half) in one
-        // 64-bit word per node (zeroed before the launch)
-        unsigned long long* fd = reinterpret_cast<unsigned long long*>(deg);
-        if (pr != ROOT) atomicAdd(&fd[pr], 1ull << 32);
-        atomicAdd(&fd[g], (unsigned long long)pval[g]);
-      } else {
-        if (pr != ROOT) atomicAdd(&deg[pr], 1u);
-        fin[g] = pval[g];
-      }
-    }
+    if (pey & PEX_EXIT)
+      pr = (uint32_t)y;
+    else if (pey != PEX_TERM)
+      pr = (uint32_t)((y / (4 * S)) * (4 * S) + pey);
+    if (pr != ROOT) atomicAdd(&node[pr], CHILD);
+    if constexpr (std::is_same<V, uint32_t>::value)
+      atomicAdd(&node[g], (unsigned long long)pval[g]);
+    else
+      fin[g] = pval[g];
     par[g] = pr;
   }
 }
 
-// The sources (exits without children) listed, and the exits counted, with
-// one atomic per block on each grid-wide counter: a first pass counts this
-// thread's sources, a block scan gives each thread its offset inside the
-// block's range, and a second pass writes them (same slots, same order).
-// (PK: children counts packed in the high half of 64-bit node words)
-template <bool PK>
-__global__ void __launch_bounds__(256) k_top_sources(const uint16_t* pex, const uint32_t* deg, uint32_t* list,
-                                                     uint32_t* counters, int64_t nslots) {
-  auto childless = [&](int64_t g) {
-    return PK ? (reinterpret_cast<const unsigned long long*>(deg)[g] >> 32) == 0ull : deg[g] == 0u;
-  };
-  __shared__ uint32_t sh[256];
-  __shared__ uint32_t sh_base;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t g0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t nsrc = 0, nex = 0;
-  for (int64_t g = g0; g < nslots; g += stride) {
-    const bool ex = (pex[g] & PEX_EXIT) != 0;
-    nex += ex;
-    nsrc += ex && childless(g);
-  }
-  // block-wide inclusive scan of the source counts (Hillis-Steele)
-  sh[threadIdx.x] = nsrc;
-  __syncthreads();
-  for (int off = 1; off < 256; off <<= 1) {
-    const uint32_t add = threadIdx.x >= off ? sh[threadIdx.x - off] : 0u;
-    __syncthreads();
-    sh[threadIdx.x] += add;
-    __syncthreads();
-  }
-  const uint32_t block_src = sh[255];
-  uint32_t excl = sh[threadIdx.x] - nsrc;
-  __syncthreads();
-  // exits: reduce into sh[0] with a second scan-free pass
-  sh[threadIdx.x] = nex;
-  __syncthreads();
-  for (int off = 128; off > 0; off >>= 1) {
-    if (threadIdx.x < off) sh[threadIdx.x] += sh[threadIdx.x + off];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    sh_base = block_src ? atomicAdd(&counters[0], block_src) : 0u;
-    if (sh[0]) atomicAdd(&counters[1], sh[0]);
-  }
-  __syncthreads();
-  uint32_t pos = sh_base + excl;
-  if (nsrc)
-    for (int64_t g = g0; g < nslots; g += stride)
-      if ((pex[g] & PEX_EXIT) && childless(g)) list[pos++] = (uint32_t)g;
-}
-
-// Algorithm 6 with global atomics: last-arriver walks up the exit forest.
-// Unit counts: one packed 64-bit atomic per step delivers the value and tells
-// the last child (no fences); each finished node stores its value for the
-// down sweep.  Float-float: value add, fence, children count, fence.
+// Algorithm 6 with global atomics: last-arriver walks up the exit forest from
+// the sources, each started by the thread that comes across it (the slots'
+// walks are short; a list of the sources, to give every thread one, took two
+// passes of its own: 8192 x 8192 11 us and 27 for the walks, 32768 x 32768 37
+// and 188).  Unit counts: one 64-bit atomic per step delivers the value and
+// tells the last child (no fences); each finished node stores its value for
+// the down sweep.  Float-float: value add, then children count, released and
+// acquired by its atomic.
+// counters: [1] exits, [2] finished.
 template <class V>
-__global__ void k_top_walk(const uint32_t* par, V* fin, uint32_t* deg, const uint32_t* list, uint32_t* counters) {
-  const uint32_t n = *(volatile const uint32_t*)&counters[0];
-  uint32_t done = 0;
-  if constexpr (std::is_same<V, uint32_t>::value) {
-    unsigned long long* fd = reinterpret_cast<unsigned long long*>(deg);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-      uint32_t x = list[i];
-      uint32_t v = (uint32_t)fd[x];  // a source: its own value
+__global__ void __launch_bounds__(256) k_top_walk(const uint16_t* pex, const uint32_t* par, V* fin,
+                                                  unsigned long long* node, uint32_t* counters, int64_t nslots) {
+  uint32_t done = 0, exits = 0;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nslots; g += stride) {
+    if (!(pex[g] & PEX_EXIT)) continue;
+    exits++;
+    const unsigned long long w = *(volatile const unsigned long long*)&node[g];
+    if (w >> 48) continue;  // has children: their walks come here
+    uint32_t x = (uint32_t)g;
+    if constexpr (std::is_same<V, uint32_t>::value) {
+      uint32_t v = (uint32_t)w;
       for (;;) {
         fin[x] = v;
         done++;
         const uint32_t p = par[x];
         if (p == ROOT) break;
-        const unsigned long long old = atomicAdd(&fd[p], (unsigned long long)v - (1ull << 32));
-        if ((old >> 32) != 1ull) break;
+        const unsigned long long old = atomicAdd(&node[p], (unsigned long long)v - LEFT);
+        if (left_of(old) != 1u) break;
         v += (uint32_t)old;
         x = p;
       }
-    }
-  } else {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-      uint32_t x = list[i];
+    } else {
       V v = fin[x];
       done++;
       for (;;) {
         const uint32_t p = par[x];
         if (p == ROOT) break;
         vatomic_add(&fin[p], v);
-        if (atomic_add_acq_rel_gpu(&deg[p], 0u - 1u) != 1u) break;  // releases the addition; acquires the others'
+        // the high half of the word: releases the addition; acquires the others'
+        const uint32_t old = atomic_add_acq_rel_gpu(reinterpret_cast<uint32_t*>(&node[p]) + 1, 0u - 1u);
+        if ((old & 0xFFFFu) != 1u) break;
         x = p;
         v = vload_volatile(&fin[p]);
         done++;
       }
     }
   }
-  if (done) atomicAdd(&counters[2], done);
-}
-
-__global__ void k_top_check(const uint32_t* counters, uint32_t* status) {
-  if (threadIdx.x == 0 && blockIdx.x == 0 && counters[1] != counters[2]) set_status(status, D8_ERR_CYCLE);
+  __shared__ uint32_t sum[2];
+  if (threadIdx.x < 2) sum[threadIdx.x] = 0u;
+  __syncthreads();
+  if (exits) atomicAdd(&sum[0], exits);
+  if (done) atomicAdd(&sum[1], done);
+  __syncthreads();
+  if (threadIdx.x < 2 && sum[threadIdx.x]) atomicAdd(&counters[1 + threadIdx.x], sum[threadIdx.x]);
 }
 
 // ---- top level by pointer jumping (strategy 2).  The queue walk above costs
@@ -697,7 +664,9 @@ __global__ void k_topj_check(const uint32_t* flags, int R, uint32_t* status) {
   if (threadIdx.x == 0 && blockIdx.x == 0 && flags[R] != 0u) set_status(status, D8_ERR_CYCLE);
 }
 
-// every exit listed (same scheme as k_top_sources: one atomic per block)
+// every exit listed, with one atomic per block on the list's length: a first
+// pass counts this thread's exits, a block scan (Hillis-Steele) gives each
+// thread its offset inside the block's range, a second pass writes them
 __global__ void __launch_bounds__(256) k_topj_list(const uint16_t* pex, uint32_t* list, uint32_t* counters,
                                                    int64_t nslots) {
   __shared__ uint32_t sh[256];
@@ -724,8 +693,8 @@ __global__ void __launch_bounds__(256) k_topj_list(const uint16_t* pex, uint32_t
 
 template <int S, int G, class V, class CV>
 static cudaError_t launch_level_up(const DemTable& cdt, const DemTable& gdt, const uint16_t* cpex, const void* cpval,
-                                   uint16_t* gpex, void* gpval, int64_t ngroups, uint32_t* queue, uint32_t* status,
-                                   cudaStream_t s) {
+                                   uint16_t* gpex, void* gpval, unsigned long long* node, int64_t ngroups,
+                                   uint32_t* queue, uint32_t* status, cudaStream_t s) {
   using L = GroupLayout<S, G, V>;
   auto k = k_group_up<S, G, V, CV>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
@@ -733,19 +702,18 @@ static cudaError_t launch_level_up(const DemTable& cdt, const DemTable& gdt, con
   int per_sm = 1, dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NTG, L::bytes);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NTG<S, G>, L::bytes);
   int64_t grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * sms;
   if (grid > ngroups) grid = ngroups;
-  e = cudaMemsetAsync(queue, 0, sizeof(uint32_t), s);
-  if (e != cudaSuccess) return e;
-  k<<<(unsigned)grid, NTG, L::bytes, s>>>(cdt, gdt, cpex, static_cast<const CV*>(cpval), gpex, static_cast<V*>(gpval),
-                                          ngroups, queue, status);
+  k<<<(unsigned)grid, NTG<S, G>, L::bytes, s>>>(cdt, gdt, cpex, static_cast<const CV*>(cpval), gpex,
+                                                static_cast<V*>(gpval), node, ngroups, queue, status);
   return cudaGetLastError();
 }
 
 template <int S, int G, class V, class CV, bool RECV>
 static cudaError_t launch_level_down(const DemTable& cdt, const DemTable& gdt, const uint16_t* cpex, const void* cpval,
-                                     void* cfin, const void* gfin, int64_t ngroups, uint32_t* queue, cudaStream_t s) {
+                                     void* cfin, const void* gfin, int64_t ngroups, uint32_t* queue,
+                                     const uint32_t* counters, uint32_t* status, cudaStream_t s) {
   using L = GroupLayout<S, G, V>;
   auto k = k_group_down<S, G, V, CV, RECV>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
@@ -753,13 +721,11 @@ static cudaError_t launch_level_down(const DemTable& cdt, const DemTable& gdt, c
   int per_sm = 1, dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NTG, L::bytes);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NTG<S, G>, L::bytes);
   int64_t grid = (int64_t)(per_sm < 1 ? 1 : per_sm) * sms;
   if (grid > ngroups) grid = ngroups;
-  e = cudaMemsetAsync(queue, 0, sizeof(uint32_t), s);
-  if (e != cudaSuccess) return e;
-  k<<<(unsigned)grid, NTG, L::bytes, s>>>(cdt, gdt, cpex, static_cast<const CV*>(cpval), static_cast<V*>(cfin),
-                                          static_cast<const V*>(gfin), ngroups, queue);
+  k<<<(unsigned)grid, NTG<S, G>, L::bytes, s>>>(cdt, gdt, cpex, static_cast<const CV*>(cpval), static_cast<V*>(cfin),
+                                                static_cast<const V*>(gfin), ngroups, queue, counters, status);
   return cudaGetLastError();
 }
 
@@ -767,7 +733,6 @@ template <int S, class V, class CV>
 static cudaError_t launch_top_jump(const DemTable& dt, const HLevel& lv, const HTop& top, cudaStream_t s, int* nl) {
   const int64_t ns = lv.nunits * 4 * S;
   cudaError_t e = cudaMemsetAsync(top.flags, 0, sizeof(uint32_t) * (MAX_ROUNDS + 2), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(top.counters, 0, sizeof(uint32_t) * 4, s);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
@@ -776,7 +741,7 @@ static cudaError_t launch_top_jump(const DemTable& dt, const HLevel& lv, const H
   if (b > (int64_t)sms * 16) b = (int64_t)sms * 16;
   if (b < 1) b = 1;
   V* fin = static_cast<V*>(lv.fin);
-  V* add = reinterpret_cast<V*>(top.deg);
+  V* add = reinterpret_cast<V*>(top.node);
   k_topj_init<S, V, CV><<<(unsigned)b, 256, 0, s>>>(dt, lv.pex, static_cast<const CV*>(lv.pval), fin, top.par, add,
                                                     top.flags, ns);
   k_topj_list<<<(unsigned)b, 256, 0, s>>>(lv.pex, top.list, top.counters, ns);
@@ -798,37 +763,34 @@ template <int S, class V, class CV>
 static cudaError_t launch_top(const DemTable& dt, const HLevel& lv, const HTop& top, cudaStream_t s, int* nl) {
   if (top.jump) return launch_top_jump<S, V, CV>(dt, lv, top, s, nl);
   const int64_t ns = lv.nunits * 4 * S;
-  cudaError_t e = cudaMemsetAsync(top.deg, 0, sizeof(unsigned long long) * (size_t)ns, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(top.counters, 0, sizeof(uint32_t) * 4, s);
-  if (e != cudaSuccess) return e;
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int64_t b = (ns + 255) / 256;
-  if (b > (int64_t)sms * 16) b = (int64_t)sms * 16;
-  if (b < 1) b = 1;
-  k_top_init<S, V, CV><<<(unsigned)b, 256, 0, s>>>(dt, lv.pex, static_cast<const CV*>(lv.pval),
-                                                   static_cast<V*>(lv.fin), top.par, top.deg, ns);
-  k_top_sources<std::is_same<V, uint32_t>::value><<<(unsigned)b, 256, 0, s>>>(lv.pex, top.deg, top.list,
-                                                                             top.counters, ns);
-  k_top_walk<V><<<(unsigned)(sms * 8), 256, 0, s>>>(top.par, static_cast<V*>(lv.fin), top.deg, top.list,
-                                                    top.counters);
-  k_top_check<<<1, 32, 0, s>>>(top.counters, top.status);
-  *nl += 4;
+  const unsigned b = (unsigned)min64((ns + 255) / 256, (int64_t)sms * 16);
+  k_top_init<S, V, CV><<<b, 256, 0, s>>>(dt, lv.pex, static_cast<const CV*>(lv.pval), static_cast<V*>(lv.fin), top.par,
+                                         top.node, ns);
+  k_top_walk<V><<<(unsigned)min64(b, (int64_t)sms * 8), 256, 0, s>>>(lv.pex, top.par, static_cast<V*>(lv.fin), top.node,
+                                                                     top.counters, ns);
+  *nl += 2;
   return cudaGetLastError();
 }
 
 }  // namespace cmb
 
-// Level schedule: tiles of side T, then groups of G = 4 (from 32 or 64) or
-// G = 2 children, up to a group side of 512 cells; the global queue solve
-// takes the rest.  (A 1024-cell level cost more than the longer top-level
-// chains it saves: measured at 8192^2 and 32768^2.)
-int hier_levels(int T, int64_t max_side, int* S, int* G, int max_levels) {
+// Level schedule: groups of 8 x 8 tiles (wide; 32 or 64 a side), or of 4 x 4,
+// then of 2 x 2 children, up to a group side of 512 cells; the global queue
+// solve takes the rest.  (A 1024-cell level cost more than the longer
+// top-level chains it saves: measured at 8192^2 and 32768^2.)  One level of 8 x
+// 8 in blocks of 1024 threads instead of 4 x 4 and 2 x 2 in blocks of 256: the
+// whole combine takes 182 us at 8192^2 (237), 1.69 ms at 32768^2 (2.02), 110 us
+// at 3001 x 5003 (142).  Not for float-float values (8 x 8 children do not fit
+// shared memory), nor under strategy "jump", whose long chains are walked
+// inside a group: two levels halve them.
+int hier_levels(int T, int64_t max_side, bool wide, int* S, int* G, int max_levels) {
   int n = 0;
   int s = T;
   while (n < max_levels && s < max_side && s < 512) {
-    const int g = (s <= 64) ? 4 : 2;
+    const int g = (s <= 64) ? (wide ? 8 : 4) : 2;
     S[n] = s;
     G[n] = g;
     s *= g;
@@ -850,13 +812,17 @@ static cudaError_t combine_hier_t(const HPlan& hp, cudaStream_t s, int* nlaunch)
     const int S = c.S, G = g.S / c.S;
 #define D8_UP(SS, GG)                                                                                             \
   if (S == SS && G == GG) {                                                                                      \
-    e = l == 1 ? launch_level_up<SS, GG, V, CV0>(c.dt, g.dt, c.pex, c.pval, g.pex, g.pval, g.nunits, hp.queue + l,  \
-                                                 hp.status, s)                                                   \
-               : launch_level_up<SS, GG, V, V>(c.dt, g.dt, c.pex, c.pval, g.pex, g.pval, g.nunits, hp.queue + l,    \
-                                               hp.status, s);                                                    \
+    unsigned long long* node = l == hp.nlev && hp.need_top && !hp.top.jump ? hp.top.node : nullptr;               \
+    e = l == 1 ? launch_level_up<SS, GG, V, CV0>(c.dt, g.dt, c.pex, c.pval, g.pex, g.pval, node, g.nunits,         \
+                                                 hp.queue + l, hp.status, s)                                      \
+               : launch_level_up<SS, GG, V, V>(c.dt, g.dt, c.pex, c.pval, g.pex, g.pval, node, g.nunits,           \
+                                               hp.queue + l, hp.status, s);                                       \
     ++*nlaunch;                                                                                                  \
     continue;                                                                                                    \
   }
+    if constexpr (std::is_same<V, uint32_t>::value) {
+      D8_UP(32, 8) D8_UP(64, 8)
+    }
     D8_UP(32, 4) D8_UP(64, 4) D8_UP(128, 2) D8_UP(256, 2)
 #undef D8_UP
     return cudaErrorInvalidValue;
@@ -865,16 +831,9 @@ static cudaError_t combine_hier_t(const HPlan& hp, cudaStream_t s, int* nlaunch)
   // top
   const HLevel& t = hp.lev[hp.nlev];
   if (hp.need_top) {
-    const bool l0 = hp.nlev == 0;
-#define D8_TOP(SS)                                                                                 \
-  case SS:                                                                                         \
-    e = l0 ? launch_top<SS, V, CV0>(t.dt, t, hp.top, s, nlaunch) : launch_top<SS, V, V>(t.dt, t, hp.top, s, nlaunch); \
-    break;
-    switch (t.S) {
-      D8_TOP(32) D8_TOP(64) D8_TOP(128) D8_TOP(256) D8_TOP(512)
-      default: return cudaErrorInvalidValue;
-    }
-#undef D8_TOP
+    // (a grid of more than one unit has levels up to 512)
+    if (t.S != 512) return cudaErrorInvalidValue;
+    e = launch_top<512, V, V>(t.dt, t, hp.top, s, nlaunch);
     if (e != cudaSuccess) return e;
   }
   // down: level l -> l-1 (at the tiles: unit counts leave the receivers' inflow)
@@ -885,13 +844,17 @@ static cudaError_t combine_hier_t(const HPlan& hp, cudaStream_t s, int* nlaunch)
     const int S = c.S, G = g.S / c.S;
 #define D8_DN(SS, GG)                                                                                               \
   if (S == SS && G == GG) {                                                                                        \
+    const uint32_t* cnt = l == hp.nlev && hp.need_top && !hp.top.jump ? hp.top.counters : nullptr;                \
     e = l == 1 ? launch_level_down<SS, GG, V, CV0, RECV>(c.dt, g.dt, c.pex, c.pval, c.fin, g.fin, g.nunits,         \
-                                                         hp.queue + 16 + l, s)                                     \
+                                                         hp.queue + 16 + l, cnt, hp.status, s)                    \
                : launch_level_down<SS, GG, V, V, false>(c.dt, g.dt, c.pex, c.pval, c.fin, g.fin, g.nunits,          \
-                                                        hp.queue + 16 + l, s);                                     \
+                                                        hp.queue + 16 + l, cnt, hp.status, s);                    \
     ++*nlaunch;                                                                                                    \
     continue;                                                                                                      \
   }
+    if constexpr (std::is_same<V, uint32_t>::value) {
+      D8_DN(32, 8) D8_DN(64, 8)
+    }
     D8_DN(32, 4) D8_DN(64, 4) D8_DN(128, 2) D8_DN(256, 2)
 #undef D8_DN
     return cudaErrorInvalidValue;

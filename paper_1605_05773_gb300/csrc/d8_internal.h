@@ -110,10 +110,10 @@ struct HTop {  // the top level's solve in global memory (queue method or pointe
   uint32_t* par;
   uint32_t* par2;  // pointer jumping: the second parent buffer
   uint32_t* flags; // pointer jumping: per-round "still active" flags (MAX_ROUNDS + 2)
-  uint32_t* deg;  // 8 bytes per slot: unit counts pack children left (high) and value (low);
-                  // pointer jumping: this round's additions (value type)
-  uint32_t* list;
-  uint32_t* counters;  // [0] sources, [1] exits, [2] finished
+  unsigned long long* node;  // per slot: children counts and, unit counts, the value (k_top_init);
+                             // pointer jumping: this round's additions (value type)
+  uint32_t* list;      // pointer jumping: the exits
+  uint32_t* counters;  // pointer jumping: [0] exits; queue walk: [1] exits, [2] finished
   uint32_t* status;
 };
 struct HPlan {
@@ -123,11 +123,11 @@ struct HPlan {
   HLevel lev[HMAX];
   bool need_top;
   HTop top;
-  uint32_t* queue;  // 32 work-queue counters
+  uint32_t* queue;  // 32 work-queue counters, the top's counters at 48: zero at the start
   uint32_t* status;
 };
 // group sides of the levels above tiles of side T, for grids up to max_side
-int hier_levels(int T, int64_t max_side, int* S, int* G, int max_levels);
+int hier_levels(int T, int64_t max_side, bool wide, int* S, int* G, int max_levels);
 // the largest side of a grid that one group of the single-launch combine
 // covers (unit counts)
 int solve_side(int T);
