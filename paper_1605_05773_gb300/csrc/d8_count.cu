@@ -27,11 +27,12 @@
 //    short chase: the exits of the perimeter cells.
 //  * the next tile's codes are requested before this one's walks.
 //
-// Measured, T = 64: 32768 x 32768 fractal 3.82 ms, 8192 x 8192 262 us (before:
+// Measured, T = 64: 32768 x 32768 fractal 3.77 ms, 8192 x 8192 261 us (before:
 // 6.53 ms and 435 us, 128 threads, a 16-bit segment record per cell beside the
-// word, 8 tiles per SM, one ring of starts per warp).  11264 warp instructions
-// per tile (21000).  Where the 262 us go: words 40, sweep 43, batches 60, the
-// last walks 57, counts to A 12, summary 32, the rest 17.
+// word, 8 tiles per SM, one ring of starts per warp); 3001 x 5003, rows at odd
+// addresses: 85 us (110 with byte loads and strided stores).  11264 warp
+// instructions per tile (21000).  Where the 261 us go: words 40, sweep 43,
+// batches 60, the last walks 57, counts to A 12, summary 32, the rest 17.
 #include "d8_device.cuh"
 
 namespace d8 {
@@ -174,35 +175,52 @@ __device__ __forceinline__ int signed_byte(uint2 v, uint32_t k) {
   return r;
 }
 
-// The codes of a tile, loaded ahead: four consecutive cells of a row per
-// 32-bit word, rows i0, i0 + RS, ... of group q per thread.
+// The codes of a whole tile, loaded ahead: four consecutive cells of a row per
+// 32-bit word, rows i0, i0 + RS, ... of group q per thread.  Every load is
+// issued before any is used, one word per group.  Rows that start at an odd
+// address are read as the aligned words that cover them and shifted into place
+// when they are used; the word after a row's last group is held by the lane of
+// that row's number among the thread's.  (Ragged tiles read theirs later.)
 template <int T>
 struct Codes {
-  static constexpr int NQ = T * T / 4 / NTC;    // four-cell groups per thread
-  static constexpr int RS = NTC / Place<T>::Q;  // rows from one group of a thread to its next
-  uint32_t four[NQ];
-  __device__ static __forceinline__ int row0() { return threadIdx.x / Place<T>::Q; }
-  __device__ static __forceinline__ int group() { return threadIdx.x & (Place<T>::Q - 1); }
+  static constexpr int Q = Place<T>::Q;
+  static constexpr int NQ = T * T / 4 / NTC;  // four-cell groups per thread
+  static constexpr int RS = NTC / Q;          // rows from one group of a thread to its next
+  static_assert(NQ <= Q, "a lane per row for the words after the rows");
+  uint32_t word[NQ], after;
+  __device__ static __forceinline__ int row0() { return threadIdx.x / Q; }
+  __device__ static __forceinline__ int group() { return threadIdx.x & (Q - 1); }
+  // address of the codes of this thread's group in row0() + r * RS
+  __device__ static __forceinline__ const uint8_t* first(const DemDesc& d, const TileGeo& g, int r) {
+    return d.dir + (g.i0 + row0() + r * RS) * d.lddir + (g.j0 + 4 * group());
+  }
+  __device__ static __forceinline__ bool aligned(const DemDesc& d) {
+    return ((reinterpret_cast<uintptr_t>(d.dir) | (uintptr_t)d.lddir) & 3u) == 0;
+  }
 
-  // every load is issued before any is used (one 32-bit load per group when
-  // the layout allows)
   __device__ __forceinline__ void load(const DemDesc& d, const TileGeo& g) {
-    const bool vec = (g.tw == T) && ((reinterpret_cast<uintptr_t>(d.dir) & 3u) == 0) && (d.lddir % 4 == 0);
-    const uint8_t* src = d.dir + (g.i0 + row0()) * d.lddir + (g.j0 + 4 * group());
+    if (g.tw != T || g.th != T) return;
+    if (aligned(d)) {
 #pragma unroll
-    for (int r = 0; r < NQ; r++) {
-      four[r] = 0;
-      if (row0() + r * RS < g.th) {
-        if (vec) {
-          four[r] = __ldg(reinterpret_cast<const unsigned int*>(src));
-        } else {
+      for (int r = 0; r < NQ; r++) word[r] = __ldg(reinterpret_cast<const unsigned int*>(first(d, g, r)));
+    } else {
 #pragma unroll
-          for (int k = 0; k < 4; k++)
-            if (4 * group() + k < g.tw) four[r] |= (uint32_t)__ldg(src + k) << (8 * k);
-        }
+      for (int r = 0; r < NQ; r++)
+        word[r] = __ldg(reinterpret_cast<const unsigned int*>(reinterpret_cast<uintptr_t>(first(d, g, r)) & ~(uintptr_t)3));
+      // lane q: the word that ends row row0() + q * RS, where its bytes are needed
+      after = 0;
+      if (group() < NQ) {
+        const uintptr_t end = reinterpret_cast<uintptr_t>(d.dir + (g.i0 + row0() + group() * RS) * d.lddir + g.j0 + T);
+        if (end & 3u) after = __ldg(reinterpret_cast<const unsigned int*>(end & ~(uintptr_t)3));
       }
-      src += RS * d.lddir;
     }
+  }
+  // once loaded: word[r] becomes the codes of group r
+  __device__ __forceinline__ void shift(const DemDesc& d, const TileGeo& g) {
+    if (g.tw != T || g.th != T || aligned(d)) return;
+#pragma unroll
+    for (int r = 0; r < NQ; r++)
+      word[r] = unaligned_four<Q>(word[r], __shfl_sync(FULL, after, r, Q), first(d, g, r));
   }
 };
 
@@ -226,7 +244,7 @@ __device__ __forceinline__ void set_words(const Codes<T>& codes, const DemDesc& 
     uint32_t wrong = 0;
 #pragma unroll
     for (int r = 0; r < NQ; r++) {
-      const uint32_t four = codes.four[r];
+      const uint32_t four = codes.word[r];
       wrong |= ((four & 0x7F7F7F7Fu) + 0x76767676u) | four;  // bit 7 of a byte: above 9
       uint2 dist_of[4];
 #pragma unroll
@@ -248,10 +266,20 @@ __device__ __forceinline__ void set_words(const Codes<T>& codes, const DemDesc& 
     if (wrong & 0x80808080u) set_status(status, D8_ERR_ARG);  // (such a cell's path ends there)
     return;
   }
-#pragma unroll 4
-  for (int c = threadIdx.x; c < T * T; c += NTC) {
-    const int i = c / T, j = c % T;
-    if (i < g.th && j < g.tw) add_cell<T>(word, i, j, __ldg(d.dir + (g.i0 + i) * d.lddir + (g.j0 + j)), g, d, status);
+  constexpr int U = 16;  // codes read at once
+#pragma unroll 1
+  for (int c0 = threadIdx.x; c0 < T * T; c0 += U * NTC) {
+    uint8_t code[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int c = c0 + u * NTC, i = c / T, j = c % T;
+      code[u] = i < g.th && j < g.tw ? __ldg(d.dir + (g.i0 + i) * d.lddir + (g.j0 + j)) : (uint8_t)0;
+    }
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int c = c0 + u * NTC, i = c / T, j = c % T;
+      if (i < g.th && j < g.tw) add_cell<T>(word, i, j, code[u], g, d, status);
+    }
   }
 }
 
@@ -272,22 +300,22 @@ __device__ __forceinline__ void end_at_grid_edge(const DemDesc& d, const TileGeo
   }
 }
 
-// A[tile] = the in-tile counts, four consecutive cells per thread per step (one
-// 16-byte store when the layout allows).  Returns whether one of this thread's
+// A[tile] = the in-tile counts: four consecutive cells per thread in one 16-byte
+// store when the layout allows, else one.  Returns whether one of this thread's
 // cells still waits for an input: it lies on or below a cycle.
 template <int T>
 __device__ __forceinline__ bool store_counts(const DemDesc& d, const TileGeo& g, const uint32_t* word) {
   using P = Place<T>;
   using C = Cell<T>;
-  constexpr int RS = NTC / P::Q;  // rows from one group of a thread to its next
-  const int i0 = threadIdx.x / P::Q, j = 4 * (threadIdx.x & (P::Q - 1));
-  uint32_t* dst = static_cast<uint32_t*>(d.A) + (g.i0 + i0) * d.ldA + (g.j0 + j);
-  const bool vec = g.tw == T && ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0) && (d.ldA & 3) == 0;
-  const uint32_t* w0[4];
-#pragma unroll
-  for (int k = 0; k < 4; k++) w0[k] = word + P::of(i0, j + k);
   uint32_t left = 0;
-  if (vec && g.th == T) {
+  const bool vec = g.tw == T && g.th == T && ((reinterpret_cast<uintptr_t>(d.A) & 15u) == 0) && (d.ldA & 3) == 0;
+  if (vec) {
+    constexpr int RS = NTC / P::Q;  // rows from one group of a thread to its next
+    const int i0 = threadIdx.x / P::Q, j = 4 * (threadIdx.x & (P::Q - 1));
+    uint32_t* dst = static_cast<uint32_t*>(d.A) + (g.i0 + i0) * d.ldA + (g.j0 + j);
+    const uint32_t* w0[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) w0[k] = word + P::of(i0, j + k);
 #pragma unroll
     for (int r = 0; r < T / RS; r++) {
       uint32_t w[4];
@@ -299,14 +327,18 @@ __device__ __forceinline__ bool store_counts(const DemDesc& d, const TileGeo& g,
       dst += RS * d.ldA;
     }
   } else {
-    for (int r = 0; r < T / RS && i0 + r * RS < g.th; r++) {
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-        const uint32_t w = w0[k][r * RS * T];
-        left |= w;  // (the absent cells' words are 0)
-        if (j + k < g.tw) dst[k] = w >> C::CB;
+    // consecutive lanes store consecutive columns
+    constexpr int RS = NTC / T;  // rows at once
+    const int i0 = threadIdx.x / T, j = threadIdx.x % T;
+    uint32_t* dst = static_cast<uint32_t*>(d.A) + (g.i0 + i0) * d.ldA + (g.j0 + j);
+    if (j < g.tw) {
+#pragma unroll 8
+      for (int i = i0; i < g.th; i += RS) {
+        const uint32_t w = word[P::of(i, j)];
+        left |= w;
+        *dst = w >> C::CB;
+        dst += RS * d.ldA;
       }
-      dst += RS * d.ldA;
     }
   }
   return left >= LEFT1;
@@ -451,6 +483,7 @@ __global__ void __launch_bounds__(NTC, 12) k_up_count(DemTable dt, Pipe p) {
       misc[2] = gridDim.x + atomicAdd(p.queue, 1u);
     }
     __syncthreads();
+    codes.shift(d, g);
     set_words<T>(codes, d, g, word, tab, p.status);
     __syncthreads();
     end_at_grid_edge<T>(d, g, word);  // (only the summary reads what it changes)

@@ -101,6 +101,18 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// A row of Q * 4 bytes that may start at any address, held by Q consecutive
+// lanes as the aligned words w that cover it (lane q: the word with the first
+// of its four bytes); after: the word after the last one.  Returns lane q's
+// four bytes; `first` is the address of lane q's first byte.  All lanes of the
+// warp call this.
+template <int Q>
+__device__ __forceinline__ uint32_t unaligned_four(uint32_t w, uint32_t after, const uint8_t* first) {
+  uint32_t next = __shfl_down_sync(0xFFFFFFFFu, w, 1);
+  if ((threadIdx.x & (Q - 1)) == Q - 1) next = after;
+  return __funnelshift_r(w, next, 8u * (uint32_t)(reinterpret_cast<uintptr_t>(first) & 3u));
+}
+
 // DEM of a tile, by value so its fields can live in registers
 __device__ __forceinline__ DemDesc dem_of(const DemTable& t, int64_t tile) {
   if (t.ndem == 1) return t.one;
