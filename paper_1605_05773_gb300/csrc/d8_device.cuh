@@ -209,6 +209,12 @@ __device__ __forceinline__ uint8_t classify(int code, int i, int j, const TileGe
 
 __device__ __forceinline__ void set_status(uint32_t* status, int code) { atomicOr(status, 1u << code); }
 
+// A flag that many blocks raise and the next launch reads: written only while
+// it is seen down, since thousands of writes to one word queue up.
+__device__ __forceinline__ void raise_flag(uint32_t* flag) {
+  if (*(volatile uint32_t*)flag == 0u) *(volatile uint32_t*)flag = 1u;
+}
+
 // Tile work queue: persistent blocks take tile indices until the n tiles run
 // out.  Block b starts with tile b; later indices come from a device counter
 // (zeroed before the launch) offset by the grid size.  With plenty of tiles

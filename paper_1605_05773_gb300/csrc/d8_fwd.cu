@@ -69,7 +69,7 @@ __global__ void k_pj_scatter(Pipe p, int r) {
     Pn[g] = pp;
     active |= (pp != ROOT);
   }
-  if (__syncthreads_or(active) && threadIdx.x == 0) p.flags[r + 1] = 1u;
+  if (__syncthreads_or(active) && threadIdx.x == 0) raise_flag(&p.flags[r + 1]);
 }
 
 template <class V>
