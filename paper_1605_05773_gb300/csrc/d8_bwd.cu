@@ -184,16 +184,49 @@ __global__ void __launch_bounds__(BwdCfg<T>::NTB, T >= 64 ? 2 : 4) k_bwd_up(DemT
   }
 }
 
-// Append the lanes whose `take` is set to list[] at the position counter
-// *cnt hands out (one atomic per warp); every lane of the warp calls this.
-__device__ __forceinline__ void warp_append(bool take, uint32_t item, uint32_t* list, uint32_t* cnt) {
-  const unsigned m = __ballot_sync(0xFFFFFFFFu, take);
-  if (m == 0u) return;
-  const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-  uint32_t pos = 0;
-  if (lane == leader) pos = atomicAdd(cnt, (uint32_t)__popc(m));
-  pos = __shfl_sync(0xFFFFFFFFu, pos, leader);
-  if (take) list[pos + __popc(m & ((1u << lane) - 1u))] = item;
+constexpr int BPJ_U = 4;     // list items or slots per thread and pass
+constexpr int BPJ_NT = 256;  // threads per block of the rounds
+constexpr int BPJ_END = 1024;  // threads of the block that ends them
+
+// Append the items whose `take` is set to list[] at the position counter *cnt
+// hands out, with one atomic per block and pass.  (One per warp queued up
+// behind each other: at 8192 x 8192 the rounds took 353 us and the init 86.)
+// Every thread of the block calls this.
+template <int NT>
+__device__ __forceinline__ void block_append(const bool (&take)[BPJ_U], const uint32_t (&item)[BPJ_U], uint32_t* list,
+                                             uint32_t* cnt) {
+  __shared__ uint32_t start[NT / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned m[BPJ_U];
+  uint32_t n = 0;
+#pragma unroll
+  for (int u = 0; u < BPJ_U; u++) {
+    m[u] = __ballot_sync(0xFFFFFFFFu, take[u]);
+    n += __popc(m[u]);
+  }
+  if (lane == 0) start[warp] = n;
+  __syncthreads();
+  if (warp == 0) {  // where each warp's items start
+    uint32_t mine = lane < NT / 32 ? start[lane] : 0u, sum = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, sum, o);
+      if (lane >= o) sum += x;
+    }
+    const uint32_t all = __shfl_sync(0xFFFFFFFFu, sum, 31);
+    uint32_t base = 0;
+    if (lane == 0 && all) base = atomicAdd(cnt, all);
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    if (lane < NT / 32) start[lane] = base + sum - mine;
+  }
+  __syncthreads();
+  uint32_t pos = start[warp];
+#pragma unroll
+  for (int u = 0; u < BPJ_U; u++) {
+    if (take[u]) list[pos + __popc(m[u] & ((1u << lane) - 1u))] = item[u];
+    pos += __popc(m[u]);
+  }
+  // (start[] is next written after the barrier of the next call's first half)
 }
 
 // combine init: H0(x) = path sum of x's successor inside its tile, parent =
@@ -201,42 +234,53 @@ __device__ __forceinline__ void warp_append(bool take, uint32_t item, uint32_t* 
 // now and go to both value buffers; the others are listed for round 0
 // (flags[r] counts the list of round r).
 template <int T>
-__global__ void k_bpj_init(DemTable dt, Pipe p) {
+__global__ void __launch_bounds__(BPJ_NT) k_bpj_init(DemTable dt, Pipe p) {
   ff* H = static_cast<ff*>(p.S);
   ff* H2 = static_cast<ff*>(p.S2);
   const ff* pval = static_cast<const ff*>(p.pval);
-  const int lane = threadIdx.x & 31;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; base < p.nslots; base += stride) {
-    const int64_t g = base + lane;
-    uint32_t par = ROOT;
-    if (g < p.nslots) {
-      const uint16_t pe = p.pex[g];
-      ff v{0.0f, 0.0f};
-      if (pe & PEX_EXIT) {
-        const int64_t t = g / (4 * T);
-        const int s = (int)(g - t * (4 * T));
-        const DemDesc d = dem_of(dt, t);
-        const TileGeo geo = tile_geo(d, t - d.tile_base, T);
-        int i, j;
-        slot_cell(s, geo.th, geo.tw, T, i, j);
-        const int k = pe & 7;
-        const int64_t y = global_slot(d, geo.i0 + i + code_di(k), geo.j0 + j + code_dj(k), T);
-        const uint16_t pey = p.pex[y];
-        if (pey & PEX_EXIT)
-          par = (uint32_t)y;
-        else if (pey != PEX_TERM)
-          par = (uint32_t)((y / (4 * T)) * (4 * T) + pey);
-        v = pval[y];
-      }
-      p.P[0][g] = par;
-      H[g] = v;
-      if (par == ROOT) {
-        p.P[1][g] = ROOT;
-        H2[g] = v;
-      }
+  const int64_t nt = (int64_t)gridDim.x * BPJ_NT;
+  for (int64_t base = (int64_t)blockIdx.x * BPJ_NT; base < p.nslots; base += BPJ_U * nt) {
+    bool take[BPJ_U];
+    uint32_t item[BPJ_U];
+    uint16_t pe[BPJ_U];
+#pragma unroll
+    for (int u = 0; u < BPJ_U; u++) {
+      const int64_t g = base + threadIdx.x + u * nt;
+      pe[u] = g < p.nslots ? p.pex[g] : PEX_TERM;
     }
-    warp_append(par != ROOT, (uint32_t)g, p.list[0], &p.flags[0]);
+#pragma unroll
+    for (int u = 0; u < BPJ_U; u++) {
+      const int64_t g = base + threadIdx.x + u * nt;
+      uint32_t par = ROOT;
+      if (g < p.nslots) {
+        ff v{0.0f, 0.0f};
+        if (pe[u] & PEX_EXIT) {
+          const int64_t t = g / (4 * T);
+          const int s = (int)(g - t * (4 * T));
+          const DemDesc d = dem_of(dt, t);
+          const TileGeo geo = tile_geo(d, t - d.tile_base, T);
+          int i, j;
+          slot_cell(s, geo.th, geo.tw, T, i, j);
+          const int k = pe[u] & 7;
+          const int64_t y = global_slot(d, geo.i0 + i + code_di(k), geo.j0 + j + code_dj(k), T);
+          const uint16_t pey = p.pex[y];
+          if (pey & PEX_EXIT)
+            par = (uint32_t)y;
+          else if (pey != PEX_TERM)
+            par = (uint32_t)((y / (4 * T)) * (4 * T) + pey);
+          v = pval[y];
+        }
+        p.P[0][g] = par;
+        H[g] = v;
+        if (par == ROOT) {
+          p.P[1][g] = ROOT;
+          H2[g] = v;
+        }
+      }
+      take[u] = par != ROOT;
+      item[u] = (uint32_t)g;
+    }
+    block_append<BPJ_NT>(take, item, p.list[0], &p.flags[0]);
   }
 }
 
@@ -246,29 +290,24 @@ __global__ void k_bpj_init(DemTable dt, Pipe p) {
 // final H into the other buffer, so that both buffers end up final for every
 // slot (a later round may gather it from either).  Each thread takes BPJ_U
 // list items per pass and issues all their loads before using any (the
-// gathers are dependent pairs of random loads).  The pass loop runs the same
-// number of times in every lane of a warp (the stride is a multiple of 32),
-// as warp_append requires.
-constexpr int BPJ_U = 4;
-__global__ void __launch_bounds__(256) k_bpj_round(Pipe p, int r) {
-  const uint32_t n = *(volatile uint32_t*)&p.flags[r];
-  if (n == 0u) return;
+// gathers are dependent pairs of random loads).
+template <int NT>
+__device__ __forceinline__ void bpj_round(const Pipe& p, int r, uint32_t n, uint32_t first, uint32_t step,
+                                          uint32_t* next_count) {
   const ff* Hc = static_cast<const ff*>((r & 1) ? p.S2 : p.S);
   ff* Hn = static_cast<ff*>((r & 1) ? p.S : p.S2);
   const uint32_t* Pc = pick(p.P[0], p.P[1], r & 1);
   uint32_t* Pn = pick(p.P[0], p.P[1], (r + 1) & 1);
   const uint32_t* lc = p.list[r & 1];
   uint32_t* ln = p.list[(r + 1) & 1];
-  const int lane = threadIdx.x & 31;
-  const int64_t nt = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; base < (int64_t)n; base += BPJ_U * nt) {
+  for (uint64_t base = first; base < n; base += (uint64_t)BPJ_U * step) {
     uint32_t g[BPJ_U], par[BPJ_U], pp[BPJ_U];
     ff h[BPJ_U], hp[BPJ_U];
-    bool ok[BPJ_U];
+    bool ok[BPJ_U], keep[BPJ_U];
 #pragma unroll
     for (int u = 0; u < BPJ_U; u++) {
-      const int64_t i = base + lane + u * nt;
-      ok[u] = i < (int64_t)n;
+      const uint64_t i = base + threadIdx.x + (uint64_t)u * step;
+      ok[u] = i < n;
       g[u] = ok[u] ? lc[i] : 0u;
     }
 #pragma unroll
@@ -289,23 +328,38 @@ __global__ void __launch_bounds__(256) k_bpj_round(Pipe p, int r) {
     }
 #pragma unroll
     for (int u = 0; u < BPJ_U; u++) {
-      bool keep = false;
+      keep[u] = false;
       if (ok[u]) {
         if (par[u] != ROOT) {
           h[u] = ff_add(h[u], hp[u]);
-          keep = true;
+          keep[u] = true;
         }
         Hn[g[u]] = h[u];
         Pn[g[u]] = pp[u];
       }
-      warp_append(keep, g[u], ln, &p.flags[r + 1]);
     }
+    block_append<NT>(keep, g, ln, next_count);
   }
 }
 
-// after R rounds the list must be empty; an exit still open lies on a cycle
-__global__ void k_bpj_check(Pipe p, int R) {
-  if (threadIdx.x == 0 && blockIdx.x == 0 && p.flags[R] != 0u) set_status(p.status, D8_ERR_CYCLE);
+__global__ void __launch_bounds__(BPJ_NT) k_bpj_round(Pipe p, int r) {
+  bpj_round<BPJ_NT>(p, r, *(volatile uint32_t*)&p.flags[r], blockIdx.x * BPJ_NT, gridDim.x * BPJ_NT, &p.flags[r + 1]);
+}
+
+// The rounds from r on in one block, until the list is empty; an exit still
+// open after round R - 1 lies on a cycle.
+__global__ void __launch_bounds__(BPJ_END) k_bpj_end(Pipe p, int r, int R) {
+  __shared__ uint32_t count;  // the next round's list
+  uint32_t n = p.flags[r];
+  for (; n && r < R; r++) {
+    if (threadIdx.x == 0) count = 0u;
+    __syncthreads();
+    bpj_round<BPJ_END>(p, r, n, 0u, BPJ_END, &count);
+    __syncthreads();  // the round's writes, before the next round's reads
+    n = count;
+    __syncthreads();
+  }
+  if (n && threadIdx.x == 0) set_status(p.status, D8_ERR_CYCLE);
 }
 
 // dw(q) = (in-tile path sum of q, already in dw) + H(exit of q); four
@@ -425,21 +479,29 @@ cudaError_t launch_bwd_up(const DemTable& dt, const Pipe& p, cudaStream_t s, int
 // Rounds R = rounds + 2: any chain of the exit forest closes within `rounds`
 // (2^rounds > slot count), and the copy round of the last exits to close
 // comes one round later, so the list of round R is empty unless a cycle holds
-// exits open.  Rounds after the list empties return at once.
+// exits open.  Rounds after the list empties return at once (the rounds that
+// few fields need are launched small: an empty one takes half as long); on grids of up to
+// END_SLOTS slots, whose lists one block gets through, the rounds that only
+// winding fields need (paths of tiles longer than twice the grid's side) are
+// left to one such block instead of a launch each.
+constexpr int64_t END_SLOTS = 1 << 16;
 template <int T>
 static cudaError_t launch_combine_bwd_t(const DemTable& dt, const Pipe& p, cudaStream_t s, int* nlaunch) {
   const int R = p.rounds + 2;
   if (R > MAX_ROUNDS + 1) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(p.flags, 0, sizeof(uint32_t) * (MAX_ROUNDS + 2), s);
   if (e != cudaSuccess) return e;
-  k_bpj_init<T><<<grid_for_b(p.nslots, 16), 256, 0, s>>>(dt, p);
+  const int64_t threads = (p.nslots + BPJ_U - 1) / BPJ_U;
+  k_bpj_init<T><<<grid_for_b(threads, 8), BPJ_NT, 0, s>>>(dt, p);
   ++*nlaunch;
-  const unsigned gr = grid_for_b((p.nslots + BPJ_U - 1) / BPJ_U, 4);
-  for (int r = 0; r < R; r++) {
-    k_bpj_round<<<gr, 256, 0, s>>>(p, r);
+  int ordinary = 2;  // rounds for paths of up to twice the side in tiles, and the copy round
+  while ((int64_t)1 << (ordinary - 2) < 2 * (dt.one.ntx > dt.one.nty ? dt.one.ntx : dt.one.nty)) ordinary++;
+  int r = 0;
+  for (; r < R && (p.nslots > END_SLOTS || r < ordinary); r++) {
+    k_bpj_round<<<grid_for_b(threads, r < ordinary ? 4 : 1), BPJ_NT, 0, s>>>(p, r);
     ++*nlaunch;
   }
-  k_bpj_check<<<1, 32, 0, s>>>(p, R);
+  k_bpj_end<<<1, BPJ_END, 0, s>>>(p, r, R);
   ++*nlaunch;
   return cudaGetLastError();
 }
