@@ -367,8 +367,8 @@ d8_status run_forward(d8_ctx* c, const DemDesc& d0, int mode, int rule, cudaStre
     e = launch_combine_hier(hp, s, &sc.n);
   }
   if (e != cudaSuccess) return cuda_fail(e);
-  p.recv = !weighted;
-  if (p.recv && hs.nlev == 0 && !hs.solve) p.S = nullptr;
+  p.recv = true;
+  if (hs.nlev == 0 && !hs.solve) p.S = nullptr;
   {
     StageScope sc(c, ST_DOWN, s);
     e = launch_down(dt, p, weighted, s, &sc.n);

@@ -43,7 +43,8 @@ struct GroupLayout {
   static constexpr size_t off_val = ((size_t)NS * 2 + 15) / 16 * 16;         // value
   static constexpr size_t off_pd = off_val + (size_t)NS * sizeof(V);         // u32 parent << 16 | children left
   static constexpr size_t off_src = off_pd + (size_t)NS * 4;                 // u16 source lists
-  static constexpr size_t off_misc = off_src + (size_t)NS * 2;
+  // (parents, counts and sources together also hold the receivers' inflow)
+  static constexpr size_t off_misc = off_pd + (size_t)NS * (sizeof(V) > 6 ? sizeof(V) : 6);
   static constexpr size_t bytes = off_misc + 64;
 };
 
@@ -336,22 +337,21 @@ __global__ void __launch_bounds__(NTG<S, G>) k_group_up(DemTable cdt, DemTable g
 
 // infl[n] = the sum of the final areas of the group's child exits that drain
 // into node n's cell
-template <int S, int G, int NT>
-__device__ __forceinline__ void receivers_inflow(const GroupGeo& g, const uint16_t* spx, const uint32_t* val,
-                                                 uint32_t* infl) {
+template <int S, int G, int NT, class V>
+__device__ __forceinline__ void receivers_inflow(const GroupGeo& g, const uint16_t* spx, const V* val, V* infl) {
   constexpr int NS = G * G * 4 * S;
-  for (int n = threadIdx.x; n < NS; n += NT) infl[n] = 0u;
+  for (int n = threadIdx.x; n < NS; n += NT) infl[n] = V{};
   __syncthreads();
   for (int n = threadIdx.x; n < NS; n += NT) {
     const uint16_t pe = spx[n];
     if (!(pe & PEX_EXIT)) continue;
     const int n2 = target_node<S, G>(g, n, pe);
-    if (n2 >= 0) atomicAdd(&infl[n2], val[n]);
+    if (n2 >= 0) vatomic_add(&infl[n2], val[n]);
   }
 }
 
-// The group's border inflow and its children's final values.  RECV (unit
-// counts, the children are tiles): cfin gets per slot not the exits' final
+// The group's border inflow and its children's final values.  RECV (the
+// children are tiles): cfin gets per slot not the exits' final
 // areas but the receivers' inflow, the sum of the final areas of the exits of
 // other tiles that drain into the slot's cell, which is what the finalising
 // pass needs (it then reads one contiguous row per tile; gathering the areas
@@ -421,11 +421,11 @@ __global__ void __launch_bounds__(NTG<S, G>) k_group_down(DemTable cdt, DemTable
     group_walk<S, G, NT, V>(spx, val, pd, srcl);
     __syncthreads();
     if constexpr (RECV) {
-      uint32_t* infl = pd;  // the walk is done with it
-      receivers_inflow<S, G, NT>(gg, spx, val, infl);
+      V* infl = reinterpret_cast<V*>(pd);  // the walk is done with it
+      receivers_inflow<S, G, NT, V>(gg, spx, val, infl);
 #pragma unroll 1
       for (int r = 0; r < NB; r++)
-        if (bslot[r] >= 0) atomicAdd(&infl[bslot[r]], bin[r]);
+        if (bslot[r] >= 0) vatomic_add(&infl[bslot[r]], bin[r]);
       __syncthreads();
     }
     for (int n = threadIdx.x; n < NS; n += NT) {
@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(NTG<S, G>) k_group_down(DemTable cdt, DemTable
       if (RECV && (cy >= cd.nty || cx >= cd.ntx)) continue;
       V* dst = cfin + (cd.tile_base + cy * cd.ntx + cx) * (4 * S) + s;
       if constexpr (RECV)
-        *dst = pd[n];
+        *dst = reinterpret_cast<const V*>(pd)[n];
       else
         *dst = val[n];
     }
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(NTS) k_group_solve(DemTable dt, const uint16_t
   atomicAdd(&misc[1], exits);
   __syncthreads();
   if (threadIdx.x == 0 && misc[0] != misc[1]) set_status(status, D8_ERR_CYCLE);
-  receivers_inflow<S, G, NTS>(gg, spx, val, pd);
+  receivers_inflow<S, G, NTS, uint32_t>(gg, spx, val, pd);
   __syncthreads();
   for (int n = threadIdx.x; n < L::NS; n += NTS) {
     const int lt = n / (4 * S), cy = lt / G, cx = lt % G;
@@ -838,8 +838,8 @@ static cudaError_t combine_hier_t(const HPlan& hp, cudaStream_t s, int* nlaunch)
     e = launch_top<512, V, V>(t.dt, t, hp.top, s, nlaunch);
     if (e != cudaSuccess) return e;
   }
-  // down: level l -> l-1 (at the tiles: unit counts leave the receivers' inflow)
-  constexpr bool RECV = std::is_same<V, uint32_t>::value;
+  // down: level l -> l-1 (at the tiles: the receivers' inflow)
+  constexpr bool RECV = true;
   for (int l = hp.nlev; l >= 1 && e == cudaSuccess; l--) {
     const HLevel& c = hp.lev[l - 1];
     const HLevel& g = hp.lev[l];

@@ -204,7 +204,7 @@ cudaError_t launch_inject_inflow(const DemDesc& d, const Pipe& p, cudaStream_t s
 cudaError_t launch_down(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s, int* nlaunch) {
   if (p.recv && !p.S && !p.top_in && !p.bot_in) return cudaSuccess;  // one tile: A is final
   ++*nlaunch;
-  return p.recv ? launch_down_count(dt, p, s) : launch_down_unit(dt, p, weighted, s);
+  return p.recv ? launch_down_recv(dt, p, weighted, s) : launch_down_unit(dt, p, s);
 }
 
 }  // namespace d8

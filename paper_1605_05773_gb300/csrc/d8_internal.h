@@ -61,7 +61,7 @@ struct Pipe {
   void* pval;        // per slot: in-tile area at exits (fwd) / path sum (bwd)
   uint32_t* P[2];    // flat combines (adjoint, allocation-free entry): pointer-jumping parents
   void* S;           // per slot, read by the finalising pass: final value at exits, or (recv) the receivers' inflow
-  bool recv;         // unit counts after the layered combine; S null: no inflow between tiles
+  bool recv;         // after the layered combine; S null: no inflow between tiles
   void* S2;          // flat combines: second value buffer (adjoint) / delta buffer (counts)
   uint32_t* flags;   // combine: per-round "still active" flags, MAX_ROUNDS+2
   uint32_t* status;  // device status word (OR of 1 << d8_status)
@@ -135,12 +135,12 @@ cudaError_t launch_combine_hier(const HPlan& hp, cudaStream_t s, int* nlaunch);
 
 // tile pass of unit counts, ring walks (d8_count.cu)
 cudaError_t launch_up_count(const DemTable& dt, const Pipe& p, cudaStream_t s);
-// finalise of unit counts from the receivers' inflow (d8_final.cu)
-cudaError_t launch_down_count(const DemTable& dt, const Pipe& p, cudaStream_t s);
+// finalise from the receivers' inflow (d8_final.cu)
+cudaError_t launch_down_recv(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s);
 // tile passes: unit counts of 128 x 128 tiles or with the lane-mask walk,
-// weighted; finalise, weighted or of unit counts from the exits' values (d8_unit.cu)
+// weighted; finalise of unit counts from the exits' values (d8_unit.cu)
 cudaError_t launch_up_unit(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s);
-cudaError_t launch_down_unit(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s);
+cudaError_t launch_down_unit(const DemTable& dt, const Pipe& p, cudaStream_t s);
 
 // ---- pit and flat removal (d8_fill.cu)
 size_t fill_ws_bytes(int64_t H, int64_t W);

@@ -1,6 +1,6 @@
 // d8_unit.cu -- tile passes: weighted areas, unit counts of 128 x 128 tiles and
 // under the lane-mask strategy (other unit counts: d8_count.cu), and the
-// finalising passes.
+// finalising pass of the allocation-free entry (others: d8_final.cu).
 //
 //  k_up_unit    per tile: codes from the direction field, the in-tile
 //               dependency count (Algorithm 1), the in-tile up-slope counts
@@ -9,10 +9,10 @@
 //               (A 128 x 128 tile's count and cell index do not fit one word
 //               of d8_count.cu.)
 //  k_up_lm      the same for unit counts with the lane-mask walk.
-//  k_fin_unit,  per tile finalise (Algorithms 7-8) from the exits' final
-//  k_fin_w      values: A already holds the in-tile counts or areas; the resolved inflow from neighbouring
-//               tiles is pushed down the in-tile paths it reaches and added
-//               there.
+//  k_fin_unit   per tile finalise (Algorithms 7-8) of unit counts from the
+//               exits' final values: A already holds the in-tile counts; the
+//               resolved inflow from neighbouring tiles is pushed down the
+//               in-tile paths it reaches and added there.
 //
 // Layout choices for GB300:
 //  * one packed 32-bit word per cell in shared memory holds the cell's
@@ -165,21 +165,6 @@ struct FinLayout {
   static constexpr size_t off_rcell = off_code + TT;     // uint16 per perimeter slot
   static constexpr size_t off_rin = off_rcell + (size_t)4 * T * 2;  // uint32 per slot
   static constexpr size_t off_ring = off_rin + (size_t)4 * T * 4;   // uint8 codes around the tile
-  static constexpr size_t off_misc = (off_ring + 2 * (T + 2) + 2 * T + 15) / 16 * 16;
-  static constexpr size_t bytes = off_misc + 64;
-};
-
-// finalising pass, weighted: the inflow routed through each cell as a
-// fixed-point number in three 32-bit words (FxLimbs; word 0 of every cell,
-// then word 1, then word 2)
-template <int T>
-struct FinWLayout {
-  static constexpr size_t TT = (size_t)T * T;
-  static constexpr size_t off_w = 0;                     // uint32 [3][TT]
-  static constexpr size_t off_code = TT * 12;            // uint8 code per cell
-  static constexpr size_t off_rcell = off_code + TT;     // uint16 per perimeter slot
-  static constexpr size_t off_rin = off_rcell + (size_t)4 * T * 2;  // ff per slot
-  static constexpr size_t off_ring = off_rin + (size_t)4 * T * sizeof(ff);  // uint8 codes around the tile
   static constexpr size_t off_misc = (off_ring + 2 * (T + 2) + 2 * T + 15) / 16 * 16;
   static constexpr size_t bytes = off_misc + 64;
 };
@@ -773,268 +758,6 @@ __global__ void __launch_bounds__(NTF, 8) k_fin_unit(DemTable dt, Pipe p) {
   }
 }
 
-// 96-bit two's-complement fixed point, three 32-bit words (w0 lowest).
-struct fx96 {
-  uint32_t w0, w1, w2;
-};
-
-// round(f * 2^q) (ties away from zero) for a finite f with |f| 2^q < 2^94
-__device__ __forceinline__ fx96 fx96_of(float f, int q) {
-  const uint32_t bits = __float_as_uint(f);
-  const int E = (int)((bits >> 23) & 0xFFu);
-  const uint32_t mant = (bits & 0x7FFFFFu) | (E ? 0x800000u : 0u);
-  const int s = (E ? E : 1) - 150 + q;  // f * 2^q = mant * 2^s
-  uint64_t lo = 0;
-  uint32_t hi = 0;
-  if (mant != 0u) {
-    if (s >= 64) {
-      hi = mant << (s - 64);
-    } else if (s >= 0) {
-      lo = (uint64_t)mant << s;
-      hi = s > 40 ? (uint32_t)(mant >> (64 - s)) : 0u;
-    } else if (s > -26) {
-      lo = ((uint64_t)mant + (1ull << (-s - 1))) >> (-s);
-    }
-  }
-  if (bits >> 31) {  // negate the 96-bit value
-    lo = ~lo + 1ull;
-    hi = ~hi + (lo == 0ull ? 1u : 0u);
-  }
-  return fx96{(uint32_t)lo, (uint32_t)(lo >> 32), hi};
-}
-
-__device__ __forceinline__ fx96 fx96_add(fx96 a, fx96 b) {
-  const uint64_t al = a.w0 | ((uint64_t)a.w1 << 32), bl = b.w0 | ((uint64_t)b.w1 << 32);
-  const uint64_t l = al + bl;
-  return fx96{(uint32_t)l, (uint32_t)(l >> 32), a.w2 + b.w2 + (l < al ? 1u : 0u)};
-}
-
-// The finalise's per-cell fixed-point accumulator: word 0 is the low 32 bits,
-// summed modulo 2^32 with the carry of each addition taken from the atomic's
-// reply; words 1 and 2 are limbs of LB bits (unsigned, then signed) summed
-// without carries, their spare bits absorbing up to 4T additions (one per
-// receiver).  A value x with |x| < 2^(32 + 2 LB) enters as x0 = x mod 2^32,
-// x1 = (x >> 32) mod 2^LB, x2 = x >> (32 + LB); the three words then hold the
-// exact sum as w0 + w1 2^32 + w2 2^(32 + LB), whatever the order.
-template <int T>
-struct FxLimbs {
-  static constexpr int LB = T >= 128 ? 22 : (T >= 64 ? 23 : 24);  // 4T (LB-bit limb + carry) sums < 2^31
-  static constexpr int VB = 32 + 2 * LB;                          // value bits, sign included
-};
-
-template <int T>
-__device__ __forceinline__ void fx_split(fx96 v, uint32_t& x0, uint32_t& x1, uint32_t& x2) {
-  constexpr int LB = FxLimbs<T>::LB;
-  const long long rest = (long long)(v.w1 | ((unsigned long long)v.w2 << 32));  // v >> 32, |rest| < 2^(2 LB)
-  x0 = v.w0;
-  x1 = (uint32_t)rest & ((1u << LB) - 1u);
-  x2 = (uint32_t)(int)(rest >> LB);
-}
-
-// the three words of a cell back to a 96-bit two's-complement value
-template <int T>
-__device__ __forceinline__ fx96 fx_join(uint32_t w0, uint32_t w1, uint32_t w2) {
-  constexpr int LB = FxLimbs<T>::LB;
-  const uint64_t lo = (uint64_t)w0 + ((uint64_t)w1 << 32);  // w1 < 2^31
-  const long long t = (long long)(int)w2;                  // signed sum of the top limbs
-  const uint64_t tl = (uint64_t)t << (32 + LB);
-  const fx96 a{(uint32_t)lo, (uint32_t)(lo >> 32), 0u};
-  const fx96 b{(uint32_t)tl, (uint32_t)(tl >> 32), (uint32_t)(t >> (32 - LB))};
-  return fx96_add(a, b);
-}
-
-// 2^k as fp32 for -126 <= k <= 127 (built from its exponent field: exact)
-__device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + k) << 23); }
-
-// The fixed-point value (w0, w1, w2) * 2^-q as float-float: the top 62 bits
-// of the magnitude rounded to fp32, plus their exact remainder rounded to
-// fp32 (a relative error of at most 2^-48 from the remainder's rounding and
-// 2^-61 from the bits below the top 62).  2^-q is passed as two powers of two
-// p1 * p2 of the normal range; each product below is exact until the last,
-// which rounds once.
-__device__ __forceinline__ ff fx96_to_ff(uint32_t w0, uint32_t w1, uint32_t w2, float p1, float p2) {
-  uint64_t lo = w0 | ((uint64_t)w1 << 32);
-  uint32_t hi = w2;
-  const bool neg = (hi >> 31) != 0u;
-  if (neg) {
-    lo = ~lo + 1ull;
-    hi = ~hi + (lo == 0ull ? 1u : 0u);
-  }
-  const int p = hi ? 95 - __clz(hi) : (lo ? 63 - __clzll(lo) : 0);  // leading bit
-  int sh = 0;
-  uint64_t U = lo;
-  if (p > 61) {
-    sh = p - 61;
-    U = (lo >> sh) | (hi ? ((uint64_t)hi << (64 - sh)) : 0ull);
-  }
-  const float fh = __ull2float_rn(U);  // U < 2^62 rounded to 24 bits: an integer
-  const float fl = __ll2float_rn((long long)(U - __float2ull_rn(fh)));
-  const float sc = pow2f(sh);  // sh <= 34
-  const ff r{__fmul_rn(__fmul_rn(__fmul_rn(fh, sc), p1), p2), __fmul_rn(__fmul_rn(__fmul_rn(fl, sc), p1), p2)};
-  return neg ? ff{-r.hi, -r.lo} : r;
-}
-
-// Algorithms 7-8 for weighted areas, on the same sub-forest and with the same
-// walks as the unit finalise.  The inflow is added in fixed point so that the
-// additions stay exact and commute: F(c) is an integer in units of 2^-q held
-// in three 32-bit words (FxLimbs: VB = 78 value bits for 64 x 64 tiles).  The
-// scale is set per tile from the receivers' inflows: with |in_r| < 2^e_r,
-// S = sum over receivers of 2^e_r (an exact integer sum of powers of two, so
-// the same in every run) bounds the sum of their magnitudes, and q makes
-// S * 2^q <= 2^(VB - 2), so that no partial sum reaches 2^(VB - 1) in
-// magnitude.  Each receiver's float-float inflow is rounded once to a
-// multiple of 2^-q, an error below 2^-q <= 2^-(VB - 4) * sum |in_r| (2^-74
-// for 64 x 64 tiles), far below fp32 resolution even when the tile's inflows
-// span twenty orders of magnitude; after that the sums are exact, so the
-// result does not depend on the schedule.  Finally A = fp32(A +
-// F), F converted to float-float.  A non-finite inflow (non-finite weights)
-// cannot be scaled: the tile keeps its in-tile areas and D8_ERR_NONFINITE is
-// raised.
-template <int T>
-__global__ void __launch_bounds__(NTF, T >= 64 ? 4 : 8) k_fin_w(DemTable dt, Pipe p) {
-  using L = FinWLayout<T>;
-  extern __shared__ __align__(16) unsigned char sm[];
-  uint32_t* F0 = reinterpret_cast<uint32_t*>(sm + L::off_w);  // words 0, 1, 2 at F0, F0 + TT, F0 + 2 TT
-  uint8_t* code = sm + L::off_code;
-  uint16_t* rcell = reinterpret_cast<uint16_t*>(sm + L::off_rcell);
-  ff* rin = reinterpret_cast<ff*>(sm + L::off_rin);
-  uint8_t* ring = sm + L::off_ring;
-  uint32_t* misc = reinterpret_cast<uint32_t*>(sm + L::off_misc);
-  const ff* xval = static_cast<const ff*>(p.S);
-  constexpr int TT = T * T;
-  constexpr int NQ = TT / 4 / NTF > 0 ? TT / 4 / NTF : 1;  // quads per thread in the write-back
-
-  // F starts at zero; every tile leaves the words it touched at zero again
-  for (int q = threadIdx.x; q < 3 * TT / 4; q += NTF) reinterpret_cast<uint4*>(F0)[q] = make_uint4(0, 0, 0, 0);
-  TileQueue tq(p.queue + 1, p.ntiles);
-  for (int64_t t = tq.first(); t < p.ntiles; t = tq.next()) {
-    const DemDesc d = dem_of(dt, t);
-    const TileGeo g = tile_geo(d, t - d.tile_base, T);
-    unsigned long long* S = reinterpret_cast<unsigned long long*>(misc + 2);
-    if (threadIdx.x == 0) {
-      misc[0] = 0;  // receivers
-      misc[1] = 0;  // largest exponent bound, + 1024
-      misc[4] = 0;  // a non-finite inflow seen
-      *S = 0ull;
-    }
-    fin_codes<T>(d, g, code, ring);
-    __syncthreads();
-    // |x| < 2^ebound(x) for finite x (subnormals and zero: 2^-126)
-    auto ebound = [](float x) -> int {
-      const int eb = (int)((__float_as_uint(x) >> 23) & 0xFFu);
-      return eb == 0 ? -126 : eb - 126;
-    };
-    // Algorithm 7: the receivers and their resolved inflow, listed
-    for (int s = threadIdx.x; s < 4 * T; s += NTF) {
-      int i, j;
-      if (!slot_cell(s, g.th, g.tw, T, i, j)) continue;
-      ff in{0.0f, 0.0f};
-      bool any = false;
-#pragma unroll
-      for (int k = 0; k < 8; k++) {
-        const int li = i + code_di(k), lj = j + code_dj(k);
-        if (li >= 0 && lj >= 0 && li < g.th && lj < g.tw) continue;
-        if (fin_ring_code<T>(ring, g, li, lj) != (uint32_t)opposite(k)) continue;  // also rejects cells off the grid
-        in = ff_add(in, xval[global_slot(d, g.i0 + li, g.j0 + lj, T)]);
-        any = true;
-      }
-      if (any) {
-        const int r = (int)atomicAdd(&misc[0], 1u);
-        rcell[r] = (uint16_t)(i * T + j);
-        rin[r] = in;
-        if (isfinite(in.hi))
-          atomicMax(&misc[1], (uint32_t)(ebound(in.hi) + 1024));
-        else
-          misc[4] = 1u;
-      }
-    }
-    __syncthreads();
-    const int nrec = (int)misc[0];
-    if (misc[4]) {  // an infinite or NaN inflow
-      if (threadIdx.x == 0) set_status(p.status, D8_ERR_NONFINITE);
-      __syncthreads();  // misc is reset by the next tile
-      continue;
-    }
-    if (nrec == 0) {  // no inflow: A is final
-      __syncthreads();
-      continue;
-    }
-    // S = sum of 2^(e_r - emax + 40), each term rounded up to at least 1
-    const int emax = (int)misc[1] - 1024;
-    for (int r = threadIdx.x; r < nrec; r += NTF) {
-      const int sh = ebound(rin[r].hi) - emax + 40;
-      atomicAdd(S, sh <= 0 ? 1ull : 1ull << sh);
-    }
-    __syncthreads();
-    // sum |in_r| < S * 2^(emax - 40) <= 2^(ceil(log2 S) + emax - 40)
-    const int q = FxLimbs<T>::VB - 2 - (64 - __clzll(*S - 1ull)) - (emax - 40);
-    // 2^-q as two powers of two of the normal range (|q| <= 250: -126 <= emax <= 128)
-    const float p1 = pow2f(-q / 2), p2 = pow2f(-q - (-q / 2));
-    // Algorithm 8 on the receivers' paths, in fixed point
-    for (int r = threadIdx.x; r < nrec; r += NTF) {
-      const ff in = rin[r];
-      uint32_t x0, x1, x2;
-      fx_split<T>(fx96_add(fx96_of(in.hi, q), fx96_of(in.lo, q)), x0, x1, x2);
-      int c = rcell[r], i = c / T, j = c & (T - 1);
-      for (int step = 0; step <= TT; step++) {
-        const uint32_t o0 = atomicAdd(F0 + c, x0);
-        const int k = code[c];  // the walk goes on while the reply is in flight
-        const uint32_t up = x1 + ((o0 + x0 < o0) ? 1u : 0u);
-        if (up) atomicAdd(F0 + TT + c, up);
-        if (x2) atomicAdd(F0 + 2 * TT + c, x2);
-        if (k >= 8) break;
-        i += code_di(k);
-        j += code_dj(k);
-        if ((unsigned)i >= (unsigned)g.th || (unsigned)j >= (unsigned)g.tw) break;
-        c = i * T + j;
-      }
-    }
-    __syncthreads();
-    // A = fp32(A + F) where F is non-zero; those words go back to zero
-#pragma unroll
-    for (int rr = 0; rr < NQ; rr++) {
-      const int qd = threadIdx.x + rr * NTF;
-      const uint4 a4 = reinterpret_cast<const uint4*>(F0)[qd];
-      const uint4 b4 = reinterpret_cast<const uint4*>(F0 + TT)[qd];
-      const uint4 c4 = reinterpret_cast<const uint4*>(F0 + 2 * TT)[qd];
-      if (!(a4.x | a4.y | a4.z | a4.w | b4.x | b4.y | b4.z | b4.w | c4.x | c4.y | c4.z | c4.w)) continue;
-      reinterpret_cast<uint4*>(F0)[qd] = make_uint4(0, 0, 0, 0);
-      reinterpret_cast<uint4*>(F0 + TT)[qd] = make_uint4(0, 0, 0, 0);
-      reinterpret_cast<uint4*>(F0 + 2 * TT)[qd] = make_uint4(0, 0, 0, 0);
-      const int c = qd * 4, i = c / T, j = c - i * T;
-      if (i >= g.th) continue;
-      const uint32_t w0[4] = {a4.x, a4.y, a4.z, a4.w}, w1[4] = {b4.x, b4.y, b4.z, b4.w},
-                     w2[4] = {c4.x, c4.y, c4.z, c4.w};
-      ff f[4];
-      bool on[4];
-#pragma unroll
-      for (int k = 0; k < 4; k++) {
-        const fx96 v = fx_join<T>(w0[k], w1[k], w2[k]);
-        on[k] = (v.w0 | v.w1 | v.w2) != 0u;
-        f[k] = on[k] ? fx96_to_ff(v.w0, v.w1, v.w2, p1, p2) : ff{0.0f, 0.0f};
-      }
-      float* dst = static_cast<float*>(d.A) + (g.i0 + i) * d.ldA + (g.j0 + j);
-      if (g.tw == T && ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0)) {
-        float4 a = *reinterpret_cast<float4*>(dst);
-        float* av = reinterpret_cast<float*>(&a);
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-          const ff r = ff_add(ff{av[k], 0.0f}, f[k]);
-          if (on[k]) av[k] = __fadd_rn(r.hi, r.lo);
-        }
-        *reinterpret_cast<float4*>(dst) = a;
-      } else {
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-          if (j + k >= g.tw || !on[k]) continue;
-          const ff r = ff_add(ff{dst[k], 0.0f}, f[k]);
-          dst[k] = __fadd_rn(r.hi, r.lo);
-        }
-      }
-    }
-  }
-}
-
 template <class K>
 static unsigned persistent_grid_u(K kernel, int threads, size_t smem, int64_t ntiles) {
   int dev = 0, sms = 1, per_sm = 0;
@@ -1063,17 +786,12 @@ static cudaError_t launch_up_unit_t(const DemTable& dt, const Pipe& p, cudaStrea
   return cudaGetLastError();
 }
 
-template <int T, bool WT>
+template <int T>
 static cudaError_t launch_down_unit_t(const DemTable& dt, const Pipe& p, cudaStream_t s) {
-  const size_t bytes = WT ? FinWLayout<T>::bytes : FinLayout<T>::bytes;
-  void (*k)(DemTable, Pipe);
-  if constexpr (WT)
-    k = k_fin_w<T>;
-  else
-    k = k_fin_unit<T>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  const size_t bytes = FinLayout<T>::bytes;
+  cudaError_t e = cudaFuncSetAttribute(k_fin_unit<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
-  k<<<persistent_grid_u(k, NTF, bytes, p.ntiles), NTF, bytes, s>>>(dt, p);
+  k_fin_unit<T><<<persistent_grid_u(k_fin_unit<T>, NTF, bytes, p.ntiles), NTF, bytes, s>>>(dt, p);
   return cudaGetLastError();
 }
 
@@ -1092,14 +810,8 @@ cudaError_t launch_up_unit(const DemTable& dt, const Pipe& p, bool weighted, cud
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_down_unit(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s) {
-  if (!weighted) return p.T == 64 ? unit::launch_down_unit_t<64, false>(dt, p, s) : cudaErrorInvalidValue;
-  switch (p.T) {
-    case 32: return unit::launch_down_unit_t<32, true>(dt, p, s);
-    case 64: return unit::launch_down_unit_t<64, true>(dt, p, s);
-    case 128: return unit::launch_down_unit_t<128, true>(dt, p, s);
-  }
-  return cudaErrorInvalidValue;
+cudaError_t launch_down_unit(const DemTable& dt, const Pipe& p, cudaStream_t s) {
+  return p.T == 64 ? unit::launch_down_unit_t<64>(dt, p, s) : cudaErrorInvalidValue;
 }
 
 }  // namespace d8
