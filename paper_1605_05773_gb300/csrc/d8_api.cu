@@ -213,8 +213,8 @@ size_t hier_bytes(const HShape& hs, size_t vb) {
     b += align256(ns * 2) + 2 * align256(ns * vb);
   }
   const size_t nt = (size_t)hs.nunits[hs.nlev] * 4 * hs.S[hs.nlev];
-  // par, par2, list; children counts or additions (8 B); round flags
-  if (hs.need_top) b += 3 * align256(nt * 4) + align256(nt * 8) + align256(sizeof(uint32_t) * (MAX_ROUNDS + 2));
+  // par, par2, list; node words (8 B) or two rounds' additions; round flags
+  if (hs.need_top) b += 3 * align256(nt * 4) + align256(nt * 2 * vb) + align256(sizeof(uint32_t) * (MAX_ROUNDS + 2));
   b += align256(sizeof(uint32_t) * 64);
   return b;
 }
@@ -267,7 +267,7 @@ HPlan carve_hier(void* base, const HShape& hs, const Pipe& p, const DemTable* dt
     hp.top.par2 = reinterpret_cast<uint32_t*>(q);
     q += align256(nt * 4);
     hp.top.node = reinterpret_cast<unsigned long long*>(q);
-    q += align256(nt * 8);
+    q += align256(nt * 2 * vb);
     hp.top.list = reinterpret_cast<uint32_t*>(q);
     q += align256(nt * 4);
     hp.top.flags = reinterpret_cast<uint32_t*>(q);

@@ -111,7 +111,7 @@ struct HTop {  // the top level's solve in global memory (queue method or pointe
   uint32_t* par2;  // pointer jumping: the second parent buffer
   uint32_t* flags; // pointer jumping: per-round "still active" flags (MAX_ROUNDS + 2)
   unsigned long long* node;  // per slot: children counts and, unit counts, the value (k_top_init);
-                             // pointer jumping: this round's additions (value type)
+                             // pointer jumping: two rounds' additions (value type)
   uint32_t* list;      // pointer jumping: the exits
   uint32_t* counters;  // pointer jumping: [0] exits; queue walk: [1] exits, [2] finished
   uint32_t* status;
