@@ -38,15 +38,14 @@
 namespace d8 {
 namespace count {
 
-// 64 threads, 12 tiles per SM: 262 us; 128 threads, 8 tiles: 320 (two more
-// warps wait out the last walks)
-constexpr int NTC = 64;  // threads per tile block
-constexpr int NW = NTC / 32;
+// NT, the threads of a tile's block, is 64 with 12 tiles per SM: 262 us at 8192
+// x 8192; 128 threads, 8 tiles: 320 (two more warps wait out the last walks).
+// Few tiles: see launch_t.
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int STEPS = 4;   // cells a walk advances per batch (3: 274 us, 6: 276, 4: 271 at the time)
 constexpr int SWEEP = 4;   // rows of the block's cells swept at once (1: 309 us, 2: 297, 4: 293 at the time)
 // walks on a warp's stack: 31 and a sweep's, or what all warps leave over
-constexpr int CAP = 32 * (1 + SWEEP > NW ? 1 + SWEEP : NW);
+constexpr int cap(int warps) { return 32 * (1 + SWEEP > warps ? 1 + SWEEP : warps); }
 
 // Where cell (i, j) of a tile is stored: within its row by (column mod 4,
 // column / 4), rows rotated among the bank groups, so that the cells k of 32
@@ -81,8 +80,9 @@ struct Cell {
   __device__ static __forceinline__ int code(uint32_t w) { return (int)((w >> 2) & 0xFu); }  // cells that are not IN
 };
 
-template <int T>
+template <int T, int NT>
 struct Layout {
+  static constexpr int NW = NT / 32, CAP = cap(NW);
   static constexpr size_t TT = (size_t)T * T;
   static constexpr size_t off_word = 0;                         // uint32 per cell
   static constexpr size_t off_spare = TT * 4;                   // uint32 [32], right after word: see spare()
@@ -100,7 +100,7 @@ __device__ __forceinline__ uint32_t& at(uint32_t* word, uint32_t o) {
 // instructions than the step).
 template <int T>
 __device__ __forceinline__ uint32_t spare() {
-  return (uint32_t)(Layout<T>::off_spare + 4 * (threadIdx.x & 31));
+  return (uint32_t)(T * T * 4 + 4 * (threadIdx.x & 31));
 }
 
 // Bits of the neighbours of tile cell (i, j) that lie outside a th x tw tile.
@@ -154,10 +154,10 @@ struct Table {
   // entry of column 0 of a group, in units of 8 bytes (columns follow)
   __device__ static __forceinline__ int of(int rk, int ck, int rc) { return ((rk * 3 + ck) * CLASSES + rc) * 4; }
 };
-template <int T>
+template <int T, int NT>
 __device__ __forceinline__ void fill_table(int8_t* tab) {
   using P = Place<T>;
-  for (int e = threadIdx.x; e < Table<T>::BYTES; e += NTC) {
+  for (int e = threadIdx.x; e < Table<T>::BYTES; e += NT) {
     const int code = e & 7, k = (e / 8) & 3, rc = (e / 32) & P::RM, ck = e / (32 * (P::RM + 1)) % 3,
               rk = e / (32 * (P::RM + 1)) / 3;
     const int i = rc + P::RM + 1, j = 4 + k;  // any cell of that class away from the tile's edge
@@ -181,11 +181,11 @@ __device__ __forceinline__ int signed_byte(uint2 v, uint32_t k) {
 // address are read as the aligned words that cover them and shifted into place
 // when they are used; the word after a row's last group is held by the lane of
 // that row's number among the thread's.  (Ragged tiles read theirs later.)
-template <int T>
+template <int T, int NT>
 struct Codes {
   static constexpr int Q = Place<T>::Q;
-  static constexpr int NQ = T * T / 4 / NTC;  // four-cell groups per thread
-  static constexpr int RS = NTC / Q;          // rows from one group of a thread to its next
+  static constexpr int NQ = T * T / 4 / NT;  // four-cell groups per thread
+  static constexpr int RS = NT / Q;          // rows from one group of a thread to its next
   static_assert(NQ <= Q, "a lane per row for the words after the rows");
   uint32_t word[NQ], after;
   __device__ static __forceinline__ int row0() { return threadIdx.x / Q; }
@@ -225,13 +225,13 @@ struct Codes {
 };
 
 // The words of tile g (zeroed before) from its codes: Algorithm 1.
-template <int T>
-__device__ __forceinline__ void set_words(const Codes<T>& codes, const DemDesc& d, const TileGeo& g, uint32_t* word,
+template <int T, int NT>
+__device__ __forceinline__ void set_words(const Codes<T, NT>& codes, const DemDesc& d, const TileGeo& g, uint32_t* word,
                                           const uint2* tab, uint32_t* status) {
   using P = Place<T>;
   using C = Cell<T>;
-  constexpr int NQ = Codes<T>::NQ, RS = Codes<T>::RS;
-  const int i0 = Codes<T>::row0(), q = Codes<T>::group();
+  constexpr int NQ = Codes<T, NT>::NQ, RS = Codes<T, NT>::RS;
+  const int i0 = Codes<T, NT>::row0(), q = Codes<T, NT>::group();
   if (g.th == T && g.tw == T) {
     // whole tiles: the tables give the places of the targets inside the tile
     const int ck = q == 0 ? 0 : (q == P::Q - 1 ? 2 : 1), rc = i0 & P::RM;
@@ -268,16 +268,16 @@ __device__ __forceinline__ void set_words(const Codes<T>& codes, const DemDesc& 
   }
   constexpr int U = 16;  // codes read at once
 #pragma unroll 1
-  for (int c0 = threadIdx.x; c0 < T * T; c0 += U * NTC) {
+  for (int c0 = threadIdx.x; c0 < T * T; c0 += U * NT) {
     uint8_t code[U];
 #pragma unroll
     for (int u = 0; u < U; u++) {
-      const int c = c0 + u * NTC, i = c / T, j = c % T;
+      const int c = c0 + u * NT, i = c / T, j = c % T;
       code[u] = i < g.th && j < g.tw ? __ldg(d.dir + (g.i0 + i) * d.lddir + (g.j0 + j)) : (uint8_t)0;
     }
 #pragma unroll
     for (int u = 0; u < U; u++) {
-      const int c = c0 + u * NTC, i = c / T, j = c % T;
+      const int c = c0 + u * NT, i = c / T, j = c % T;
       if (i < g.th && j < g.tw) add_cell<T>(word, i, j, code[u], g, d, status);
     }
   }
@@ -285,11 +285,11 @@ __device__ __forceinline__ void set_words(const Codes<T>& codes, const DemDesc& 
 
 // At the grid's edge a target off the grid is a path end, not an exit (whole
 // tiles; set_words took every target outside the tile for an exit).
-template <int T>
+template <int T, int NT>
 __device__ __forceinline__ void end_at_grid_edge(const DemDesc& d, const TileGeo& g, uint32_t* word) {
   using C = Cell<T>;
   if (g.th != T || g.tw != T || (g.i0 > 0 && g.j0 > 0 && g.i0 + T < d.H && g.j0 + T < d.W)) return;
-  for (int s = threadIdx.x; s < 4 * T; s += NTC) {
+  for (int s = threadIdx.x; s < 4 * T; s += NT) {
     int i, j;
     if (!slot_cell(s, T, T, T, i, j)) continue;
     uint32_t* w = &word[Place<T>::of(i, j)];
@@ -303,14 +303,14 @@ __device__ __forceinline__ void end_at_grid_edge(const DemDesc& d, const TileGeo
 // A[tile] = the in-tile counts: four consecutive cells per thread in one 16-byte
 // store when the layout allows, else one.  Returns whether one of this thread's
 // cells still waits for an input: it lies on or below a cycle.
-template <int T>
+template <int T, int NT>
 __device__ __forceinline__ bool store_counts(const DemDesc& d, const TileGeo& g, const uint32_t* word) {
   using P = Place<T>;
   using C = Cell<T>;
   uint32_t left = 0;
   const bool vec = g.tw == T && g.th == T && ((reinterpret_cast<uintptr_t>(d.A) & 15u) == 0) && (d.ldA & 3) == 0;
   if (vec) {
-    constexpr int RS = NTC / P::Q;  // rows from one group of a thread to its next
+    constexpr int RS = NT / P::Q;  // rows from one group of a thread to its next
     const int i0 = threadIdx.x / P::Q, j = 4 * (threadIdx.x & (P::Q - 1));
     uint32_t* dst = static_cast<uint32_t*>(d.A) + (g.i0 + i0) * d.ldA + (g.j0 + j);
     const uint32_t* w0[4];
@@ -328,7 +328,7 @@ __device__ __forceinline__ bool store_counts(const DemDesc& d, const TileGeo& g,
     }
   } else {
     // consecutive lanes store consecutive columns
-    constexpr int RS = NTC / T;  // rows at once
+    constexpr int RS = NT / T;  // rows at once
     const int i0 = threadIdx.x / T, j = threadIdx.x % T;
     uint32_t* dst = static_cast<uint32_t*>(d.A) + (g.i0 + i0) * d.ldA + (g.j0 + j);
     if (j < g.tw) {
@@ -347,12 +347,12 @@ __device__ __forceinline__ bool store_counts(const DemDesc& d, const TileGeo& g,
 // Perimeter summary of a finished tile: for each perimeter slot, the exit of
 // the cell's in-tile path (Algorithms 3-4 seen from the exit side) found by
 // following links, and the in-tile count at the slot.
-template <int T>
+template <int T, int NT>
 __device__ __forceinline__ void perimeter_summary(const TileGeo& g, int64_t t, uint32_t* word, bool cyc,
                                                   const Pipe& p) {
   using P = Place<T>;
   using C = Cell<T>;
-  constexpr int N = 4 * T / NTC;  // slots per thread, followed side by side
+  constexpr int N = 4 * T / NT;  // slots per thread, followed side by side
   uint16_t* pex = p.pex + t * (4 * T);
   uint32_t* pval = static_cast<uint32_t*>(p.pval) + t * (4 * T);
   uint32_t w[N], o[N], v[N];
@@ -361,12 +361,12 @@ __device__ __forceinline__ void perimeter_summary(const TileGeo& g, int64_t t, u
     int i, j;
     w[r] = 0u;
     o[r] = 0u;
-    if (slot_cell(threadIdx.x + r * NTC, g.th, g.tw, T, i, j)) {
+    if (slot_cell(threadIdx.x + r * NT, g.th, g.tw, T, i, j)) {
       o[r] = 4u * (uint32_t)P::of(i, j);
       w[r] = at(word, o[r]);
     }
     v[r] = cyc ? 0u : w[r];
-    pval[threadIdx.x + r * NTC] = w[r] >> C::CB;
+    pval[threadIdx.x + r * NT] = w[r] >> C::CB;
   }
   for (int guard = 0; guard < 2 * T * T; guard++) {
     uint32_t any = 0;
@@ -387,7 +387,7 @@ __device__ __forceinline__ void perimeter_summary(const TileGeo& g, int64_t t, u
       pe = (uint16_t)(PEX_EXIT | C::code(w[r]));
     else if ((w[r] & IN) && (v[r] & (IN | EXIT)) == EXIT)
       pe = (uint16_t)slot_of(P::row(o[r] >> 2), P::column(o[r] >> 2), g.th, g.tw, T);
-    pex[threadIdx.x + r * NTC] = pe;
+    pex[threadIdx.x + r * NT] = pe;
   }
 }
 
@@ -449,11 +449,11 @@ __device__ __forceinline__ void finish(uint32_t o, bool on, uint32_t* word) {
   if (on && o != start) at(word, start) = (at(word, start) & ~C::LINK) | o;
 }
 
-template <int T>
-__global__ void __launch_bounds__(NTC, 12) k_up_count(DemTable dt, Pipe p) {
-  using L = Layout<T>;
+template <int T, int NT>
+__global__ void __launch_bounds__(NT, NT <= 64 ? 12 : 4) k_up_count(DemTable dt, Pipe p) {
+  using L = Layout<T, NT>;
   using C = Cell<T>;
-  constexpr int TT = T * T, ROWS = TT / NTC;
+  constexpr int TT = T * T, ROWS = TT / NT, NW = L::NW, CAP = L::CAP;
   extern __shared__ __align__(16) unsigned char sm[];
   uint32_t* word = reinterpret_cast<uint32_t*>(sm + L::off_word);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -463,10 +463,10 @@ __global__ void __launch_bounds__(NTC, 12) k_up_count(DemTable dt, Pipe p) {
   uint32_t* misc = reinterpret_cast<uint32_t*>(sm + L::off_misc);  // pooled walks, warps done, next tile
   const unsigned lt = (1u << lane) - 1u;
 
-  fill_table<T>(reinterpret_cast<int8_t*>(sm + L::off_tab));
+  fill_table<T, NT>(reinterpret_cast<int8_t*>(sm + L::off_tab));
   // Block b starts with tile b, later ones come from the queue, one ahead:
   // the next tile's codes are requested before this one's walks.
-  Codes<T> codes;
+  Codes<T, NT> codes;
   int64_t t = blockIdx.x;
   if (t < p.ntiles) {
     const DemDesc d = dem_of(dt, t);
@@ -477,16 +477,16 @@ __global__ void __launch_bounds__(NTC, 12) k_up_count(DemTable dt, Pipe p) {
     const TileGeo g = tile_geo(d, t - d.tile_base, T);
     __syncthreads();  // everyone is done with the tile before
     uint4* w4 = reinterpret_cast<uint4*>(word);
-    for (int c = threadIdx.x; c < TT / 4; c += NTC) w4[c] = make_uint4(0, 0, 0, 0);
+    for (int c = threadIdx.x; c < TT / 4; c += NT) w4[c] = make_uint4(0, 0, 0, 0);
     if (threadIdx.x == 0) {
       misc[0] = misc[1] = 0;
       misc[2] = gridDim.x + atomicAdd(p.queue, 1u);
     }
     __syncthreads();
     codes.shift(d, g);
-    set_words<T>(codes, d, g, word, tab, p.status);
+    set_words<T, NT>(codes, d, g, word, tab, p.status);
     __syncthreads();
-    end_at_grid_edge<T>(d, g, word);  // (only the summary reads what it changes)
+    end_at_grid_edge<T, NT>(d, g, word);  // (only the summary reads what it changes)
     next = misc[2];
     if (next < p.ntiles) {
       const DemDesc dn = dem_of(dt, next);
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(NTC, 12) k_up_count(DemTable dt, Pipe p) {
         bool ready[SWEEP];
 #pragma unroll
         for (int u = 0; u < SWEEP; u++) {
-          const uint32_t w = word[threadIdx.x + (r + u) * NTC];
+          const uint32_t w = word[threadIdx.x + (r + u) * NT];
           const bool src = (w & (~(C::ONE - 1u) | IN)) == (C::ONE | IN);  // with a target in the tile
           s[u] = src ? w & C::LINK : spare<T>();
           const uint32_t old = atomicAdd(&at(word, s[u]), C::ONE - LEFT1);
@@ -549,28 +549,47 @@ __global__ void __launch_bounds__(NTC, 12) k_up_count(DemTable dt, Pipe p) {
     }
     if (alone) finish<T>(lane < n ? *(volatile uint16_t*)&stack[lane] : spare<T>(), lane < n, word);
     __syncthreads();
-    const bool cyc = __syncthreads_or(store_counts<T>(d, g, word));
+    const bool cyc = __syncthreads_or(store_counts<T, NT>(d, g, word));
     if (threadIdx.x == 0 && cyc) set_status(p.status, D8_ERR_CYCLE);
-    perimeter_summary<T>(g, t, word, cyc, p);
+    perimeter_summary<T, NT>(g, t, word, cyc, p);
   }
 }
 
-template <int T>
-static cudaError_t launch_t(const DemTable& dt, const Pipe& p, cudaStream_t s) {
-  constexpr size_t bytes = Layout<T>::bytes;
-  auto k = k_up_count<T>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
+// Blocks of kernel k that run at once on the device.
+template <class K>
+static int64_t resident(K k, int threads, size_t bytes) {
   int dev = 0, sms = 1, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NTC, bytes) != cudaSuccess || per_sm < 1) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, bytes) != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
     per_sm = 1;
   }
-  const int64_t grid = min64((int64_t)per_sm * sms, p.ntiles);
-  k<<<(unsigned)(grid < 1 ? 1 : grid), NTC, bytes, s>>>(dt, p);
+  return (int64_t)per_sm * sms;
+}
+
+template <int T, int NT>
+static cudaError_t launch_nt(const DemTable& dt, const Pipe& p, int64_t at_once, cudaStream_t s) {
+  const int64_t grid = min64(at_once, p.ntiles);
+  k_up_count<T, NT><<<(unsigned)(grid < 1 ? 1 : grid), NT, Layout<T, NT>::bytes, s>>>(dt, p);
   return cudaGetLastError();
+}
+
+// Wide blocks where all tiles are under way at once: a tile's own latency is
+// what the pass takes then.  512 x 512 (64 tiles): 17 us, 27 in blocks of 64
+// threads; 576 tiles: 25 and 29; 676, more than the 608 wide blocks that fit at
+// once: 33 and 30.  32 x 32 tiles, 256 of them: 12.8 and 15.8.
+template <int T>
+static cudaError_t launch_t(const DemTable& dt, const Pipe& p, cudaStream_t s) {
+  constexpr int WIDE = 4 * T, NT = 64;
+  cudaError_t e = cudaFuncSetAttribute(k_up_count<T, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)Layout<T, WIDE>::bytes);
+  if (e != cudaSuccess) return e;
+  const int64_t wide = resident(k_up_count<T, WIDE>, WIDE, Layout<T, WIDE>::bytes);
+  if (p.ntiles <= wide) return launch_nt<T, WIDE>(dt, p, wide, s);
+  e = cudaFuncSetAttribute(k_up_count<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Layout<T, NT>::bytes);
+  if (e != cudaSuccess) return e;
+  return launch_nt<T, NT>(dt, p, resident(k_up_count<T, NT>, NT, Layout<T, NT>::bytes), s);
 }
 
 }  // namespace count
