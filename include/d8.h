@@ -173,7 +173,7 @@ d8_status d8_accumulate_backward(d8_ctx* ctx, const uint8_t* dir, int64_t H, int
  * the filled surface's dependencies wind across the 64 x 64 tiles).
  * Non-finite z sets D8_ERR_NONFINITE in the status word (F is then
  * unspecified).  The call synchronises `stream` (it checks for convergence
- * on the host after 8 rounds, then every 16).
+ * on the host every 8 rounds).
  * Errors: D8_ERR_ARG, D8_ERR_NOMEM, D8_ERR_CUDA, D8_ERR_TIMEOUT (not settled
  * after 2^20 rounds). */
 d8_status d8_fill(d8_ctx* ctx, const float* z, int64_t H, int64_t W, int64_t ldz, float eps, float* F,

@@ -16,8 +16,11 @@
 // one-cell halo, into shared memory and relaxes the tile to a fixed point of
 // that halo in directional passes (thread r walks row r left to right, then
 // right to left, then column r down and up; a pass carries a change across
-// the whole tile).  Every pass evaluates every cell, so the first pass that
-// changes nothing ends the visit.  Then the tile is written back, and a
+// the whole tile).  Every pass evaluates every cell, so a pass that changes
+// nothing ends the visit; so does the fourth, and the tile is then listed for
+// the next round itself.  (A change has crossed the tile by then: going on to
+// the fixed point, 10 to 12 passes, makes the neighbours wait for work that
+// their own changes undo again.)  Then the tile is written back, and a
 // neighbouring tile is listed for the next round if one of its cells beside
 // this tile would drop under this tile's new border.  A round that lists
 // nothing ends the fill: every tile is then at a fixed point of its final
@@ -36,8 +39,10 @@
 // coarse grids get a fixed number of rounds and no host check; each level
 // starts from the bounds of the level above it.
 //
-// Measured: 8192 x 8192 raw fractal 5.9 ms, 8192 x 8192 noisy plane 1.16 ms,
-// 700 x 933 fractal 0.42 ms; without the coarse levels 6.5, 3.2 and 0.45 ms
+// Measured: 8192 x 8192 raw fractal 5.1 ms, 8192 x 8192 noisy plane 1.09 ms,
+// 700 x 933 fractal 0.36 ms (visits to the fixed point 5.9, 1.12 and 0.40
+// ms; at most 3 passes 5.5 and 0.45, 5 passes 5.5 and 0.37); without the coarse
+// levels too 6.5, 3.2 and 0.45 ms
 // (the fractal's lakes, thousands of cells wide, still fill one tile a round);
 // before (256 threads per tile, two waves over dirty cells, then sweeps of
 // four passes until a whole sweep changed nothing; lanes down a row shared
@@ -56,7 +61,7 @@ constexpr int RATIO = 4;                // side ratio of a level to the next fin
 constexpr int NTF = T;                  // one thread per row, or column, of the tile
 constexpr int HW = T + 2;               // rows and columns of a tile with its halo
 constexpr int RS = T + 3;               // row stride of those arrays: odd, so lanes down a column hit distinct banks
-constexpr int MAX_PASSES = 16 * T;      // passes before a visit gives up and lists its own tile again
+constexpr int MAX_PASSES = 4;           // passes before a visit ends and lists its own tile again
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
 struct Layout {
@@ -329,8 +334,7 @@ __global__ void __launch_bounds__(NTF) k_fill_round(const float* z, int64_t H, i
 
 namespace fill {
 
-constexpr int CHUNK = 16;     // rounds between host checks, at most
-constexpr int FIRST = 8;      // rounds before the first check
+constexpr int CHUNK = 8;      // rounds launched at once: between host checks, and at most on a coarse grid
 constexpr int MAX_LEVELS = 8;
 constexpr size_t HEAD = 256;  // bytes of a level's counts (CHUNK + 1) and work queues (CHUNK)
 static_assert(RATIO == 4, "k_fill_init and k_fill_pool move blocks' rows as float4");
@@ -353,8 +357,9 @@ static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Levels are added while the last one has more than one tile, for grids of
 // more than 8 tiles a side: smaller ones settle in about as many rounds as the
-// coarse grids would take (500 x 500: 343 us without levels, 400 with; 700 x
-// 933: 452 and 434; 3000 x 3000: 1464 and 934).  Returns their number; bytes: the workspace.
+// coarse grids would take (when visits went to the fixed point, 500
+// x 500: 343 us without levels, 400 with; 700 x 933: 452 and 434; 3000 x 3000:
+// 1464 and 934).  Returns their number; bytes: the workspace.
 // What must be zero at the start comes first, `zeroed` bytes of it.
 static int levels(int64_t H, int64_t W, void* ws, Level* lv, size_t* zeroed, size_t* bytes) {
   int n = 0;
@@ -489,10 +494,10 @@ cudaError_t run_fill(const float* z, int64_t H, int64_t W, int64_t ldz, float ep
   if (e != cudaSuccess) return e;
   int64_t r = 0;
   for (;;) {
-    const int m = r == 0 ? FIRST : CHUNK;
+    constexpr int m = CHUNK;
     e = rounds(G, CellRaise{eps}, r, m, sms, s, nlaunch);
     r += m;
-    uint32_t h[CHUNK + 1];
+    uint32_t h[m + 1];
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, G.counts, sizeof(uint32_t) * (m + 1), cudaMemcpyDeviceToHost, s);
     // the last count is the next chunk's first
     if (e == cudaSuccess) e = cudaMemcpyAsync(G.counts, G.counts + m, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
