@@ -12,7 +12,7 @@
 // neighbour's older (higher) value can only delay, never spoil, the result.
 //
 // GPU layout: 64 x 64 tiles.  A round visits the tiles listed for it: a block
-// of 64 threads loads the tile's z and the current F of the tile, each with a
+// loads the tile's z and the current F of the tile, each with a
 // one-cell halo, into shared memory and relaxes the tile to a fixed point of
 // that halo in directional passes (thread r walks row r left to right, then
 // right to left, then column r down and up; a pass carries a change across
@@ -25,6 +25,10 @@
 // this tile would drop under this tile's new border.  A round that lists
 // nothing ends the fill: every tile is then at a fixed point of its final
 // halo, so F is the global fixed point.
+// A visit is a chain of latencies, 64 steps a pass; the other threads of its
+// block only share in loading, storing and looking at the border, whose loops
+// would add half of the passes' time (64 threads: 8192 x 8192 5.14 ms, 700 x
+// 933 358 us; 128: 4.71 and 314; 256: 4.58 and 293).
 //
 // Start from above: the fixed point is reached from any start that is nowhere
 // below it, and the nearer the start, the fewer visits.  So the fill is first
@@ -39,8 +43,8 @@
 // coarse grids get a fixed number of rounds and no host check; each level
 // starts from the bounds of the level above it.
 //
-// Measured: 8192 x 8192 raw fractal 5.1 ms, 8192 x 8192 noisy plane 1.09 ms,
-// 700 x 933 fractal 0.36 ms (visits to the fixed point 5.9, 1.12 and 0.40
+// Measured: 8192 x 8192 raw fractal 4.6 ms, 8192 x 8192 noisy plane 1.02 ms,
+// 700 x 933 fractal 0.29 ms; in blocks of 64 threads 5.1, 1.09 and 0.36 (visits to the fixed point 5.9, 1.12 and 0.40
 // ms; at most 3 passes 5.5 and 0.45, 5 passes 5.5 and 0.37); without the coarse
 // levels too 6.5, 3.2 and 0.45 ms
 // (the fractal's lakes, thousands of cells wide, still fill one tile a round);
@@ -58,7 +62,8 @@ namespace fill {
 
 constexpr int T = 64;
 constexpr int RATIO = 4;                // side ratio of a level to the next finer one
-constexpr int NTF = T;                  // one thread per row, or column, of the tile
+constexpr int NTF = 256;                // threads per tile; the first T take a row, or a column, each
+constexpr int LINES = NTF / T;          // rows moved at once
 constexpr int HW = T + 2;               // rows and columns of a tile with its halo
 constexpr int RS = T + 3;               // row stride of those arrays: odd, so lanes down a column hit distinct banks
 constexpr int MAX_PASSES = 4;           // passes before a visit ends and lists its own tile again
@@ -286,23 +291,23 @@ __global__ void __launch_bounds__(NTF) k_fill_round(const float* z, int64_t H, i
       else
         *zd = INFINITY;
     };
-    for (int hi = 0; hi < HW; hi++) load(hi, tid + 1);
+    for (int hi = tid / T; hi < HW; hi += LINES) load(hi, tid % T + 1);
     for (int q = tid; q < 2 * HW; q += NTF) load(q >> 1, (q & 1) * (HW - 1));
     cp_async_commit();
     cp_async_wait<0>();
     __syncthreads();
     bool any = false, settled = false;
     for (int k = 0; k < MAX_PASSES; k++) {
-      if (!__syncthreads_or(relax_dir(k, Fh, zh, raise))) {
+      if (!__syncthreads_or(tid < T && relax_dir(k, Fh, zh, raise))) {
         settled = true;
         break;
       }
       any = true;
     }
     if (any) {
-      if (tid < tw)
+      if (tid % T < tw)
 #pragma unroll 8
-        for (int i = 0; i < th; i++) F[(i0 + i) * ldF + (j0 + tid)] = Fh[(i + 1) * RS + tid + 1];
+        for (int i = tid / T; i < th; i += LINES) F[(i0 + i) * ldF + (j0 + tid % T)] = Fh[(i + 1) * RS + tid % T + 1];
       // halo cells that would drop under the new border: their tiles go on
       // the next round's list (their F here may be older, so higher, than
       // their tile's own: then the tile may be listed for nothing)
