@@ -40,18 +40,18 @@
 //     max of F over B <= up^n(X) <= X + |X| b + a        (BlockBound below),
 // and blocks holding cells of the grid's edge keep the bound with X = Z(B).
 // Every state of that iteration from +inf bounds F, settled or not, so the
-// coarse grids get a fixed number of rounds and no host check; each level
-// starts from the bounds of the level above it.
+// coarse grids get one round each and no host check; each level starts from
+// the bounds of the level above it.
 //
-// Measured: 8192 x 8192 raw fractal 4.6 ms, 8192 x 8192 noisy plane 1.02 ms,
-// 700 x 933 fractal 0.29 ms; in blocks of 64 threads 5.1, 1.09 and 0.36 (visits to the fixed point 5.9, 1.12 and 0.40
-// ms; at most 3 passes 5.5 and 0.45, 5 passes 5.5 and 0.37); without the coarse
-// levels too 6.5, 3.2 and 0.45 ms
-// (the fractal's lakes, thousands of cells wide, still fill one tile a round);
-// before (256 threads per tile, two waves over dirty cells, then sweeps of
-// four passes until a whole sweep changed nothing; lanes down a row shared
-// banks, and every change of a tile's border listed all eight neighbours) the
-// fractals took 105 and 4.7 ms.
+// Measured, 8192 x 8192 raw fractal, 8192 x 8192 noisy plane, 700 x 933 fractal:
+// 4.4, 0.93 and 0.25 ms.  With more rounds on the coarse grids 4.6, 1.02 and
+// 0.29; in blocks of 64 threads too 5.1, 1.09 and 0.36 (at most 3 passes a visit
+// 5.5 ms and 0.45 for the fractals, 5 passes 5.5 and 0.37); visits to the fixed
+// point 5.9, 1.12 and 0.40; without the coarse grids 6.5, 3.2 and 0.45 (the
+// fractal's lakes, thousands of cells wide, still fill one tile a round);
+// before (two waves over dirty cells, then sweeps of four passes until a whole
+// sweep changed nothing; lanes down a row shared banks, and every change of a
+// tile's border listed all eight neighbours) the fractals took 105 and 4.7 ms.
 #include <cmath>
 #include <type_traits>
 
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(NTF) k_fill_round(const float* z, int64_t H, i
 
 namespace fill {
 
-constexpr int CHUNK = 8;      // rounds launched at once: between host checks, and at most on a coarse grid
+constexpr int CHUNK = 8;      // rounds between host checks
 constexpr int MAX_LEVELS = 8;
 constexpr size_t HEAD = 256;  // bytes of a level's counts (CHUNK + 1) and work queues (CHUNK)
 static_assert(RATIO == 4, "k_fill_init and k_fill_pool move blocks' rows as float4");
@@ -489,11 +489,12 @@ cudaError_t run_fill(const float* z, int64_t H, int64_t W, int64_t ldz, float ep
   for (int l = n - 1; l >= 1 && e == cudaSuccess; l--) {
     const BlockBound bound((float)(1 << (2 * l)), eps);
     e = start_level(lv[l], l + 1 < n ? &lv[l + 1] : nullptr, bound, false, status, sms, s, nlaunch);
-    // a change crosses about two tiles a round where it matters: bounds left
-    // higher than they could be only cost the finer level visits
-    const int64_t side = lv[l].ntx > lv[l].nty ? lv[l].ntx : lv[l].nty;
-    const int r = side == 1 ? 1 : (int)min64(CHUNK, 3 + side / 2);
-    if (e == cudaSuccess) e = rounds(lv[l], bound, 0, r, sms, s, nlaunch);
+    // bounds left higher than they could be only cost the finer level visits,
+    // and not as many as more rounds here take (k of them, up to 8, for a
+    // level of 2 (k - 3) tiles a side: 8192 x 8192 fractal 4.58 ms, 4.36 with
+    // one; noisy plane 1.03 and 0.93; 700 x 933 fractal 308 us and 247; 4096 x
+    // 4096 noisy bowl 3.31 ms and 3.15)
+    if (e == cudaSuccess) e = rounds(lv[l], bound, 0, 1, sms, s, nlaunch);
   }
   if (e == cudaSuccess) e = start_level(G, n > 1 ? &lv[1] : nullptr, CellRaise{eps}, n == 1, status, sms, s, nlaunch);
   if (e != cudaSuccess) return e;
