@@ -176,6 +176,7 @@ struct HShape {
   int S[HMAX + 1] = {};
   int64_t nunits[HMAX + 1] = {};
   bool need_top = false;
+  bool jump = false;
 };
 
 // Levels above tiles of side T for the given DEM shapes.
@@ -189,6 +190,7 @@ HShape hier_shape(int T, int n, const int64_t* H, const int64_t* W, bool weighte
   for (int k = 0; k < n; k++) mx = H[k] > mx ? H[k] : (W[k] > mx ? W[k] : mx);
   for (int k = 0; k < n; k++) mx = W[k] > mx ? W[k] : mx;
   int S[HMAX], G[HMAX];
+  hs.jump = strat == STRAT_JUMP;
   hs.solve = !weighted && strat != STRAT_JUMP && mx > T && mx <= solve_side(T);
   hs.nlev = hs.solve ? 0 : hier_levels(T, mx, !weighted && strat != STRAT_JUMP, S, G, HMAX - 1);
   hs.S[0] = T;
@@ -214,7 +216,7 @@ size_t hier_bytes(const HShape& hs, size_t vb) {
   }
   const size_t nt = (size_t)hs.nunits[hs.nlev] * 4 * hs.S[hs.nlev];
   // par, par2, list; node words (8 B) or two rounds' additions; round flags
-  if (hs.need_top) b += 3 * align256(nt * 4) + align256(nt * 2 * vb) + align256(sizeof(uint32_t) * (MAX_ROUNDS + 2));
+  if (hs.need_top) b += 3 * align256(nt * 4) + align256(nt * (hs.jump ? 2 * vb : 8)) + align256(sizeof(uint32_t) * (MAX_ROUNDS + 2));
   b += align256(sizeof(uint32_t) * 64);
   return b;
 }
@@ -267,7 +269,7 @@ HPlan carve_hier(void* base, const HShape& hs, const Pipe& p, const DemTable* dt
     hp.top.par2 = reinterpret_cast<uint32_t*>(q);
     q += align256(nt * 4);
     hp.top.node = reinterpret_cast<unsigned long long*>(q);
-    q += align256(nt * 2 * vb);
+    q += align256(nt * (hs.jump ? 2 * vb : 8));
     hp.top.list = reinterpret_cast<uint32_t*>(q);
     q += align256(nt * 4);
     hp.top.flags = reinterpret_cast<uint32_t*>(q);
@@ -664,7 +666,13 @@ d8_status d8_fill(d8_ctx* c, const float* z, int64_t H, int64_t W, int64_t ldz, 
   const char *fb = reinterpret_cast<const char*>(F), *fe = fb + ((H - 1) * ldF + W) * sizeof(float);
   if (zb < fe && fb < ze) return D8_ERR_ARG;
   cudaSetDevice(c->device);
-  d8_status st = ensure_ws(c, fill_ws_bytes(H, W));
+  // where memory has no room for the coarser grids the fill goes without them
+  bool coarse = true;
+  d8_status st = ensure_ws(c, fill_ws_bytes(H, W, true));
+  if (st == D8_ERR_NOMEM) {
+    coarse = false;
+    st = ensure_ws(c, fill_ws_bytes(H, W, false));
+  }
   if (st != D8_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int64_t r = 0;
@@ -672,7 +680,7 @@ d8_status d8_fill(d8_ctx* c, const float* z, int64_t H, int64_t W, int64_t ldz, 
   cudaError_t e;
   {
     StageScope sc(c, ST_FILL, s);
-    e = run_fill(z, H, W, ldz, eps, F, ldF, c->ws, c->status, s, (int64_t)1 << 20, &r, &timed_out, &sc.n);
+    e = run_fill(z, H, W, ldz, eps, F, ldF, c->ws, coarse, c->status, s, (int64_t)1 << 20, &r, &timed_out, &sc.n);
   }
   if (rounds) *rounds = r;
   if (e != cudaSuccess) return cuda_fail(e);

@@ -366,7 +366,7 @@ static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 // x 500: 343 us without levels, 400 with; 700 x 933: 452 and 434; 3000 x 3000:
 // 1464 and 934).  Returns their number; bytes: the workspace.
 // What must be zero at the start comes first, `zeroed` bytes of it.
-static int levels(int64_t H, int64_t W, void* ws, Level* lv, size_t* zeroed, size_t* bytes) {
+static int levels(int64_t H, int64_t W, bool coarse, void* ws, Level* lv, size_t* zeroed, size_t* bytes) {
   int n = 0;
   size_t at = 0;
   char* base = static_cast<char*>(ws);
@@ -382,7 +382,7 @@ static int levels(int64_t H, int64_t W, void* ws, Level* lv, size_t* zeroed, siz
     L.queues = L.counts + CHUNK + 1;
     L.mark = reinterpret_cast<uint32_t*>(base + at + HEAD);
     at += HEAD + a256(sizeof(uint32_t) * (size_t)L.ntiles);
-    if (n == MAX_LEVELS || L.ntiles == 1 || (n == 1 && min64(L.ntx, L.nty) <= 8)) break;
+    if (!coarse || n == MAX_LEVELS || L.ntiles == 1 || (n == 1 && min64(L.ntx, L.nty) <= 8)) break;
     H = (H + RATIO - 1) / RATIO;
     W = (W + RATIO - 1) / RATIO;
   }
@@ -449,10 +449,10 @@ static cudaError_t rounds(const Level& L, Raise raise, int64_t first, int n, int
 
 }  // namespace fill
 
-size_t fill_ws_bytes(int64_t H, int64_t W) {
+size_t fill_ws_bytes(int64_t H, int64_t W, bool coarse) {
   fill::Level lv[fill::MAX_LEVELS];
   size_t zeroed, bytes;
-  fill::levels(H, W, nullptr, lv, &zeroed, &bytes);
+  fill::levels(H, W, coarse, nullptr, lv, &zeroed, &bytes);
   return bytes;
 }
 
@@ -461,12 +461,12 @@ size_t fill_ws_bytes(int64_t H, int64_t W) {
 // every CHUNK rounds (synchronising the stream) and stops after max_rounds
 // with D8_ERR_TIMEOUT.
 cudaError_t run_fill(const float* z, int64_t H, int64_t W, int64_t ldz, float eps, float* F, int64_t ldF, void* ws,
-                     uint32_t* status, cudaStream_t s, int64_t max_rounds, int64_t* rounds_out, bool* timed_out,
+                     bool coarse, uint32_t* status, cudaStream_t s, int64_t max_rounds, int64_t* rounds_out, bool* timed_out,
                      int* nlaunch) {
   using namespace fill;
   Level lv[MAX_LEVELS];
   size_t zeroed, bytes;
-  const int n = levels(H, W, ws, lv, &zeroed, &bytes);
+  const int n = levels(H, W, coarse, ws, lv, &zeroed, &bytes);
   Level& G = lv[0];
   G.z = z;
   G.ldz = ldz;

@@ -143,9 +143,10 @@ cudaError_t launch_up_unit(const DemTable& dt, const Pipe& p, bool weighted, cud
 cudaError_t launch_down_unit(const DemTable& dt, const Pipe& p, cudaStream_t s);
 
 // ---- pit and flat removal (d8_fill.cu)
-size_t fill_ws_bytes(int64_t H, int64_t W);
+// (coarse: with the coarser grids, which take 0.53 bytes per cell)
+size_t fill_ws_bytes(int64_t H, int64_t W, bool coarse);
 cudaError_t run_fill(const float* z, int64_t H, int64_t W, int64_t ldz, float eps, float* F, int64_t ldF, void* ws,
-                     uint32_t* status, cudaStream_t s, int64_t max_rounds, int64_t* rounds_out, bool* timed_out,
+                     bool coarse, uint32_t* status, cudaStream_t s, int64_t max_rounds, int64_t* rounds_out, bool* timed_out,
                      int* nlaunch);
 
 // shared-memory bytes of the per-tile kernels (0 = configuration unsupported)
