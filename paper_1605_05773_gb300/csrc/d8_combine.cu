@@ -515,6 +515,10 @@ static cudaError_t launch_solve(const HLevel& t, uint32_t* status, cudaStream_t 
 // of side 512 has 2048 slots and at most nine units drain into one: 16 bits.)
 constexpr unsigned long long CHILD = (1ull << 32) | (1ull << 48), LEFT = 1ull << 32;
 __device__ __forceinline__ uint32_t left_of(unsigned long long w) { return (uint32_t)(w >> 32) & 0xFFFFu; }
+__device__ __forceinline__ uint32_t children(const unsigned long long* node, uint32_t p) {
+  return (uint32_t)(*(volatile const unsigned long long*)&node[p] >> 48);
+}
+constexpr uint32_t LONG_WALK = 64;  // steps
 
 // parents, children counts and values (the words were zeroed by the level below)
 template <int S, class V, class CV>
@@ -555,7 +559,12 @@ __global__ void k_top_init(DemTable dt, const uint16_t* pex, const CV* pval, V* 
 // and 188).  Unit counts: one 64-bit atomic per step delivers the value and
 // tells the last child (no fences); each finished node stores its value for
 // the down sweep.  Float-float: value add, then children count, released and
-// acquired by its atomic.
+// acquired by its atomic.  The next parent is loaded beside the atomic, so a
+// step waits for one reply, not two.  A walk that has gone far is on a chain,
+// where most nodes have one child: nobody else adds to those, so plain loads do.
+// (Looking from the first step on costs short walks more than it saves: 32768 x
+// 32768 combine 1.56 and 1.62 ms.)  An 8192 x 8192 boustrophedon, 122,895 steps:
+// 32.6 ms (50.4 before, 42.8 without the plain loads), weighted 56 (155).
 // counters: [1] exits, [2] finished.
 template <class V>
 __global__ void __launch_bounds__(256) k_top_walk(const uint16_t* pex, const uint32_t* par, V* fin,
@@ -567,31 +576,46 @@ __global__ void __launch_bounds__(256) k_top_walk(const uint16_t* pex, const uin
     exits++;
     const unsigned long long w = *(volatile const unsigned long long*)&node[g];
     if (w >> 48) continue;  // has children: their walks come here
-    uint32_t x = (uint32_t)g;
+    uint32_t x = (uint32_t)g, run = 0;
     if constexpr (std::is_same<V, uint32_t>::value) {
-      uint32_t v = (uint32_t)w;
+      uint32_t v = (uint32_t)w, p = par[x];
       for (;;) {
         fin[x] = v;
         done++;
-        const uint32_t p = par[x];
         if (p == ROOT) break;
+        const uint32_t next = par[p];  // in flight beside the atomic: a step waits for one reply, not two
+        if (++run > LONG_WALK && children(node, p) == 1u) {
+          v += (uint32_t)node[p];
+          x = p;
+          p = next;
+          continue;
+        }
         const unsigned long long old = atomicAdd(&node[p], (unsigned long long)v - LEFT);
         if (left_of(old) != 1u) break;
         v += (uint32_t)old;
         x = p;
+        p = next;
       }
     } else {
       V v = fin[x];
+      uint32_t p = par[x];
       done++;
       for (;;) {
-        const uint32_t p = par[x];
         if (p == ROOT) break;
+        const uint32_t next = par[p];
+        if (++run > LONG_WALK && children(node, p) == 1u) {
+          v = vadd(fin[p], v);
+          fin[p] = v;
+          p = next;
+          done++;
+          continue;
+        }
         vatomic_add(&fin[p], v);
         // the high half of the word: releases the addition; acquires the others'
         const uint32_t old = atomic_add_acq_rel_gpu(reinterpret_cast<uint32_t*>(&node[p]) + 1, 0u - 1u);
         if ((old & 0xFFFFu) != 1u) break;
-        x = p;
         v = vload_volatile(&fin[p]);
+        p = next;
         done++;
       }
     }
