@@ -481,7 +481,7 @@ def run_fill(dev, steps: int):
         out[f"fractal_raw_{n}"] = {"ms_per_fill": ms, "value": n * n / (ms / 1e3), "unit": "cells/s",
                                    "tile_rounds": rounds, "cells_raised": raised,
                                    "timing": "host wall clock around the synchronous call (it checks convergence "
-                                             "on the host every 16 rounds)"}
+                                             "on the host every 8 rounds)"}
         del zt, F
     crop = np.ascontiguousarray(demgen.fractal_raw(2048, 2048, demgen.SEED_BASE))
     t0 = time.perf_counter()
