@@ -897,7 +897,6 @@ static cudaError_t combine_hier_t(const HPlan& hp, cudaStream_t s, int* nlaunch)
     if (e != cudaSuccess) return e;
   }
   // down: level l -> l-1 (at the tiles: the receivers' inflow)
-  constexpr bool RECV = true;
   for (int l = hp.nlev; l >= 1 && e == cudaSuccess; l--) {
     const HLevel& c = hp.lev[l - 1];
     const HLevel& g = hp.lev[l];
@@ -905,7 +904,7 @@ static cudaError_t combine_hier_t(const HPlan& hp, cudaStream_t s, int* nlaunch)
 #define D8_DN(SS, GG)                                                                                               \
   if (S == SS && G == GG) {                                                                                        \
     const uint32_t* cnt = l == hp.nlev && hp.need_top && !hp.top.jump ? hp.top.counters : nullptr;                \
-    e = l == 1 ? launch_level_down<SS, GG, V, CV0, RECV>(c.dt, g.dt, c.pex, c.pval, c.fin, g.fin, g.nunits,         \
+    e = l == 1 ? launch_level_down<SS, GG, V, CV0, true>(c.dt, g.dt, c.pex, c.pval, c.fin, g.fin, g.nunits,         \
                                                          hp.queue + 16 + l, cnt, hp.status, s)                    \
                : launch_level_down<SS, GG, V, V, false>(c.dt, g.dt, c.pex, c.pval, c.fin, g.fin, g.nunits,          \
                                                         hp.queue + 16 + l, cnt, hp.status, s);                    \

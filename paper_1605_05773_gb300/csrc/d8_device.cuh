@@ -185,28 +185,6 @@ __device__ __forceinline__ int64_t global_slot(const DemDesc& d, int64_t gi, int
 constexpr uint16_t PEX_EXIT = 0x8000u;
 constexpr uint16_t PEX_TERM = 0x7FFFu;
 
-// ---- per-cell class flags in shared memory ---------------------------------
-constexpr uint8_t CL_IN = 0x08;      // target inside the tile; bits 0..2 = code
-constexpr uint8_t CL_EXIT = 0x10;    // target in another tile; bits 0..2 = code
-constexpr uint8_t CL_TERM = 0x20;    // path ends here
-constexpr uint8_t CL_ABSENT = 0x40;  // outside a ragged tile
-
-// Classify a code of cell (i, j) of a tile: in-tile target, exit, or end.
-__device__ __forceinline__ uint8_t classify(int code, int i, int j, const TileGeo& g, const DemDesc& d,
-                                            uint32_t* status) {
-  if (code > 9) {
-    atomicOr(status, 1u << D8_ERR_ARG);
-    return CL_TERM;
-  }
-  if (code >= 8) return CL_TERM;
-  const int di = code_di(code), dj = code_dj(code);
-  const int64_t gi = g.i0 + i + di, gj = g.j0 + j + dj;
-  if (gi < 0 || gj < 0 || gi >= d.H || gj >= d.W) return CL_TERM;
-  const int li = i + di, lj = j + dj;
-  if (li >= 0 && lj >= 0 && li < g.th && lj < g.tw) return (uint8_t)(CL_IN | code);
-  return (uint8_t)(CL_EXIT | code);
-}
-
 __device__ __forceinline__ void set_status(uint32_t* status, int code) { atomicOr(status, 1u << code); }
 
 // A flag that many blocks raise and the next launch reads: written only while
