@@ -202,12 +202,12 @@ __device__ __forceinline__ void block_append(const bool (&take)[BPJ_U], const ui
   }
   __syncthreads();
   uint32_t pos = start[warp];
+  __syncwarp();  // every lane has read its warp's entry, which lane 0 writes in the next call before any barrier
 #pragma unroll
   for (int u = 0; u < BPJ_U; u++) {
     if (take[u]) list[pos + __popc(m[u] & ((1u << lane) - 1u))] = item[u];
     pos += __popc(m[u]);
   }
-  // (start[] is next written after the barrier of the next call's first half)
 }
 
 // combine init: H0(x) = path sum of x's successor inside its tile, parent =
