@@ -358,6 +358,15 @@ __device__ __forceinline__ ff fx96_to_ff(uint32_t w0, uint32_t w1, uint32_t w2, 
   return neg ? ff{-r.hi, -r.lo} : r;
 }
 
+// The same value with |lo| at most half an ulp of hi (TwoSum: exact whatever the
+// parts' sizes; the combine's sums are not normalised, and where they cancel
+// the low part can be all there is).
+__device__ __forceinline__ ff normalised(ff a) {
+  const float s = __fadd_rn(a.hi, a.lo);
+  const float b = __fsub_rn(s, a.hi);
+  return ff{s, __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, b)), __fsub_rn(a.lo, b))};
+}
+
 // The tile's codes lie with the padded row stride of Ahead; the fixed-point
 // words of cell (i, j) at i * T + (j ^ 4 (i mod 8)), which puts vertical
 // neighbours in different banks without the padding's memory (four tiles per
@@ -526,7 +535,7 @@ __global__ void __launch_bounds__(NTW, T >= 128 ? 1 : (T >= 64 ? 4 : 8)) k_fin_a
       const uint32_t k = code[i * S + j];
       const int ti = i + code_di(k & 7), tj = j + code_dj(k & 7);
       if (k < 8u && ((unsigned)ti >= (unsigned)g.th || (unsigned)tj >= (unsigned)g.tw)) code[i * S + j] = 8;
-      const ff in = ahead.in[r];
+      const ff in = normalised(ahead.in[r]);
       if (in.hi == 0.0f && in.lo == 0.0f) continue;
       const uint32_t at = atomicAdd(&misc[0], 1u);
       rcell[at] = (uint16_t)(i * S + j);
