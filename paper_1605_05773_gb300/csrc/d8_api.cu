@@ -50,12 +50,16 @@ struct d8_ctx {
   std::vector<Timing> pending;
   double ms[ST_COUNT] = {};
   int64_t launches[ST_COUNT] = {};
-  // the last forward call's combine, for d8_combine_stats
+  // the last forward call's combine, for d8_combine_stats: the counters and
+  // flags in the workspace while nothing else has taken their place
+  // (keep_stats), then what they said
   int last_levels = 0;
   int64_t last_top_units = 0;
   bool last_jump = false;
   uint32_t* last_counters = nullptr;
   uint32_t* last_flags = nullptr;
+  int64_t last_exits = 0;
+  int last_rounds = -1;
 };
 
 struct d8_batch {
@@ -278,10 +282,30 @@ HPlan carve_hier(void* base, const HShape& hs, const Pipe& p, const DemTable* dt
   return hp;
 }
 
+// Reads the last combine's statistics out of the workspace, once: before they
+// are asked for, and before the workspace is freed or a fill writes over them.
+d8_status keep_stats(d8_ctx* c, cudaStream_t s) {
+  if (!c->last_counters) return D8_OK;
+  uint32_t cnt[4] = {}, fl[MAX_ROUNDS + 2] = {};
+  cudaError_t e = cudaMemcpyAsync(cnt, c->last_counters, sizeof(cnt), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && c->last_jump) e = cudaMemcpyAsync(fl, c->last_flags, sizeof(fl), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  c->last_counters = c->last_flags = nullptr;
+  if (e != cudaSuccess) return D8_ERR_CUDA;
+  c->last_exits = c->last_jump ? cnt[0] : cnt[1];  // every exit listed, or counted by the walks
+  if (c->last_jump) {
+    int r = 0;
+    while (r < MAX_ROUNDS + 1 && fl[r]) r++;
+    c->last_rounds = r;
+  }
+  return D8_OK;
+}
+
 d8_status ensure_ws(d8_ctx* c, size_t bytes) {
   if (c->ws_bytes >= bytes) return D8_OK;
   if (c->ws) {
     cudaDeviceSynchronize();
+    keep_stats(c, nullptr);
     cudaFree(c->ws);
     c->ws = nullptr;
     c->ws_bytes = 0;
@@ -366,6 +390,8 @@ d8_status run_forward(d8_ctx* c, const DemDesc& d0, int mode, int rule, cudaStre
     c->last_jump = hp.top.jump;
     c->last_counters = hs.need_top ? hp.top.counters : nullptr;
     c->last_flags = hs.need_top ? hp.top.flags : nullptr;
+    c->last_exits = 0;
+    c->last_rounds = -1;
     e = launch_combine_hier(hp, s, &sc.n);
   }
   if (e != cudaSuccess) return cuda_fail(e);
@@ -483,25 +509,12 @@ d8_status d8_combine_stats(d8_ctx* c, d8_stream stream, int64_t* out, int n) {
   if (!c || !out || n < 4) return D8_ERR_ARG;
   cudaSetDevice(c->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const d8_status st = keep_stats(c, s);
   out[0] = c->last_levels;
   out[1] = c->last_top_units;
-  out[2] = 0;
-  out[3] = -1;
-  if (!c->last_counters) return D8_OK;
-  uint32_t cnt[4] = {}, fl[MAX_ROUNDS + 2] = {};
-  cudaError_t e = cudaMemcpyAsync(cnt, c->last_counters, sizeof(cnt), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess && c->last_jump) e = cudaMemcpyAsync(fl, c->last_flags, sizeof(fl), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return D8_ERR_CUDA;
-  if (c->last_jump) {
-    out[2] = cnt[0];  // every exit listed
-    int r = 0;
-    while (r < MAX_ROUNDS + 1 && fl[r]) r++;
-    out[3] = r;
-  } else {
-    out[2] = cnt[1];  // exits counted by the source listing
-  }
-  return D8_OK;
+  out[2] = c->last_exits;
+  out[3] = c->last_rounds;
+  return st;
 }
 
 d8_status d8_get_status(d8_ctx* c, d8_stream stream) {
@@ -675,6 +688,8 @@ d8_status d8_fill(d8_ctx* c, const float* z, int64_t H, int64_t W, int64_t ldz, 
   }
   if (st != D8_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (reinterpret_cast<char*>(c->last_counters) < static_cast<char*>(c->ws) + fill_ws_bytes(H, W, coarse))
+    keep_stats(c, s);
   int64_t r = 0;
   bool timed_out = false;
   cudaError_t e;
