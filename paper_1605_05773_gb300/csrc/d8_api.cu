@@ -11,6 +11,7 @@
 
 #include "d8.h"
 #include "d8_internal.h"
+#include "d8_workspace.h"
 
 using namespace d8;
 
@@ -42,8 +43,7 @@ struct d8_ctx {
   int device = 0;
   int T = 64;
   int strat = d8::STRAT_RING;
-  void* ws = nullptr;
-  size_t ws_bytes = 0;
+  d8::Workspace ws;
   uint32_t* status = nullptr;
   int profiling = 0;
   std::vector<cudaEvent_t> free_events;
@@ -301,24 +301,27 @@ d8_status keep_stats(d8_ctx* c, cudaStream_t s) {
   return D8_OK;
 }
 
-d8_status ensure_ws(d8_ctx* c, size_t bytes) {
-  if (c->ws_bytes >= bytes) return D8_OK;
-  if (c->ws) {
+struct CtxMemory {
+  d8_ctx* c;
+  void* alloc(size_t n) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, n) == cudaSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
+  }
+  void release(void* p) {
     cudaDeviceSynchronize();
     keep_stats(c, nullptr);
-    cudaFree(c->ws);
-    c->ws = nullptr;
-    c->ws_bytes = 0;
+    cudaFree(p);
   }
-  cudaError_t e = cudaMalloc(&c->ws, bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    c->ws = nullptr;
-    return D8_ERR_NOMEM;
-  }
-  c->ws_bytes = bytes;
-  return D8_OK;
+};
+
+// want bytes of workspace, or at least need when there is no room for them
+d8_status ensure_ws(d8_ctx* c, size_t want, size_t need) {
+  CtxMemory mem{c};
+  return c->ws.ensure(mem, want, need) ? D8_OK : D8_ERR_NOMEM;
 }
+d8_status ensure_ws(d8_ctx* c, size_t bytes) { return ensure_ws(c, bytes, bytes); }
 
 DemDesc make_desc(int64_t H, int64_t W, int T) {
   DemDesc d{};
@@ -355,7 +358,7 @@ d8_status run_forward(d8_ctx* c, const DemDesc& d0, int mode, int rule, cudaStre
   const size_t pb = align256(pipe_bytes(ntiles, T, vb));
   d8_status st = ensure_ws(c, pb + hb);
   if (st != D8_OK) return st;
-  Pipe p = carve_pipe(c->ws, ntiles, T, vb, c->status);
+  Pipe p = carve_pipe(c->ws.p, ntiles, T, vb, c->status);
   p.strat = c->strat;
   p.top_in = top_in;
   p.bot_in = bot_in;
@@ -384,7 +387,7 @@ d8_status run_forward(d8_ctx* c, const DemDesc& d0, int mode, int rule, cudaStre
       dl.tile_base = 0;
       dts[l] = single(dl);
     }
-    const HPlan hp = carve_hier(static_cast<char*>(c->ws) + pb, hs, p, dts, weighted);
+    const HPlan hp = carve_hier(static_cast<char*>(c->ws.p) + pb, hs, p, dts, weighted);
     c->last_levels = hs.solve ? 1 : hs.nlev;
     c->last_top_units = hs.need_top ? hs.nunits[hs.nlev] : 0;
     c->last_jump = hp.top.jump;
@@ -452,7 +455,7 @@ d8_status d8_destroy(d8_ctx* c) {
   if (!c) return D8_OK;
   cudaSetDevice(c->device);
   cudaDeviceSynchronize();
-  if (c->ws) cudaFree(c->ws);
+  if (c->ws.p) cudaFree(c->ws.p);
   if (c->status) cudaFree(c->status);
   for (auto& t : c->pending) {
     cudaEventDestroy(t.a);
@@ -645,10 +648,10 @@ d8_status d8_accumulate_backward(d8_ctx* c, const uint8_t* dir, int64_t H, int64
   const size_t lb = align256((size_t)ntiles * 4 * T * 4);
   d8_status st = ensure_ws(c, pb + xb + 2 * lb);
   if (st != D8_OK) return st;
-  Pipe p = carve_pipe(c->ws, ntiles, T, 8, c->status);
-  p.xid = reinterpret_cast<uint16_t*>(static_cast<char*>(c->ws) + pb);
-  p.list[0] = reinterpret_cast<uint32_t*>(static_cast<char*>(c->ws) + pb + xb);
-  p.list[1] = reinterpret_cast<uint32_t*>(static_cast<char*>(c->ws) + pb + xb + lb);
+  Pipe p = carve_pipe(c->ws.p, ntiles, T, 8, c->status);
+  p.xid = reinterpret_cast<uint16_t*>(static_cast<char*>(c->ws.p) + pb);
+  p.list[0] = reinterpret_cast<uint32_t*>(static_cast<char*>(c->ws.p) + pb + xb);
+  p.list[1] = reinterpret_cast<uint32_t*>(static_cast<char*>(c->ws.p) + pb + xb + lb);
   DemTable dt = single(d);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaMemsetAsync(p.queue, 0, sizeof(uint32_t) * 16, s);
@@ -680,22 +683,19 @@ d8_status d8_fill(d8_ctx* c, const float* z, int64_t H, int64_t W, int64_t ldz, 
   if (zb < fe && fb < ze) return D8_ERR_ARG;
   cudaSetDevice(c->device);
   // where memory has no room for the coarser grids the fill goes without them
-  bool coarse = true;
-  d8_status st = ensure_ws(c, fill_ws_bytes(H, W, true));
-  if (st == D8_ERR_NOMEM) {
-    coarse = false;
-    st = ensure_ws(c, fill_ws_bytes(H, W, false));
-  }
+  const size_t with = fill_ws_bytes(H, W, true), without = fill_ws_bytes(H, W, false);
+  const d8_status st = ensure_ws(c, with, without);
   if (st != D8_OK) return st;
+  const bool coarse = c->ws.bytes >= with;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (reinterpret_cast<char*>(c->last_counters) < static_cast<char*>(c->ws) + fill_ws_bytes(H, W, coarse))
+  if (reinterpret_cast<char*>(c->last_counters) < static_cast<char*>(c->ws.p) + (coarse ? with : without))
     keep_stats(c, s);
   int64_t r = 0;
   bool timed_out = false;
   cudaError_t e;
   {
     StageScope sc(c, ST_FILL, s);
-    e = run_fill(z, H, W, ldz, eps, F, ldF, c->ws, coarse, c->status, s, (int64_t)1 << 20, &r, &timed_out, &sc.n);
+    e = run_fill(z, H, W, ldz, eps, F, ldF, c->ws.p, coarse, c->status, s, (int64_t)1 << 20, &r, &timed_out, &sc.n);
   }
   if (rounds) *rounds = r;
   if (e != cudaSuccess) return cuda_fail(e);
