@@ -19,7 +19,8 @@
 //    the code from five comparisons and predicated additions;
 //  * whole items inside the grid run a loop without any of the edges' tests
 //    (walk_inside); an item at the grid's edge, or one in which a non-finite
-//    elevation turned up, runs the general one (walk_any).
+//    elevation turned up that the rule does not mask, runs the general one
+//    (walk_any).
 // Rows that are not 16-byte aligned take 4-byte copies.  Grids
 // with few tiles are cut into shorter row segments, so that a small call
 // still fills the GPU (launch_t).
@@ -175,10 +176,26 @@ __device__ __forceinline__ void copy4_if(bool on, float* dst, const float* src) 
                :: "r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"((int)on) : "memory");
 }
 
+// Under NODATA: OUTLET for the cells of row b that are not finite or lie next to
+// a cell that is not.
+__device__ __forceinline__ uint32_t mask_nodata(const Row& a, const Row& b, const Row& c, uint32_t packed) {
+  float col[CPL + 2];  // NaN for a column with such a cell in the three rows
+#pragma unroll
+  for (int k = 0; k < CPL + 2; k++) col[k] = __fmaf_rn(a.v[k], 0.0f, __fmaf_rn(b.v[k], 0.0f, __fmul_rn(c.v[k], 0.0f)));
+#pragma unroll
+  for (int k = 0; k < CPL; k++) {
+    const float near = __fadd_rn(__fadd_rn(col[k], col[k + 1]), col[k + 2]);
+    if (near != near) packed = (packed & ~(0xFFu << (8 * k))) | (8u << (8 * k));
+  }
+  return packed;
+}
+
 // Items whose rows -1 .. n and own columns all lie on the grid and whose n is
 // a multiple of 4.  ring: PD rows of RW floats, columns j0 - 4 .. j0 + T + 3
 // of the tile; row k sits at place (k + 7) % 8.  Returns whether the warp met
-// a non-finite elevation (the codes are then redone by walk_any).
+// a non-finite elevation under a rule without masks (an error: the codes are
+// then redone by walk_any).  With masks such rows are masked in place: a raster
+// with a border or holes of NaN has whole tiles of them.
 template <int T, bool LOWEST, bool NODATA, bool VEC>
 __device__ __forceinline__ bool walk_inside(Item it, float* ring, float nz) {
   constexpr int LPT = T / CPL, RW = T + 8;
@@ -227,17 +244,23 @@ __device__ __forceinline__ bool walk_inside(Item it, float* ring, float nz) {
   fetch(ring + 6 * RW, true);  // row 7
   Slopes up, dn;
   if (!LOWEST) up = slopes_between(a, b);
-  float acc = nonfinite<NODATA>(b, NODATA ? nonfinite<NODATA>(a, 0.0f) : 0.0f);
-  bool redo = false;
+  float acc = nonfinite<NODATA>(b, 0.0f);  // NODATA: of row b alone, else of all rows so far
+  float above = NODATA ? nonfinite<NODATA>(a, 0.0f) : 0.0f;  // of row a
   for (int i = 0; i < it.n; i += 4) {
     float *cur = ring + (i & 4) * RW, *other = ring + ((i & 4) ^ 4) * RW;
 #pragma unroll
     for (int u = 0; u < 4; u++) {
       const Row c = take(cur + u * RW);
       fetch(u ? cur + (u - 1) * RW : other + 3 * RW, i + u + PD <= it.n);  // row i + u + 8
-      acc = nonfinite<NODATA>(c, acc);
+      const float next = nonfinite<NODATA>(c, NODATA ? 0.0f : acc);
       if (!LOWEST) dn = slopes_between(b, c);
       uint32_t packed = row_codes<LOWEST>(a, b, c, up, dn, nz);
+      if (NODATA) {
+        const float any = __fadd_rn(__fadd_rn(above, acc), next);
+        if (any != any) packed = mask_nodata(a, b, c, packed);
+        above = acc;
+      }
+      acc = next;
       packed = (packed & ~it.colmask) | (0x08080808u & it.colmask);
       if (VEC) {
         *reinterpret_cast<uint32_t*>(it.dir) = packed;
@@ -250,14 +273,10 @@ __device__ __forceinline__ bool walk_inside(Item it, float* ring, float nz) {
       b = c;
       up = dn;
     }
-    if (NODATA && __any_sync(FULL, acc != acc)) {
-      redo = true;
-      break;
-    }
   }
   cp_async_wait<0>();  // nothing may land in the ring after the item is done
   __syncwarp();
-  return redo || __any_sync(FULL, acc != acc);
+  return !NODATA && __any_sync(FULL, acc != acc);
 }
 
 // Any item.  Off the grid rows and columns read as zero: they only neighbour
@@ -289,15 +308,13 @@ __device__ __forceinline__ bool walk_any(Item it, float nz) {
     float bad = nonfinite<NODATA>(b, 0.0f);
     if (NODATA) bad = nonfinite<NODATA>(a, nonfinite<NODATA>(c, bad));
     if (bad != bad && i < it.n) {
+      if (NODATA) {
+        packed = mask_nodata(a, b, c, packed);
+      } else {
 #pragma unroll
-      for (int k = 0; k < CPL; k++) {
-        const bool own = !isfinite(b.v[k + 1]);
-        bool any = own;
-        if (NODATA)
-          any |= !(isfinite(a.v[k]) && isfinite(a.v[k + 1]) && isfinite(a.v[k + 2]) && isfinite(b.v[k]) &&
-                   isfinite(b.v[k + 2]) && isfinite(c.v[k]) && isfinite(c.v[k + 1]) && isfinite(c.v[k + 2]));
-        if (any) packed = (packed & ~(0xFFu << (8 * k))) | ((NODATA ? 8u : 9u) << (8 * k));
-        report |= !NODATA && own;
+        for (int k = 0; k < CPL; k++)
+          if (!isfinite(b.v[k + 1])) packed = (packed & ~(0xFFu << (8 * k))) | (9u << (8 * k));
+        report = true;
       }
     }
     const uint32_t m = (i == it.top || i == it.bottom) ? 0xFFFFFFFFu : it.colmask;
