@@ -336,17 +336,16 @@ __device__ __forceinline__ bool walk_any(Item it, float nz) {
 // NODATA masks (the rule's NODATA bit): a cell with a non-finite elevation is
 // outside the study area and gets OUTLET, and so does every cell next to one
 // (the area's edge drains off it, as the grid's edge does); nothing is
-// reported as an error.  seg_rows: rows per work item (a divisor of T).
+// reported as an error.  nseg: work items per tile, of seg_rows rows (a divisor of T).
 // nz: -0 (lowest_code).
 template <int T, bool LOWEST, bool NODATA>
-__global__ void __launch_bounds__(NTF, 5) k_flowdir_rows(DemTable dt, int64_t ntiles, int seg_rows, float nz,
+__global__ void __launch_bounds__(NTF, 5) k_flowdir_rows(DemTable dt, int64_t ntiles, int nseg, int seg_rows, float nz,
                                                          uint32_t* status) {
   constexpr int LPT = T / CPL;   // lanes per tile
   constexpr int IPW = 32 / LPT;  // items per warp
   const int lane = threadIdx.x & 31, li = lane & (LPT - 1);
   __shared__ __align__(16) float rings[NTF / LPT][PD * (T + 8)];
   float* ring = rings[threadIdx.x / LPT];
-  const int nseg = T / seg_rows;
   const int64_t nitems = ntiles * nseg;
   const int64_t step = (int64_t)gridDim.x * (NTF / 32) * IPW;
   const int64_t first = ((int64_t)blockIdx.x * (NTF / 32) + (threadIdx.x >> 5)) * IPW;
@@ -396,7 +395,9 @@ __global__ void __launch_bounds__(NTF, 5) k_flowdir_rows(DemTable dt, int64_t nt
 // in T are then read twice); below MIN_WARPS_PER_SM warps the tiles are cut
 // into segments of T / 2, T / 4, ... down to 8 rows.  (About 20 warps fit an
 // SM; with 40 here 8192 x 8192 runs 2.7 rounds of them and takes 122 us, with
-// 70 it halves its tiles and takes 98, with 140 it quarters them: 105.)
+// 70 it halves its tiles and takes 98, with 140 it quarters them: 105.)  A grid
+// lower than a tile is cut into segments of its own rows: 8 x 400000 takes 14 us,
+// 25 to 33 when two thirds of the segments lay below the grid.
 constexpr int64_t MIN_WARPS_PER_SM = 70;
 
 template <int T, bool LOWEST, bool NODATA>
@@ -410,12 +411,15 @@ static cudaError_t launch_t(const DemTable& dt, int64_t ntiles, uint32_t* status
     per_sm = 1;
   }
   constexpr int IPW = 32 / (T / CPL), IPB = IPW * (NTF / 32);
+  const int span = (int)(dt.ndem == 1 ? min64(T, dt.one.H) : T);  // rows of the highest tile
   int rows = T;
-  while (rows > 8 && ntiles * (T / rows) < MIN_WARPS_PER_SM * IPW * sms) rows /= 2;
-  int64_t grid = (ntiles * (T / rows) + IPB - 1) / IPB;
+  auto segments = [&]() { return (span + rows - 1) / rows; };
+  while (rows > 8 && ntiles * segments() < MIN_WARPS_PER_SM * IPW * sms) rows /= 2;
+  const int nseg = segments();
+  int64_t grid = (ntiles * nseg + IPB - 1) / IPB;
   const int64_t cap = (int64_t)sms * per_sm;
   if (grid > cap) grid = cap;
-  k<<<(unsigned)(grid < 1 ? 1 : grid), NTF, 0, s>>>(dt, ntiles, rows, -0.0f, status);
+  k<<<(unsigned)(grid < 1 ? 1 : grid), NTF, 0, s>>>(dt, ntiles, nseg, rows, -0.0f, status);
   return cudaGetLastError();
 }
 
