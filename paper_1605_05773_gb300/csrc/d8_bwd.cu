@@ -167,7 +167,8 @@ __global__ void __launch_bounds__(BwdCfg<T>::NTB, T >= 64 ? 2 : 4) k_bwd_up(DemT
 
 constexpr int BPJ_U = 4;     // list items or slots per thread and pass
 constexpr int BPJ_NT = 256;  // threads per block of the rounds
-constexpr int BPJ_END = 1024;  // threads of the block that ends them
+constexpr int BPJ_END = 1024;  // threads of a block of the cluster that ends them
+constexpr int END_BLOCKS = 8;  // its blocks
 
 // Append the items whose `take` is set to list[] at the position counter *cnt
 // hands out, with one atomic per block and pass.  (One per warp queued up
@@ -327,20 +328,26 @@ __global__ void __launch_bounds__(BPJ_NT) k_bpj_round(Pipe p, int r) {
   bpj_round<BPJ_NT>(p, r, *(volatile uint32_t*)&p.flags[r], blockIdx.x * BPJ_NT, gridDim.x * BPJ_NT, &p.flags[r + 1]);
 }
 
-// The rounds from r on in one block, until the list is empty; an exit still
-// open after round R - 1 lies on a cycle.
-__global__ void __launch_bounds__(BPJ_END) k_bpj_end(Pipe p, int r, int R) {
-  __shared__ uint32_t count;  // the next round's list
+// Every thread of the cluster's blocks meets here, and sees what the others wrote
+// to global memory before.
+__device__ __forceinline__ void cluster_sync() {
+  __threadfence();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  __threadfence();
+}
+
+// The rounds from r on in one cluster, until the list is empty; an exit still
+// open after round R - 1 lies on a cycle.  (n, the length of the round's list,
+// is the same in every block: its word is not written any more.)
+__global__ void __cluster_dims__(END_BLOCKS, 1, 1) __launch_bounds__(BPJ_END) k_bpj_end(Pipe p, int r, int R) {
   uint32_t n = p.flags[r];
   for (; n && r < R; r++) {
-    if (threadIdx.x == 0) count = 0u;
-    __syncthreads();
-    bpj_round<BPJ_END>(p, r, n, 0u, BPJ_END, &count);
-    __syncthreads();  // the round's writes, before the next round's reads
-    n = count;
-    __syncthreads();
+    bpj_round<BPJ_END>(p, r, n, blockIdx.x * BPJ_END, END_BLOCKS * BPJ_END, &p.flags[r + 1]);
+    cluster_sync();
+    n = *(volatile uint32_t*)&p.flags[r + 1];
   }
-  if (n && threadIdx.x == 0) set_status(p.status, D8_ERR_CYCLE);
+  if (n && blockIdx.x == 0 && threadIdx.x == 0) set_status(p.status, D8_ERR_CYCLE);
 }
 
 // dw(q) = (in-tile path sum of q, already in dw) + H(exit of q); four
@@ -462,9 +469,11 @@ cudaError_t launch_bwd_up(const DemTable& dt, const Pipe& p, cudaStream_t s, int
 // comes one round later, so the list of round R is empty unless a cycle holds
 // exits open.  Rounds after the list empties return at once (the rounds that
 // few fields need are launched small: an empty one takes half as long); on grids of up to
-// END_SLOTS slots, whose lists one block gets through, the rounds that only
-// winding fields need (paths of tiles longer than twice the grid's side) are
-// left to one such block instead of a launch each.
+// END_SLOTS slots the rounds that only winding fields need (paths of tiles longer
+// than twice the grid's side) are left to one cluster of blocks instead of a
+// launch each.  1001 x 777, whole combine: fractal 50 us (91 with a launch each),
+// boustrophedon and spiral 90 to 93 (103 to 108); one block alone took 49 and
+// 149 to 169, its lists of 10,000 exits being three or four passes a round.
 constexpr int64_t END_SLOTS = 1 << 16;
 template <int T>
 static cudaError_t launch_combine_bwd_t(const DemTable& dt, const Pipe& p, cudaStream_t s, int* nlaunch) {
@@ -482,7 +491,7 @@ static cudaError_t launch_combine_bwd_t(const DemTable& dt, const Pipe& p, cudaS
     k_bpj_round<<<grid_for_b(threads, r < ordinary ? 4 : 1), BPJ_NT, 0, s>>>(p, r);
     ++*nlaunch;
   }
-  k_bpj_end<<<1, BPJ_END, 0, s>>>(p, r, R);
+  k_bpj_end<<<END_BLOCKS, BPJ_END, 0, s>>>(p, r, R);
   ++*nlaunch;
   return cudaGetLastError();
 }
