@@ -92,10 +92,13 @@ __device__ __forceinline__ UnitGeo unit_geo(const DemDesc& d, int64_t uy, int64_
 // inside the group and the children count of every node.
 // Returns the number of child exits this thread loaded.
 // pd[n]: node n's parent (bits 16..31, or N_ROOT / N_OUT / N_NONE) and its
-// number of unfinished children (bits 0..15; a group has fewer than 2^16
-// nodes), one 32-bit word so that both live in native 32-bit atomics.
+// number of unfinished children (bits 0..14: a node's children drain into its
+// child unit's perimeter of 4 S cells, each with at most five cells outside),
+// one 32-bit word so that both live in native 32-bit atomics.  SINGLE: the node
+// has one child in all (marked in groups of long chains, group_walk).
 __device__ __forceinline__ uint32_t pd_par(uint32_t w) { return w >> 16; }
-__device__ __forceinline__ uint32_t pd_deg(uint32_t w) { return w & 0xFFFFu; }
+constexpr uint32_t SINGLE = 0x8000u;
+__device__ __forceinline__ uint32_t pd_deg(uint32_t w) { return w & (SINGLE - 1u); }
 
 // A group's extent in cells (ragged at the right and bottom), and that of its
 // child (a, b): everything inside a group is 32-bit arithmetic.
@@ -221,29 +224,16 @@ __device__ int group_load(const DemDesc& cd, const GroupGeo& gg, int64_t gy, int
   return exits;
 }
 
-// Algorithm 2 on the exit forest of a group: last-arriver walks from the
-// nodes without unfinished children.  A finished node adds its value to its
-// parent, then (after a block fence) decrements the parent's children count;
-// the last child continues at the parent (its acquire-release count atomic
-// orders it after every child's addition).  Returns the number of nodes this thread finished.
-template <int S, int G, int NT, class V>
-__device__ int group_walk(uint16_t* spx, V* val, uint32_t* pd, uint16_t* srcl) {
-  constexpr int NS = G * G * 4 * S;
-  constexpr int NW = NT / 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint16_t* my = srcl + warp * (NS / NW);
-  int n = 0;
-  for (int r = 0; r < NS / NT; r++) {
-    const int c = threadIdx.x + r * NT;
-    const bool s = (spx[c] & PEX_EXIT) && pd_deg(pd[c]) == 0u;
-    const unsigned m = __ballot_sync(FULL, s);
-    if (s) my[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)c;
-    n += __popc(m);
-  }
-  __syncthreads();
-  int done = 0, head = 0, cur = -1;
+// The walks of a warp's n sources.  CHAINS: a walk past LONG_RUN steps takes up to
+// CHAIN_STEPS nodes marked SINGLE at a time.  Nobody else adds to those, so a
+// step is a load of the node's word and three operations, where the atomics'
+// replies take 240 cycles.
+constexpr int LONG_RUN = 16, CHAIN_STEPS = 64;
+template <bool CHAINS, class V>
+__device__ __forceinline__ int walk_sources(const uint16_t* my, int n, V* val, uint32_t* pd) {
+  const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
+  int done = 0, head = 0, cur = -1, run = 0;
   V v{};
-  const unsigned lt = (1u << lane) - 1u;
   for (;;) {
     if (head < n) {
       const unsigned need = __ballot_sync(FULL, cur < 0);
@@ -252,13 +242,25 @@ __device__ int group_walk(uint16_t* spx, V* val, uint32_t* pd, uint16_t* srcl) {
         cur = my[idx];
         v = val[cur];
         done++;
+        run = 0;
       }
       head += __popc(need);
     } else if (!__any_sync(FULL, cur >= 0)) {
       break;
     }
     if (cur >= 0) {
-      const uint32_t p = pd_par(pd[cur]);
+      uint32_t p = pd_par(pd[cur]);
+      if (CHAINS && ++run > LONG_RUN) {
+        for (int k = 0; k < CHAIN_STEPS && p < N_NONE; k++) {
+          const uint32_t w = pd[p];
+          if (!(w & SINGLE)) break;
+          v = vadd(val[p], v);
+          val[p] = v;
+          cur = (int)p;
+          p = pd_par(w);
+          done++;
+        }
+      }
       if (p >= N_NONE) {
         cur = -1;
         continue;
@@ -277,6 +279,54 @@ __device__ int group_walk(uint16_t* spx, V* val, uint32_t* pd, uint16_t* srcl) {
     }
   }
   return done;
+}
+
+// Algorithm 2 on the exit forest of a group: last-arriver walks from the
+// nodes without unfinished children.  A finished node adds its value to its
+// parent, then (after a block fence) decrements the parent's children count;
+// the last child continues at the parent (its acquire-release count atomic
+// orders it after every child's addition).  exits: those this thread loaded.
+// Returns the number of nodes this thread finished.
+//
+// Unit counts: in a group whose channels wind, few exits are sources (4 to 12 %
+// on boustrophedons and spirals, 80 to 86 % on fractals and planes), and the walks
+// are chains.  There the nodes with one child are marked first, so that the walks
+// need no atomics on them.  A block decides as a whole, since the marks, and the
+// chain in the walks' loop, cost fractals 1 to 3 % of the whole call.
+// Whole accumulation of a 512 x 512 boustrophedon and spiral: 217 and 230 us (553
+// and 615 without; 326 and 621 with groups of 4 x 4 tiles and of 2 x 2, whose
+// chains are shorter), 300 x 257 spiral in 32 x 32 tiles 220 (443, 243), 600 x 700
+// spiral 364 (567, 473).
+template <int S, int G, int NT, class V>
+__device__ int group_walk(uint16_t* spx, V* val, uint32_t* pd, uint16_t* srcl, int exits) {
+  constexpr int NS = G * G * 4 * S;
+  constexpr int NW = NT / 32;
+  static_assert(5 * 4 * S < (int)SINGLE, "a children count fits below the mark");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint16_t* my = srcl + warp * (NS / NW);
+  int n = 0;
+  for (int r = 0; r < NS / NT; r++) {
+    const int c = threadIdx.x + r * NT;
+    const bool s = (spx[c] & PEX_EXIT) && pd_deg(pd[c]) == 0u;
+    const unsigned m = __ballot_sync(FULL, s);
+    if (s) my[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)c;
+    n += __popc(m);
+  }
+  if constexpr (std::is_same<V, uint32_t>::value) {
+    // the group winds if more warps say so than say it does not (one barrier
+    // counts both: half of a warp's lanes for it, the other half against it)
+    const int ex = (int)__reduce_add_sync(FULL, (unsigned)exits);
+    const bool winds = 4 * n < ex, ordinary = !winds && n + ex > 0;
+    if (__syncthreads_count(lane < 16 ? winds : !ordinary) > 16 * NW) {
+      for (int c = threadIdx.x; c < NS; c += NT)
+        if (pd_deg(pd[c]) == 1u) pd[c] |= SINGLE;
+      __syncthreads();
+      return walk_sources<true, V>(my, n, val, pd);
+    }
+  } else {
+    __syncthreads();
+  }
+  return walk_sources<false, V>(my, n, val, pd);
 }
 
 template <int S, int G, class V, class CV>
@@ -305,7 +355,7 @@ __global__ void __launch_bounds__(NTG<S, G>) k_group_up(DemTable cdt, DemTable g
     }
     const GroupGeo gg = group_geo<S, G>(gd, gy, gx);
     const int exits = group_load<S, G, NT, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
-    const int done = group_walk<S, G, NT, V>(spx, val, pd, srcl);
+    const int done = group_walk<S, G, NT, V>(spx, val, pd, srcl, exits);
     atomicAdd(&misc[0], done);
     atomicAdd(&misc[1], exits);
     __syncthreads();
@@ -401,7 +451,7 @@ __global__ void __launch_bounds__(NTG<S, G>) k_group_down(DemTable cdt, DemTable
     const int64_t lg = gu - gd.tile_base;
     const int64_t gy = lg / gd.ntx, gx = lg % gd.ntx;
     const GroupGeo gg = group_geo<S, G>(gd, gy, gx);
-    group_load<S, G, NT, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
+    const int exits = group_load<S, G, NT, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
     // inflow across the group border: each border cell r receives the final
     // areas of the outside cells draining into it; the inflow then follows
     // r's path inside its child unit to that child's exit
@@ -447,7 +497,7 @@ __global__ void __launch_bounds__(NTG<S, G>) k_group_down(DemTable cdt, DemTable
       }
     }
     __syncthreads();
-    group_walk<S, G, NT, V>(spx, val, pd, srcl);
+    group_walk<S, G, NT, V>(spx, val, pd, srcl, exits);
     __syncthreads();
     if constexpr (RECV) {
       V* infl = reinterpret_cast<V*>(pd);  // the walk is done with it
@@ -486,7 +536,7 @@ __global__ void __launch_bounds__(NTS) k_group_solve(DemTable dt, const uint16_t
   const GroupGeo gg = group_geo<S, G>(d, 0, 0);
   if (threadIdx.x < 2) misc[threadIdx.x] = 0;
   const int exits = group_load<S, G, NTS, uint32_t, uint32_t>(d, gg, 0, 0, pex, pval, spx, val, pd);
-  const int done = group_walk<S, G, NTS, uint32_t>(spx, val, pd, srcl);
+  const int done = group_walk<S, G, NTS, uint32_t>(spx, val, pd, srcl, exits);
   atomicAdd(&misc[0], done);
   atomicAdd(&misc[1], exits);
   __syncthreads();
