@@ -225,7 +225,7 @@ struct Codes {
 };
 
 // The words of tile g (zeroed before) from its codes: Algorithm 1.
-template <int T, int NT>
+template <int T, int NT, bool NARROW>
 __device__ __forceinline__ void set_words(const Codes<T, NT>& codes, const DemDesc& d, const TileGeo& g, uint32_t* word,
                                           const uint2* tab, uint32_t* status) {
   using P = Place<T>;
@@ -267,17 +267,19 @@ __device__ __forceinline__ void set_words(const Codes<T, NT>& codes, const DemDe
     return;
   }
   constexpr int U = 16;  // codes read at once
+  const int sh = NARROW ? width_shift(g) : T == 64 ? 6 : 5, end = NARROW ? g.th << sh : T * T;
+  static_assert(T == 64 || T == 32, "the shift of whole rows");
 #pragma unroll 1
-  for (int c0 = threadIdx.x; c0 < T * T; c0 += U * NT) {
+  for (int c0 = threadIdx.x; c0 < end; c0 += U * NT) {
     uint8_t code[U];
 #pragma unroll
     for (int u = 0; u < U; u++) {
-      const int c = c0 + u * NT, i = c / T, j = c % T;
+      const int c = c0 + u * NT, i = c >> sh, j = c & ((1 << sh) - 1);
       code[u] = i < g.th && j < g.tw ? __ldg(d.dir + (g.i0 + i) * d.lddir + (g.j0 + j)) : (uint8_t)0;
     }
 #pragma unroll
     for (int u = 0; u < U; u++) {
-      const int c = c0 + u * NT, i = c / T, j = c % T;
+      const int c = c0 + u * NT, i = c >> sh, j = c & ((1 << sh) - 1);
       if (i < g.th && j < g.tw) add_cell<T>(word, i, j, code[u], g, d, status);
     }
   }
@@ -303,7 +305,7 @@ __device__ __forceinline__ void end_at_grid_edge(const DemDesc& d, const TileGeo
 // A[tile] = the in-tile counts: four consecutive cells per thread in one 16-byte
 // store when the layout allows, else one.  Returns whether one of this thread's
 // cells still waits for an input: it lies on or below a cycle.
-template <int T, int NT>
+template <int T, int NT, bool NARROW>
 __device__ __forceinline__ bool store_counts(const DemDesc& d, const TileGeo& g, const uint32_t* word) {
   using P = Place<T>;
   using C = Cell<T>;
@@ -328,8 +330,9 @@ __device__ __forceinline__ bool store_counts(const DemDesc& d, const TileGeo& g,
     }
   } else {
     // consecutive lanes store consecutive columns
-    constexpr int RS = NT / T;  // rows at once
-    const int i0 = threadIdx.x / T, j = threadIdx.x % T;
+    const int sh = NARROW ? width_shift(g) : T == 64 ? 6 : 5;
+    const int RS = NT >> sh;  // rows at once
+    const int i0 = threadIdx.x >> sh, j = threadIdx.x & ((1 << sh) - 1);
     uint32_t* dst = static_cast<uint32_t*>(d.A) + (g.i0 + i0) * d.ldA + (g.j0 + j);
     if (j < g.tw) {
 #pragma unroll 8
@@ -449,7 +452,9 @@ __device__ __forceinline__ void finish(uint32_t o, bool on, uint32_t* word) {
   if (on && o != start) at(word, start) = (at(word, start) & ~C::LINK) | o;
 }
 
-template <int T, int NT>
+// NARROW (narrow_grid): the loops over a tile's cells
+// end with its rows, and its rows are counted by their own width.
+template <int T, int NT, bool NARROW>
 __global__ void __launch_bounds__(NT, NT <= 64 ? 12 : 4) k_up_count(DemTable dt, Pipe p) {
   using L = Layout<T, NT>;
   using C = Cell<T>;
@@ -484,7 +489,7 @@ __global__ void __launch_bounds__(NT, NT <= 64 ? 12 : 4) k_up_count(DemTable dt,
     }
     __syncthreads();
     codes.shift(d, g);
-    set_words<T, NT>(codes, d, g, word, tab, p.status);
+    set_words<T, NT, NARROW>(codes, d, g, word, tab, p.status);
     __syncthreads();
     end_at_grid_edge<T, NT>(d, g, word);  // (only the summary reads what it changes)
     next = misc[2];
@@ -500,8 +505,9 @@ __global__ void __launch_bounds__(NT, NT <= 64 ? 12 : 4) k_up_count(DemTable dt,
     uint16_t* stack = stacks + warp * CAP;
     int n = 0;           // walks on the stack
     bool alone = false;  // this warp came last and finishes the tile's walks
+    const int rows = NARROW ? (g.th * T + NT * SWEEP - 1) / (NT * SWEEP) * SWEEP : ROWS;
     for (int r = 0;;) {
-      while (r < ROWS && n < 32) {
+      while (r < rows && n < 32) {
         uint32_t s[SWEEP];
         bool ready[SWEEP];
 #pragma unroll
@@ -549,7 +555,7 @@ __global__ void __launch_bounds__(NT, NT <= 64 ? 12 : 4) k_up_count(DemTable dt,
     }
     if (alone) finish<T>(lane < n ? *(volatile uint16_t*)&stack[lane] : spare<T>(), lane < n, word);
     __syncthreads();
-    const bool cyc = __syncthreads_or(store_counts<T, NT>(d, g, word));
+    const bool cyc = __syncthreads_or(store_counts<T, NT, NARROW>(d, g, word));
     if (threadIdx.x == 0 && cyc) set_status(p.status, D8_ERR_CYCLE);
     perimeter_summary<T, NT>(g, t, word, cyc, p);
   }
@@ -568,28 +574,32 @@ static int64_t resident(K k, int threads, size_t bytes) {
   return (int64_t)per_sm * sms;
 }
 
-template <int T, int NT>
-static cudaError_t launch_nt(const DemTable& dt, const Pipe& p, int64_t at_once, cudaStream_t s) {
-  const int64_t grid = min64(at_once, p.ntiles);
-  k_up_count<T, NT><<<(unsigned)(grid < 1 ? 1 : grid), NT, Layout<T, NT>::bytes, s>>>(dt, p);
-  return cudaGetLastError();
-}
-
 // Wide blocks where all tiles are under way at once: a tile's own latency is
 // what the pass takes then.  512 x 512 (64 tiles): 17 us, 27 in blocks of 64
 // threads; 576 tiles: 25 and 29; 676, more than the 608 wide blocks that fit at
 // once: 33 and 30.  32 x 32 tiles, 256 of them: 12.8 and 15.8.
+template <int T, int NT, bool NARROW>
+static cudaError_t launch_nt(const DemTable& dt, const Pipe& p, bool resident_only, bool* done, cudaStream_t s) {
+  auto k = k_up_count<T, NT, NARROW>;
+  constexpr size_t bytes = Layout<T, NT>::bytes;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  const int64_t at_once = resident(k, NT, bytes);
+  *done = !resident_only || p.ntiles <= at_once;
+  if (!*done) return cudaSuccess;
+  const int64_t grid = min64(at_once, p.ntiles);
+  k<<<(unsigned)(grid < 1 ? 1 : grid), NT, bytes, s>>>(dt, p);
+  return cudaGetLastError();
+}
+
 template <int T>
 static cudaError_t launch_t(const DemTable& dt, const Pipe& p, cudaStream_t s) {
   constexpr int WIDE = 4 * T, NT = 64;
-  cudaError_t e = cudaFuncSetAttribute(k_up_count<T, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)Layout<T, WIDE>::bytes);
-  if (e != cudaSuccess) return e;
-  const int64_t wide = resident(k_up_count<T, WIDE>, WIDE, Layout<T, WIDE>::bytes);
-  if (p.ntiles <= wide) return launch_nt<T, WIDE>(dt, p, wide, s);
-  e = cudaFuncSetAttribute(k_up_count<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Layout<T, NT>::bytes);
-  if (e != cudaSuccess) return e;
-  return launch_nt<T, NT>(dt, p, resident(k_up_count<T, NT>, NT, Layout<T, NT>::bytes), s);
+  bool done = false;
+  const cudaError_t e = launch_nt<T, WIDE, false>(dt, p, true, &done, s);
+  if (e != cudaSuccess || done) return e;
+  return narrow_grid(dt, T) ? launch_nt<T, NT, true>(dt, p, false, &done, s)
+                            : launch_nt<T, NT, false>(dt, p, false, &done, s);
 }
 
 }  // namespace count

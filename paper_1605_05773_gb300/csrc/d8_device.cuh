@@ -137,6 +137,15 @@ __device__ __forceinline__ TileGeo tile_geo(const DemDesc& d, int64_t local_tile
   return g;
 }
 
+// Log2 of the power of two that a narrow tile's rows are counted by where its
+// cells are gone through.
+__device__ __forceinline__ int width_shift(const TileGeo& g) { return 32 - __clz(g.tw - 1); }
+// A grid of a quarter of a tile's side at most: its tiles are mostly empty, and
+// kernels built for it go through the cells there are.  (Whole accumulation, T = 64:
+// 3 x 1000000 324 us, 408 by the ordinary kernels; 1000000 x 3 375 and 577; 17 x
+// 100000 97 by these, whose code for full tiles is the slower, and 97.)
+inline bool narrow_grid(const DemTable& t, int T) { return t.ndem == 1 && min64(t.one.H, t.one.W) <= T / 4; }
+
 // slot of perimeter cell (i, j) of a th x tw tile, or -1 for an inner cell
 __device__ __forceinline__ int slot_of(int i, int j, int th, int tw, int T) {
   if (i == 0) return j;

@@ -65,7 +65,7 @@ __device__ __forceinline__ int step_of(uint32_t code) {
 // the codes by asynchronous copies into code[].  Rows of whole tiles are copied
 // as the aligned words that cover them, one more word than the row has when it
 // starts at an odd address, and shifted into place in finish().
-template <int T, int NT, class V>
+template <int T, int NT, class V, bool NARROW = false>
 struct Ahead {
   static constexpr int S = T + 4;
   static constexpr int NS = (4 * T + NT - 1) / NT;           // slots per thread
@@ -98,9 +98,10 @@ struct Ahead {
         dst += RS * S;
       }
     } else {
+      const int sh = width_shift(g), end = NARROW ? g.th << sh : T * T;
 #pragma unroll 8
-      for (int c = threadIdx.x; c < T * T; c += NT) {
-        const int i = c / T, j = c % T;
+      for (int c = threadIdx.x; c < end; c += NT) {
+        const int i = NARROW ? c >> sh : c / T, j = NARROW ? c & ((1 << sh) - 1) : c % T;
         if (i < g.th && j < g.tw) code[i * S + j] = __ldg(d.dir + (g.i0 + i) * d.lddir + (g.j0 + j));
       }
     }
@@ -125,10 +126,13 @@ struct Ahead {
   }
 };
 
-template <int T>
+// NARROW (narrow_grid): the loops over a tile's cells end with its rows, and its
+// rows are counted by their own width.
+template <int T, bool NARROW>
 __global__ void __launch_bounds__(NTN, 8) k_fin_count(DemTable dt, Pipe p) {
   using L = Layout<T>;
-  constexpr int TT = T * T, S = L::S, TS = (int)L::TS, NS = Ahead<T, NTN, uint32_t>::NS;
+  using AH = Ahead<T, NTN, uint32_t, NARROW>;
+  constexpr int TT = T * T, S = L::S, TS = (int)L::TS, NS = AH::NS;
   extern __shared__ __align__(16) unsigned char sm[];
   uint32_t* F = reinterpret_cast<uint32_t*>(sm + L::off_f);
   uint32_t* rin = reinterpret_cast<uint32_t*>(sm + L::off_rin);
@@ -139,7 +143,7 @@ __global__ void __launch_bounds__(NTN, 8) k_fin_count(DemTable dt, Pipe p) {
   // F starts at zero; every tile leaves the words it touched at zero again
   for (int q = threadIdx.x; q < TS / 4; q += NTN) reinterpret_cast<uint4*>(F)[q] = make_uint4(0, 0, 0, 0);
   if (threadIdx.x < 2) misc[threadIdx.x] = 0u;
-  Ahead<T, NTN, uint32_t> ahead;
+  AH ahead;
   int64_t t = blockIdx.x;
   if (t < p.ntiles) {
     const DemDesc d = dem_of(dt, t);
@@ -203,7 +207,18 @@ __global__ void __launch_bounds__(NTN, 8) k_fin_count(DemTable dt, Pipe p) {
     // when the layout allows, else single cells, in consecutive lanes; the
     // reads of U of them are issued before any is used.
     uint32_t* const A0 = static_cast<uint32_t*>(d.A) + g.i0 * d.ldA + g.j0;
-    if (g.tw == T && ((reinterpret_cast<uintptr_t>(d.A) & 15u) == 0) && (d.ldA & 3) == 0) {
+    if constexpr (NARROW) {
+      const int sh = width_shift(g), jm = (1 << sh) - 1;
+#pragma unroll 1
+      for (int q = threadIdx.x; q < g.th << sh; q += NTN) {
+        const int i = q >> sh, j = q & jm;  // (columns off the tile have no inflow)
+        const uint32_t f = F[i * S + j];
+        if (f) {
+          F[i * S + j] = 0u;
+          A0[i * d.ldA + j] += f;
+        }
+      }
+    } else if (g.tw == T && ((reinterpret_cast<uintptr_t>(d.A) & 15u) == 0) && (d.ldA & 3) == 0) {
       constexpr int NQ = TT / 4 / NTN, U = NQ < 4 ? NQ : 4;
 #pragma unroll 1
       for (int r0 = 0; r0 < NQ; r0 += U) {
@@ -589,8 +604,9 @@ static cudaError_t launch_k(K k, int threads, size_t bytes, const DemTable& dt, 
 
 template <int T>
 static cudaError_t launch_t(const DemTable& dt, const Pipe& p, bool weighted, cudaStream_t s) {
-  return weighted ? launch_k(k_fin_area<T>, NTW, LayoutW<T>::bytes, dt, p, s)
-                  : launch_k(k_fin_count<T>, NTN, Layout<T>::bytes, dt, p, s);
+  if (weighted) return launch_k(k_fin_area<T>, NTW, LayoutW<T>::bytes, dt, p, s);
+  return narrow_grid(dt, T) ? launch_k(k_fin_count<T, true>, NTN, Layout<T>::bytes, dt, p, s)
+                            : launch_k(k_fin_count<T, false>, NTN, Layout<T>::bytes, dt, p, s);
 }
 
 }  // namespace fin
