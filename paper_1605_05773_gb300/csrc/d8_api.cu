@@ -62,6 +62,20 @@ struct d8_ctx {
   int last_rounds = -1;
 };
 
+namespace {
+
+// The levels of a layered combine (hier_shape).
+struct HShape {
+  bool solve = false;  // no levels: one launch over the tiles (HPlan::solve)
+  int nlev = 0;
+  int S[HMAX + 1] = {};
+  int64_t nunits[HMAX + 1] = {};
+  bool need_top = false;
+  bool jump = false;
+};
+
+}  // namespace
+
 struct d8_batch {
   d8_ctx* ctx = nullptr;
   int n = 0;
@@ -80,11 +94,7 @@ struct d8_batch {
   int launches_per_run = 0;
   // layered combine: per level l >= 1, a table of per-DEM unit grids and a
   // unit -> DEM map (level 0 uses the tile table above)
-  int nlev = 0;
-  bool solve = false;
-  bool need_top = false;
-  int lev_S[HMAX + 1] = {};
-  int64_t lev_units[HMAX + 1] = {};
+  HShape hs;
   std::vector<DemDesc> lev_host[HMAX + 1];
   DemDesc* lev_desc[HMAX + 1] = {};
   int32_t* lev_map[HMAX + 1] = {};
@@ -174,15 +184,6 @@ Pipe carve_pipe(void* base, int64_t ntiles, int T, size_t vbytes, uint32_t* stat
 }
 
 // ---- layered combine plan (single DEM or batch) ---------------------------
-struct HShape {
-  bool solve = false;  // no levels: one launch over the tiles (HPlan::solve)
-  int nlev = 0;
-  int S[HMAX + 1] = {};
-  int64_t nunits[HMAX + 1] = {};
-  bool need_top = false;
-  bool jump = false;
-};
-
 // Levels above tiles of side T for the given DEM shapes.
 // Unit counts of grids up to solve_side take the single-launch combine: at 512
 // x 512 24 us against 59 for the four group launches and 10 more between them.
@@ -748,14 +749,8 @@ d8_status d8_batch_plan(d8_ctx* c, int n, const int64_t* H, const int64_t* W, d8
     for (int64_t t = 0; t < d.ntx * d.nty; t++) tile_dem[(size_t)(d.tile_base + t)] = k;
   }
   std::vector<int64_t> Hv(H, H + n), Wv(W, W + n);
-  const HShape hs = hier_shape(b->T, n, Hv.data(), Wv.data(), false, b->strat);
-  b->nlev = hs.nlev;
-  b->solve = hs.solve;
-  b->need_top = hs.need_top;
-  for (int l = 0; l <= hs.nlev; l++) {
-    b->lev_S[l] = hs.S[l];
-    b->lev_units[l] = hs.nunits[l];
-  }
+  b->hs = hier_shape(b->T, n, Hv.data(), Wv.data(), false, b->strat);
+  const HShape& hs = b->hs;
   b->pipe_part = align256(pipe_bytes(base, b->T, 4));
   b->ws_bytes = b->pipe_part + hier_bytes(hs, 4);
   for (int l = 1; l <= hs.nlev; l++) {
@@ -803,16 +798,10 @@ static cudaError_t batch_enqueue(d8_batch* b, int rule, cudaStream_t s, int* n_u
   if (b->n == 1) dt.ndem = 1;
   Pipe p = carve_pipe(b->ws, b->ntiles, b->T, 4, b->ctx->status);
   p.strat = b->strat;
-  HShape hs;
-  hs.nlev = b->nlev;
-  hs.solve = b->solve;
-  hs.need_top = b->need_top;
+  const HShape& hs = b->hs;
   DemTable dts[HMAX + 1];
   dts[0] = dt;
-  for (int l = 0; l <= b->nlev; l++) {
-    hs.S[l] = b->lev_S[l];
-    hs.nunits[l] = b->lev_units[l];
-    if (l == 0) continue;
+  for (int l = 1; l <= hs.nlev; l++) {
     DemTable t{};
     t.ndem = b->n;
     t.one = b->lev_host[l][0];
@@ -826,7 +815,7 @@ static cudaError_t batch_enqueue(d8_batch* b, int rule, cudaStream_t s, int* n_u
   if (e == cudaSuccess) e = launch_up(dt, p, UP_UNIT_Z, rule, s, n_up);
   if (e == cudaSuccess) e = launch_combine_hier(hp, s, n_comb);
   p.recv = true;
-  if (b->nlev == 0 && !b->solve) p.S = nullptr;
+  if (hs.nlev == 0 && !hs.solve) p.S = nullptr;
   if (e == cudaSuccess) e = launch_down(dt, p, false, s, n_down);
   return e;
 }
@@ -846,7 +835,7 @@ d8_status d8_batch_flowdir_accumulate(d8_batch* b, const float* const* z, uint8_
   // the descriptor table is read by the kernels at run time, so new buffer
   // pointers need no re-capture: upload it ahead of the graph on the stream
   cudaError_t e = cudaMemcpyAsync(b->dev_desc, b->host_desc.data(), sizeof(DemDesc) * b->n, cudaMemcpyHostToDevice, s);
-  for (int l = 1; l <= b->nlev && e == cudaSuccess; l++) {
+  for (int l = 1; l <= b->hs.nlev && e == cudaSuccess; l++) {
     for (int k = 0; k < b->n; k++) {
       b->lev_host[l][k].z = z[k];
       b->lev_host[l][k].dir = dir[k];
