@@ -152,8 +152,8 @@ d8_status d8_accumulate_weighted(d8_ctx* ctx, const uint8_t* dir, int64_t H, int
  * dw(q) = dL/dw(q) = dA(q) + dw(down-slope neighbour of q), i.e. the sum of
  * dA over q's flow path (the transpose of Eq. 1).  Per-tile path sums, a
  * pointer-jumping solve over the tile exits, then a finalising pass; the
- * tiles are 64 x 64, or 32 x 32 when d8_set_tile chose 32 (128 x 128 tiles
- * would not fit in shared memory).  Deterministic: the result does not depend
+ * tiles are 64 x 64, or 32 x 32 when d8_set_tile chose 32 (there is no pass
+ * for 128 x 128 tiles).  Deterministic: the result does not depend
  * on the launch configuration.  fp32 in and out, compensated accumulation.
  * Errors as d8_accumulate. */
 d8_status d8_accumulate_backward(d8_ctx* ctx, const uint8_t* dir, int64_t H, int64_t W, int64_t lddir,

@@ -634,9 +634,10 @@ d8_status d8_accumulate_backward(d8_ctx* c, const uint8_t* dir, int64_t H, int64
                                  const float* dA, int64_t lddA, float* dw, int64_t lddw, d8_stream stream) {
   if (!c || bad_grid(dir, H, W, lddir) || bad_grid(dA, H, W, lddA) || bad_grid(dw, H, W, lddw)) return D8_ERR_ARG;
   cudaSetDevice(c->device);
-  // The adjoint's tile pass keeps 21 bytes of shared memory per cell, so 64 x 64
-  // tiles fit two per SM; a context set to 32 x 32 tiles uses those (128 x 128
-  // would not fit).
+  // The adjoint's tile pass keeps 10 bytes of shared memory per cell, and its cells'
+  // state in registers: 64 x 64 tiles run two blocks per SM, a context set to 32 x
+  // 32 tiles uses those.  128 x 128 (160 KB: one block, of 1024 threads with 16
+  // cells each) is not built.
   const int T = c->T == 32 ? 32 : 64;
   DemDesc d = make_desc(H, W, T);
   d.dir = const_cast<uint8_t*>(dir);

@@ -28,7 +28,7 @@ namespace d8 {
 // of the tile exit its path reaches, with the exit's code above it, or NX_TERM
 // when the path ends inside the tile
 constexpr uint32_t NX_DONE = 0x8000u, NX_TERM = 0xFFFFu;
-constexpr uint32_t NX_CODE = 9;  // the code's bit position (slots take at most 8 bits)
+constexpr uint32_t NX_CODE = 9;  // the code's bit position, above the slot's
 
 // 64 x 64 tiles take 512 threads (8 cells each), 32 x 32 tiles 256 (4 each)
 template <int T>
@@ -63,7 +63,9 @@ struct BwdLayout {
 // took 735 us, blocks of 256 threads 757 us.
 template <int T>
 __global__ void __launch_bounds__(BwdCfg<T>::NTB, T >= 64 ? 2 : 4) k_bwd_up(DemTable dt, Pipe p) {
-  constexpr int NTB = BwdCfg<T>::NTB, CPT = BwdCfg<T>::CPT, TT = T * T;
+  constexpr int NTB = BwdCfg<T>::NTB, CPT = BwdCfg<T>::CPT;
+  static_assert(T * T <= (int)NX_DONE && 4 * T <= 1 << NX_CODE, "a cell, or a closed cell's slot and code, fits its word");
+  static_assert((1 << BwdCfg<T>::MAXR) > T * T, "rounds for the longest path inside a tile");
   using L = BwdLayout<T>;
   extern __shared__ __align__(16) unsigned char sm[];
   ff* gs = reinterpret_cast<ff*>(sm + L::off_gs);
