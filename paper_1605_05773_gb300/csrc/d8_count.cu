@@ -103,18 +103,9 @@ __device__ __forceinline__ uint32_t spare() {
   return (uint32_t)(T * T * 4 + 4 * (threadIdx.x & 31));
 }
 
-// Bits of the neighbours of tile cell (i, j) that lie outside a th x tw tile.
-__device__ __forceinline__ uint32_t row_off_mask(int i, int th) {
-  return (i == 0 ? 0x83u : 0u) | (i == th - 1 ? 0x38u : 0u);  // N, NE, NW / SE, S, SW
-}
-__device__ __forceinline__ uint32_t col_off_mask(int j, int tw) {
-  return (j == 0 ? 0xE0u : 0u) | (j == tw - 1 ? 0x0Eu : 0u);  // SW, W, NW / NE, E, SE
-}
-
-// One cell of a ragged tile:
-// its own word and one more input for its target.  A code 0..7 whose target is
-// outside the tile is an exit when the target is on the grid, otherwise the
-// path ends there.
+// One cell of a ragged tile: its own word and one more input for its target.  A
+// code 0..7 whose target is outside the tile is an exit when the target is on the
+// grid, otherwise the path ends there.
 template <int T>
 __device__ __forceinline__ void add_cell(uint32_t* word, int i, int j, int code, const TileGeo& g, const DemDesc& d,
                                          uint32_t* status) {

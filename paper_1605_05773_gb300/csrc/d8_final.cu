@@ -516,9 +516,9 @@ __global__ void __launch_bounds__(NTW, T >= 128 ? 1 : (T >= 64 ? 4 : 8)) k_fin_a
   uint8_t* code = sm + L::off_code;
   uint16_t* rcell = reinterpret_cast<uint16_t*>(sm + L::off_rcell);
   ff* rin = reinterpret_cast<ff*>(sm + L::off_rin);
-  // receivers, largest exponent bound + 1024, (unused), non-finite seen, next tile; the sum of bounds
+  // receivers, largest exponent bound + 1024, non-finite seen, next tile; the sum of bounds
   uint32_t* misc = reinterpret_cast<uint32_t*>(sm + L::off_misc);
-  unsigned long long* sum = reinterpret_cast<unsigned long long*>(misc + 6);
+  unsigned long long* sum = reinterpret_cast<unsigned long long*>(misc + 4);
 
   for (int q = threadIdx.x; q < 3 * TT / 4; q += NTW) reinterpret_cast<uint4*>(F0)[q] = make_uint4(0, 0, 0, 0);
   // |x| < 2^ebound(x) for finite x (subnormals and zero: 2^-126)
@@ -534,13 +534,13 @@ __global__ void __launch_bounds__(NTW, T >= 128 ? 1 : (T >= 64 ? 4 : 8)) k_fin_a
     __syncthreads();  // everyone is done with the tile before
     ahead.load(p, d, g, t, code);
     if (threadIdx.x == 0) {
-      misc[0] = misc[1] = misc[2] = misc[3] = 0u;
+      misc[0] = misc[1] = misc[2] = 0u;
       *sum = 0ull;
-      misc[4] = gridDim.x + atomicAdd(p.queue + 1, 1u);
+      misc[3] = gridDim.x + atomicAdd(p.queue + 1, 1u);
     }
     ahead.finish(d, g, code);
     __syncthreads();
-    next = misc[4];
+    next = misc[3];
     // Algorithm 7: the receivers listed; codes that leave the tile end the walk
 #pragma unroll
     for (int r = 0; r < NS; r++) {
@@ -558,12 +558,12 @@ __global__ void __launch_bounds__(NTW, T >= 128 ? 1 : (T >= 64 ? 4 : 8)) k_fin_a
       if (isfinite(in.hi)) {
         atomicMax(&misc[1], (uint32_t)(1024 + ebound(in.hi)));
       } else {
-        misc[3] = 1u;
+        misc[2] = 1u;
       }
     }
     __syncthreads();
     const int nrec = (int)misc[0];
-    if (misc[3]) {  // an infinite or NaN inflow
+    if (misc[2]) {  // an infinite or NaN inflow
       if (threadIdx.x == 0) set_status(p.status, D8_ERR_NONFINITE);
       continue;
     }
