@@ -285,20 +285,20 @@ __device__ __forceinline__ int walk_sources(const uint16_t* my, int n, V* val, u
 // nodes without unfinished children.  A finished node adds its value to its
 // parent, then (after a block fence) decrements the parent's children count;
 // the last child continues at the parent (its acquire-release count atomic
-// orders it after every child's addition).  exits: those this thread loaded.
-// Returns the number of nodes this thread finished.
+// orders it after every child's addition).  Returns the number of nodes this thread finished.
 //
 // Unit counts: in a group whose channels wind, few exits are sources (4 to 12 %
 // on boustrophedons and spirals, 80 to 86 % on fractals and planes), and the walks
 // are chains.  There the nodes with one child are marked first, so that the walks
-// need no atomics on them.  A block decides as a whole, since the marks, and the
-// chain in the walks' loop, cost fractals 1 to 3 % of the whole call.
+// need no atomics on them.  A block decides as a whole, by its warps' sources (a
+// count that the barrier takes along: a sum of sources and exits cost fractals
+// 1 to 2 % of the combine, marks and chains in every group 1 to 3 % of the call).
 // Whole accumulation of a 512 x 512 boustrophedon and spiral: 217 and 230 us (553
 // and 615 without; 326 and 621 with groups of 4 x 4 tiles and of 2 x 2, whose
 // chains are shorter), 300 x 257 spiral in 32 x 32 tiles 220 (443, 243), 600 x 700
-// spiral 364 (567, 473).
+// spiral 346 (567, 473).
 template <int S, int G, int NT, class V>
-__device__ int group_walk(uint16_t* spx, V* val, uint32_t* pd, uint16_t* srcl, int exits) {
+__device__ int group_walk(uint16_t* spx, V* val, uint32_t* pd, uint16_t* srcl) {
   constexpr int NS = G * G * 4 * S;
   constexpr int NW = NT / 32;
   static_assert(5 * 4 * S < (int)SINGLE, "a children count fits below the mark");
@@ -313,11 +313,8 @@ __device__ int group_walk(uint16_t* spx, V* val, uint32_t* pd, uint16_t* srcl, i
     n += __popc(m);
   }
   if constexpr (std::is_same<V, uint32_t>::value) {
-    // the group winds if more warps say so than say it does not (one barrier
-    // counts both: half of a warp's lanes for it, the other half against it)
-    const int ex = (int)__reduce_add_sync(FULL, (unsigned)exits);
-    const bool winds = 4 * n < ex, ordinary = !winds && n + ex > 0;
-    if (__syncthreads_count(lane < 16 ? winds : !ordinary) > 16 * NW) {
+    // the group winds if hardly a warp found sources in more than an eighth of its slots
+    if (__syncthreads_count(n > NS / NW / 8) <= NT / 8) {
       for (int c = threadIdx.x; c < NS; c += NT)
         if (pd_deg(pd[c]) == 1u) pd[c] |= SINGLE;
       __syncthreads();
@@ -355,7 +352,7 @@ __global__ void __launch_bounds__(NTG<S, G>) k_group_up(DemTable cdt, DemTable g
     }
     const GroupGeo gg = group_geo<S, G>(gd, gy, gx);
     const int exits = group_load<S, G, NT, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
-    const int done = group_walk<S, G, NT, V>(spx, val, pd, srcl, exits);
+    const int done = group_walk<S, G, NT, V>(spx, val, pd, srcl);
     atomicAdd(&misc[0], done);
     atomicAdd(&misc[1], exits);
     __syncthreads();
@@ -451,7 +448,7 @@ __global__ void __launch_bounds__(NTG<S, G>) k_group_down(DemTable cdt, DemTable
     const int64_t lg = gu - gd.tile_base;
     const int64_t gy = lg / gd.ntx, gx = lg % gd.ntx;
     const GroupGeo gg = group_geo<S, G>(gd, gy, gx);
-    const int exits = group_load<S, G, NT, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
+    group_load<S, G, NT, V, CV>(cd, gg, gy, gx, cpex, cpval, spx, val, pd);
     // inflow across the group border: each border cell r receives the final
     // areas of the outside cells draining into it; the inflow then follows
     // r's path inside its child unit to that child's exit
@@ -497,7 +494,7 @@ __global__ void __launch_bounds__(NTG<S, G>) k_group_down(DemTable cdt, DemTable
       }
     }
     __syncthreads();
-    group_walk<S, G, NT, V>(spx, val, pd, srcl, exits);
+    group_walk<S, G, NT, V>(spx, val, pd, srcl);
     __syncthreads();
     if constexpr (RECV) {
       V* infl = reinterpret_cast<V*>(pd);  // the walk is done with it
@@ -507,13 +504,13 @@ __global__ void __launch_bounds__(NTG<S, G>) k_group_down(DemTable cdt, DemTable
         if (bslot[r] >= 0) vatomic_add(&infl[bslot[r]], bin[r]);
       __syncthreads();
       store_inflow<S, G, NT, V>(cd, gy, gx, infl, cfin);
-      continue;
-    }
-    for (int n = threadIdx.x; n < NS; n += NT) {
-      if (!(spx[n] & PEX_EXIT)) continue;
-      const int lt = n / (4 * S), s = n - lt * (4 * S);
-      const int64_t cy = gy * G + lt / G, cx = gx * G + lt % G;
-      cfin[(cd.tile_base + cy * cd.ntx + cx) * (4 * S) + s] = val[n];
+    } else {
+      for (int n = threadIdx.x; n < NS; n += NT) {
+        if (!(spx[n] & PEX_EXIT)) continue;
+        const int lt = n / (4 * S), s = n - lt * (4 * S);
+        const int64_t cy = gy * G + lt / G, cx = gx * G + lt % G;
+        cfin[(cd.tile_base + cy * cd.ntx + cx) * (4 * S) + s] = val[n];
+      }
     }
   }
 }
@@ -536,7 +533,7 @@ __global__ void __launch_bounds__(NTS) k_group_solve(DemTable dt, const uint16_t
   const GroupGeo gg = group_geo<S, G>(d, 0, 0);
   if (threadIdx.x < 2) misc[threadIdx.x] = 0;
   const int exits = group_load<S, G, NTS, uint32_t, uint32_t>(d, gg, 0, 0, pex, pval, spx, val, pd);
-  const int done = group_walk<S, G, NTS, uint32_t>(spx, val, pd, srcl, exits);
+  const int done = group_walk<S, G, NTS, uint32_t>(spx, val, pd, srcl);
   atomicAdd(&misc[0], done);
   atomicAdd(&misc[1], exits);
   __syncthreads();
