@@ -312,7 +312,7 @@ __device__ int group_walk(uint16_t* spx, V* val, uint32_t* pd, uint16_t* srcl) {
     if (s) my[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)c;
     n += __popc(m);
   }
-  if constexpr (std::is_same<V, uint32_t>::value) {
+  if constexpr (std::is_same<V, uint32_t>::value && NS >= 8192) {
     // the group winds if hardly a warp found sources in more than an eighth of its slots
     if (__syncthreads_count(n > NS / NW / 8) <= NT / 8) {
       for (int c = threadIdx.x; c < NS; c += NT)
