@@ -28,9 +28,9 @@ namespace d8 {
 
 namespace cmb {
 
-// threads per group: 8 or 16 child slots each (16 at 4096 slots too: the combine
-// of weighted areas takes 136 us at 1001 x 777, where a group's latency counts,
-// for 112; 416 and 418 us at 8192 x 8192)
+// threads per group: 8 or 16 child slots each (with 16 at 4096 slots too the combine
+// of weighted areas took 136 us at 1001 x 777, where a group's latency counts,
+// for 112 at the time; 416 and 418 us at 8192 x 8192)
 template <int S, int G>
 constexpr int NTG = G * G * 4 * S >= 8192 ? 1024 : G * G * 4 * S / 8;
 constexpr unsigned FULL = 0xFFFFFFFFu;
@@ -888,9 +888,9 @@ static cudaError_t launch_top(const DemTable& dt, const HLevel& lv, const HTop& 
 // then of 2 x 2 children, up to a group side of 512 cells; the global queue
 // solve takes the rest.  (A 1024-cell level cost more than the longer
 // top-level chains it saves: measured at 8192^2 and 32768^2.)  One level of 8 x
-// 8 in blocks of 1024 threads instead of 4 x 4 and 2 x 2 in blocks of 256: the
-// whole combine takes 182 us at 8192^2 (237), 1.69 ms at 32768^2 (2.02), 110 us
-// at 3001 x 5003 (142).  Not for float-float values (8 x 8 children do not fit
+// 8 in blocks of 1024 threads instead of 4 x 4 and 2 x 2 in smaller ones: the
+// whole combine takes 144 us at 8192^2 (181), 1.60 ms at 32768^2 (2.01), 80 us
+// at 3001 x 5003 (89).  Not for float-float values (8 x 8 children do not fit
 // shared memory), nor under strategy "jump", whose long chains are walked
 // inside a group: two levels halve them.
 int hier_levels(int T, int64_t max_side, bool wide, int* S, int* G, int max_levels) {

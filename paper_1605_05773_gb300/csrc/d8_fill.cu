@@ -43,8 +43,9 @@
 // coarse grids get one round each and no host check; each level starts from
 // the bounds of the level above it.
 //
-// Measured, 8192 x 8192 raw fractal, 8192 x 8192 noisy plane, 700 x 933 fractal:
-// 4.4, 0.93 and 0.25 ms.  With more rounds on the coarse grids 4.6, 1.02 and
+// Measured, 8192 x 8192 raw fractals, 8192 x 8192 noisy plane, 700 x 933 fractals:
+// 3.1 to 5.2 (by the field), 0.90 and 0.19 to 0.30 ms.  One set of fields, 4.4,
+// 0.93 and 0.25 ms, took with more rounds on the coarse grids 4.6, 1.02 and
 // 0.29; in blocks of 64 threads too 5.1, 1.09 and 0.36 (at most 3 passes a visit
 // 5.5 ms and 0.45 for the fractals, 5 passes 5.5 and 0.37); visits to the fixed
 // point 5.9, 1.12 and 0.40; without the coarse grids 6.5, 3.2 and 0.45 (the
@@ -52,6 +53,8 @@
 // before (two waves over dirty cells, then sweeps of four passes until a whole
 // sweep changed nothing; lanes down a row shared banks, and every change of a
 // tile's border listed all eight neighbours) the fractals took 105 and 4.7 ms.
+// One channel that winds through every tile, behind a dam, 1024 x 1024: 157 ms (3.8
+// s), 7900 rounds.
 #include <cmath>
 #include <type_traits>
 
@@ -362,9 +365,10 @@ static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Levels are added while the last one has more than one tile, for grids of
 // more than 8 tiles a side: smaller ones settle in about as many rounds as the
-// coarse grids would take (when visits went to the fixed point, 500
-// x 500: 343 us without levels, 400 with; 700 x 933: 452 and 434; 3000 x 3000:
-// 1464 and 934).  Returns their number; bytes: the workspace.
+// coarse grids would take (two fractals each, with and without levels: 500 x 500
+// 174 and 186 us, 151 and 219; 600 x 600 188 and 192, 227 and 249; 700 x 933 204 and
+// 192, 269 and 263; 3000 x 3000 629 and 1410, 925 and 1345; 8192 x 8192 3.06 and 5.19
+// ms, 3.92 and 4.90).  Returns their number; bytes: the workspace.
 // What must be zero at the start comes first, `zeroed` bytes of it.
 static int levels(int64_t H, int64_t W, bool coarse, void* ws, Level* lv, size_t* zeroed, size_t* bytes) {
   int n = 0;

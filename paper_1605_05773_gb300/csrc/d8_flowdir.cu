@@ -27,8 +27,8 @@
 //
 // Measured (steepest): 32768 x 32768 1.31 ms, 4.1 TB/s (before: 2.90 ms, one
 // warp per tile, 2 columns per lane, eight ordered compare-and-selects per
-// cell); 8192 x 8192 98 us (195), 3001 x 5003 lowest with masks 50 us (84), 512
-// x 512 9.5 us (27).  41 warp instructions per 32 cells, 79 % issue active,
+// cell); 8192 x 8192 97 us (195), 3001 x 5003 with masks and a hundredth of it NaN
+// 41 us (85), 512 x 512 9 us (27).  41 warp instructions per 32 cells, 79 % issue active,
 // half-rate pipe 65 % busy, DRAM 42 %.
 #include "d8_device.cuh"
 
@@ -394,8 +394,11 @@ __global__ void __launch_bounds__(NTF, 5) k_flowdir_rows(DemTable dt, int64_t nt
 // Rows per item: whole tiles for grids that fill the GPU with them (two rows
 // in T are then read twice); below MIN_WARPS_PER_SM warps the tiles are cut
 // into segments of T / 2, T / 4, ... down to 8 rows.  (About 20 warps fit an
-// SM; with 40 here 8192 x 8192 runs 2.7 rounds of them and takes 122 us, with
-// 70 it halves its tiles and takes 98, with 140 it quarters them: 105.)  A grid
+// SM; with 35 here 8192 x 8192 runs 2.7 rounds of them and takes 121 us, with
+// 70 it halves its tiles and takes 97, with 140 it quarters them: 104.  With 35,
+// 70 and 140: 1024 x 1024 10.7, 9.7, 9.5 us; 3001 x 5003 33, 37, 37; 6000 x 6000
+// 76, 67, 69; 10000 x 7000 125, 109, 114; 12000 x 12000 217, 217, 200; 2048 x 2048,
+// 16384 x 16384 and 32768 x 32768 the same.)  A grid
 // lower than a tile is cut into segments of its own rows: 8 x 400000 takes 14 us,
 // 25 to 33 when two thirds of the segments lay below the grid.
 constexpr int64_t MIN_WARPS_PER_SM = 70;
