@@ -331,11 +331,12 @@ __global__ void __launch_bounds__(BPJ_NT) k_bpj_round(Pipe p, int r) {
 }
 
 // Every thread of the cluster's blocks meets here, and sees what the others wrote
-// to global memory before.
+// to global memory before.  (Not the .aligned forms: those want each warp
+// converged, which stores under a condition just before do not promise.)
 __device__ __forceinline__ void cluster_sync() {
   __threadfence();
-  asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  asm volatile("barrier.cluster.arrive.release;\n" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory");
   __threadfence();
 }
 
